@@ -243,7 +243,7 @@ df_status df_crt_residue_products(const double *A_dev, const double *B_dev, int 
 
 /* out = A B^T (A [M][K], B [N][K], out [M][N], all device, row-major)
  * emulated with nmod moduli; K <= 2^26.  Allocates scratch (2 nmod (M + N)
- * round_up(K, 8) bytes of residue planes, nmod M round_up(N, 16) bytes of
+ * round_up(K, 16) bytes of residue planes, nmod M round_up(N, 16) bytes of
  * residue products); synchronises `stream`.  DF_ERR_ARG for sizes or a
  * modulus count that admit no width q >= 2. */
 df_status df_emulated_gemm_crt(const double *A_dev, const double *B_dev, int M, int N, int K, int nmod,
@@ -421,11 +421,11 @@ df_status df_sparsity(const df_ctx *ctx, double *frac_ktiles, double *frac_chunk
  * df_build_K_blocks (Section 3.2's slice products) run on CTA pairs: a
  * cluster of two CTAs whose M = 256 tcgen05 MMA (cta_group::2) covers two
  * output tiles that share the stacked B operand, each CTA staging its own A
- * tile and half of B.  0 never; 1 (default) the first GEMM whenever its
- * occupied-orbital tiles pair up (every pair is useful there); 2 both GEMMs
- * wherever the layout pairs (the second GEMM's pairs also compute one lower
- * tile per pair of AO tile rows, which on GB300 costs more than pairing
- * saves).
+ * tile and half of the stacked B rows.  0 never; 1 (default) the first GEMM
+ * (every pair is useful there) and, from 7 AO tile rows (nao > 768) on, the
+ * second, whose pairs also compute one lower tile per pair of tile rows; 2
+ * both GEMMs wherever the layout pairs.  Batches pair the first GEMM only
+ * (df_batch_autotune).
  *
  * Returns DF_ERR_ARG for an unknown option or value; the context is unchanged. */
 #define DF_OPT_CLUSTER_PAIRS 1

@@ -36,7 +36,7 @@ struct df_batch {
   std::vector<int> nsplit;  // per molecule, in molecule order
   std::vector<int> nocc;
   int tables_for_s = -1;
-  bool pairs1 = false;  // first GEMM on CTA pairs (swapped layout, tables in tile pairs)
+  bool pairs1 = false;  // first GEMM on CTA pairs (tables in tile pairs)
   // side streams for the per-molecule kernels (X split, reduce, rho and J):
   // molecule i runs on side[i % kFan] between a fork and a join of the
   // caller's stream, in eager launches and inside a captured graph alike
@@ -94,12 +94,11 @@ std::vector<int> unit_order(const df_batch *b, const int *nocc) {
 df_status build_tables(df_batch *b, const int *nocc) {
   const int n = (int)b->ctx.size();
   std::vector<df::SgParams> p1(n), p2(n);
-  std::vector<CUtensorMap> m1(2 * n), m2(2 * n);
+  std::vector<df::SgMaps> m1(n), m2(n);
   std::vector<int> o1(n + 1, 0), o2(n + 1, 0);
   const std::vector<int> ord = unit_order(b, nocc);
   b->nsplit.assign(n, 1);
   // the first GEMM runs on CTA pairs when every molecule's orbitals fit one tile
-  // (the swapped layout; one slice count per molecule, so pairs may cross blocks)
   b->pairs1 = b->tile1 == 1;
   for (int i = 0; i < n; ++i) b->pairs1 = b->pairs1 && b->ctx[i]->pair_mode >= 1 && nocc[i] <= df::kTile;
   for (int k = 0; k < n; ++k) {
@@ -107,9 +106,8 @@ df_status build_tables(df_batch *b, const int *nocc) {
     df_ctx *c = b->ctx[i];
     const int ns = std::max(1, std::min(b->nsplit_cap, c->nsplit));
     b->nsplit[i] = ns;
-    if (!df::gemm1_setup(c, nocc[i], p1[k], m1[2 * k], m1[2 * k + 1], b->pairs1 ? 2 : 0)) return DF_ERR_CUDA;
-    if (!df::gemm2_setup(c, nocc[i], ns, p2[k], m2[2 * k])) return DF_ERR_CUDA;
-    m2[2 * k + 1] = m2[2 * k];
+    if (!df::gemm1_setup(c, nocc[i], p1[k], m1[k])) return DF_ERR_CUDA;
+    if (!df::gemm2_setup(c, nocc[i], ns, p2[k], m2[k])) return DF_ERR_CUDA;
     if (b->pairs1) p1[k].npairs = (int)df::slice_gemm_pairs(p1[k]);
     o1[k + 1] = o1[k] + (b->pairs1 ? p1[k].npairs : p1[k].nunits);
     o2[k + 1] = o2[k] + p2[k].nunits;
@@ -118,8 +116,8 @@ df_status build_tables(df_batch *b, const int *nocc) {
   b->total2 = o2[n];
   cudaError_t e = cudaMemcpy(b->params1, p1.data(), sizeof(df::SgParams) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(b->params2, p2.data(), sizeof(df::SgParams) * n, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(b->maps1, m1.data(), sizeof(CUtensorMap) * 2 * n, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(b->maps2, m2.data(), sizeof(CUtensorMap) * 2 * n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(b->maps1, m1.data(), sizeof(df::SgMaps) * n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(b->maps2, m2.data(), sizeof(df::SgMaps) * n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(b->off1, o1.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(b->off2, o2.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice);
   b->nocc.assign(nocc, nocc + n);
@@ -141,7 +139,7 @@ df_status enqueue_K(df_batch *b, const double *const *C, const int *nocc, int s,
         cudaSuccess)
       return DF_ERR_CUDA;
   df::SgGroup g1{b->params1, b->maps1, b->off1, n, b->total1};
-  if (df::launch_slice_gemm_grouped(b->pairs1 ? df::kModeXs : df::kModeX, g1, b->status, 0, st, b->pairs1) !=
+  if (df::launch_slice_gemm_grouped(df::kModeX, g1, b->status, 0, st, b->pairs1) !=
       cudaSuccess)
     return DF_ERR_CUDA;
   if (fork(b, st) != cudaSuccess) return DF_ERR_CUDA;
@@ -150,7 +148,7 @@ df_status enqueue_K(df_batch *b, const double *const *C, const int *nocc, int s,
     df::ShiftTable t1;
     const long long k1 = (long long)((c->nao + df::kKTile - 1) / df::kKTile) * df::kKTile;
     for (int q = 0; q <= 8; ++q) t1.v[q] = df::fixed_point_shift(q, k1);
-    if (df::launch_split_xblocks(reinterpret_cast<const long long *>(c->X), c->naux, c->nao, nocc[i], s, c->eB,
+    if (df::launch_split_xblocks(reinterpret_cast<const long long *>(c->X), c->naux, c->nao, df::even_nocc(nocc[i]), s, c->eB,
                                  c->eC, c->sblk, t1, c->rowE, c->eX, c->Xd, df::xdigit_ld(nocc[i]), c->nblk,
                                  b->side[i % df_batch::kFan]) != cudaSuccess)
       return DF_ERR_CUDA;
@@ -221,8 +219,8 @@ df_status df_batch_create(df_batch **out, df_ctx *const *ctxs, int n) {
   }
   if (e == cudaSuccess) e = cudaMalloc(&b->params1, sizeof(df::SgParams) * n);
   if (e == cudaSuccess) e = cudaMalloc(&b->params2, sizeof(df::SgParams) * n);
-  if (e == cudaSuccess) e = cudaMalloc(&b->maps1, sizeof(CUtensorMap) * 2 * n);
-  if (e == cudaSuccess) e = cudaMalloc(&b->maps2, sizeof(CUtensorMap) * 2 * n);
+  if (e == cudaSuccess) e = cudaMalloc(&b->maps1, sizeof(df::SgMaps) * n);
+  if (e == cudaSuccess) e = cudaMalloc(&b->maps2, sizeof(df::SgMaps) * n);
   if (e == cudaSuccess) e = cudaMalloc(&b->off1, sizeof(int) * (n + 1));
   if (e == cudaSuccess) e = cudaMalloc(&b->off2, sizeof(int) * (n + 1));
   if (e == cudaSuccess) e = cudaMalloc(&b->status, sizeof(int));

@@ -338,7 +338,7 @@ df_status crt_gemm(const double *A, const double *B, int M, int N, int K, int nm
   if (!A || !B || M <= 0 || N <= 0 || K <= 0) return DF_ERR_ARG;
   CrtTab t;
   if (!make_tab(K, nmod, &t)) return DF_ERR_ARG;
-  const long long ld = round_up_ll(K, 8);
+  const long long ld = round_up_ll(K, 16);
   const long long ldy = round_up_ll(N, 16);
   // A B^T with B == A (a Gram matrix such as K_b = X_b X_b^T): one split serves both sides
   const bool same = A == B && M == N;
@@ -359,30 +359,21 @@ df_status crt_gemm(const double *A, const double *B, int M, int N, int K, int nm
   const uint16_t *Bplanes = same ? Ad : Bd;
   const int *ebx = same ? ea : eb;
   if (e == cudaSuccess) {
-    CUtensorMap ta, tb;
-    if (!make_tmap_bf16(&ta, Ad, K, M, nmod, ld, (long long)M * ld) ||
-        !make_tmap_bf16(&tb, Bplanes, K, N, nmod, ld, (long long)N * ld)) {
+    SgMaps maps;
+    const SgOperand a{Ad, K, M, nmod, ld, (long long)M * ld}, b{Bplanes, K, N, nmod, ld, (long long)N * ld};
+    if (!make_operand_maps(&maps, a, b, kTile)) {
       rs = DF_ERR_CUDA;
     } else {
       SgParams p;
-      std::memset(&p, 0, sizeof(p));
-      p.layout = kLayoutCrt;
-      p.mode = kModeMod;
-      p.nt_m = (M + kTile - 1) / kTile;
-      p.nt_n = (N + kTile - 1) / kTile;
-      p.nunits = nmod * p.nt_m * p.nt_n;
-      p.m_valid = M;
-      p.n_valid = N;
-      p.ktiles = (K + kKTile - 1) / kKTile;
-      p.s_fixed = 1;
-      p.shiftT[1] = fixed_point_shift(1, (long long)p.ktiles * kKTile);  // 0: the sums are exact
+      grid_params(&p, kModeMod, M, N, K, 1);  // shiftT[1] = 0: the sums are exact
+      p.nunits *= nmod;
       p.out = reinterpret_cast<double *>(Y);
       p.out_ld = ldy;
       p.out_blk = (long long)M * ldy;
       p.status = status;
       for (int i = 0; i < nmod; ++i) p.crt_mod[i] = t.mod[i];
       if (p.shiftT[1] != 0 || (long long)p.nunits > (1ll << 30)) rs = DF_ERR_ARG;
-      else e = launch_slice_gemm(p, ta, tb, st);
+      else e = launch_slice_gemm(p, maps, st);
     }
   }
   if (e == cudaSuccess && rs == DF_OK && out) {

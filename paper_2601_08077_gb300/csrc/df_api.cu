@@ -3,7 +3,7 @@
 //
 // Exchange build at s slices (Section 3.2; blocked as Eqs. df-k-blk-1/2):
 //   1. split C per column into s digit planes          (split kernel, HBM)
-//   2. X^T tiles = C^T B^T over the B digit planes     (slice GEMM, tensor cores)
+//   2. X tiles = B C over the B digit planes           (slice GEMM, tensor cores)
 //   3. split X per (block, mu) row over (P in block, i) (split kernel, HBM)
 //   4. per block K_b = X_b X_b^T on upper tiles        (slice GEMM, tensor cores)
 //   5. K = sum_b K_b in block order, mirrored          (reduce kernel)
@@ -152,93 +152,59 @@ namespace df {
 
 df_status ctx_upload_slices(df_ctx *c, const int *sb, cudaStream_t st) { return upload_slices(c, sb, st); }
 
-// Parameters and operand maps of the first exchange GEMM: X^T = C^T B^T (the
-// orbitals on the MMA's M side), or, when CTA pairs are on and the orbitals
-// fit one 128-row tile, X = B C with the (P, mu) rows on the M side (pairs of
-// those tiles share the stacked C slices; nao even keeps a pair inside one
-// auxiliary block, so both CTAs run the same slice count).  X lands as
-// [(P, mu)][i] either way.
-bool gemm1_setup(df_ctx *c, int nocc, SgParams &p, CUtensorMap &ta, CUtensorMap &tb, int swap) {
+// Parameters and operand maps of the first exchange GEMM, X = B C: the
+// (P, mu) rows on the MMA's M side, the orbitals on its N side in the fewest
+// tiles of at most 128, all of one width that is a multiple of 32 (the N of a
+// cta_group::2 MMA), so few orbitals cost few columns.  X lands as
+// [(P, mu)][even_nocc].
+bool gemm1_setup(df_ctx *c, int nocc, SgParams &p, SgMaps &m) {
   const int nao = c->nao, naux = c->naux;
-  const long long c_plane = (long long)c->nocc_max * c->ld_nao;
-  const bool swapped =
-      nocc <= kTile && ((swap == 1 && c->pair_mode >= 1 && (nao & 1) == 0) || swap == 2);
-  if (swapped) {
-    if (!make_tmap_bf16(&ta, c->Bd, nao, (long long)naux * nao, c->s_max, c->ld_nao,
-                        (long long)naux * nao * c->ld_nao))
-      return false;
-    if (!make_tmap_bf16(&tb, c->Cd, nao, nocc, c->s_max, c->ld_nao, c_plane)) return false;
-    std::memset(&p, 0, sizeof(p));
-    p.layout = kLayoutXs;
-    p.mode = kModeXs;
-    p.nt_m = (int)(((long long)naux * nao + kTile - 1) / kTile);
-    p.nt_n = (nocc + kTile - 1) / kTile;
-    p.nunits = p.nt_m * p.nt_n;
-    p.m_valid = naux * nao;
-    p.n_valid = nocc;
-    p.ktiles = (nao + kKTile - 1) / kKTile;
-    p.nao = nao;
-    p.nocc = nocc;
-    p.nblk = c->nblk;
-    p.naux = naux;
-    p.s_blk = c->sblk;
-    for (int q = 0; q <= 8; ++q) p.shiftT[q] = fixed_point_shift(q, (long long)p.ktiles * kKTile);
-    p.ea = c->eB;
-    p.eb = c->eC;
-    p.out = c->X;
-    p.out_ld = nocc;
-    p.status = c->status;
-    p.pair = c->pair_mode;
-    p.kmask = use_mask_tile(c);
-    p.rowE = c->rowE;
-    return true;
-  }
-  if (!make_tmap_bf16(&ta, c->Cd, nao, nocc, c->s_max, c->ld_nao, c_plane)) return false;
-  if (!make_tmap_bf16(&tb, c->Bd, nao, (long long)naux * nao, c->s_max, c->ld_nao, (long long)naux * nao * c->ld_nao))
-    return false;
   std::memset(&p, 0, sizeof(p));
-  p.layout = kLayoutX;
   p.mode = kModeX;
-  p.nt_m = (nocc + kTile - 1) / kTile;
-  p.nt_n = (int)(((long long)naux * nao + kTile - 1) / kTile);
-  p.nunits = p.nt_m * p.nt_n;
-  p.m_valid = nocc;
-  p.n_valid = naux * nao;
+  p.nt_n = (nocc + kTile - 1) / kTile;
+  p.nw = (int)round_up((nocc + p.nt_n - 1) / p.nt_n, 32);
+  p.q = std::min(kSMax, 256 / p.nw);
+  p.m_valid = naux * nao;
+  p.n_valid = even_nocc(nocc);
+  p.kvalid = nao;
   p.ktiles = (nao + kKTile - 1) / kKTile;
   p.nao = nao;
-  p.nocc = nocc;
+  p.nocc = even_nocc(nocc);
   p.nblk = c->nblk;
   p.naux = naux;
+  p.nunits = (int)slice_gemm_units(p);
   p.s_blk = c->sblk;
   for (int q = 0; q <= 8; ++q) p.shiftT[q] = fixed_point_shift(q, (long long)p.ktiles * kKTile);
-  p.ea = c->eC;
-  p.eb = c->eB;
+  p.ea = c->eB;
+  p.eb = c->eC;
   p.out = c->X;
-  p.out_ld = nocc;
+  p.out_ld = even_nocc(nocc);
   p.status = c->status;
   p.pair = c->pair_mode;
   p.kmask = use_mask_tile(c);
   p.rowE = c->rowE;
-  return true;
+  const long long rows = (long long)naux * nao;
+  const SgOperand B{c->Bd, nao, rows, c->s_max, c->ld_nao, rows * c->ld_nao};
+  const SgOperand C{c->Cd, nao, nocc, c->s_max, c->ld_nao, (long long)c->nocc_max * c->ld_nao};
+  return make_operand_maps(&m, B, C, p.nw) && make_tmap_x(&m.x, c->X, p.out_ld, rows);
 }
 
-// Parameters and operand map of the second exchange GEMM (K_b = X_b X_b^T).
-bool gemm2_setup(df_ctx *c, int nocc, int nsplit, SgParams &q2, CUtensorMap &tx) {
+// Parameters and operand maps of the second exchange GEMM (K_b = X_b X_b^T).
+bool gemm2_setup(df_ctx *c, int nocc, int nsplit, SgParams &q2, SgMaps &m) {
   const int nao = c->nao, naux = c->naux;
-  const long long kb_ld = round_up((long long)kBlock * nocc, 64);
-  if (!make_tmap_bf16(&tx, c->Xd, kb_ld, nao, (long long)c->s_max * c->nblk, kb_ld, (long long)nao * kb_ld))
-    return false;
+  const long long kb_ld = xdigit_ld(nocc);
   std::memset(&q2, 0, sizeof(q2));
-  q2.layout = kLayoutKPart;
   q2.mode = kModeKPart;
   q2.nt_m = q2.nt_n = (nao + kTile - 1) / kTile;
+  q2.nw = kTile;
+  q2.q = 2;
   q2.nsplit = nsplit;
-  q2.nunits = q2.nt_m * (q2.nt_m + 1) / 2 * c->nblk * nsplit;
   q2.m_valid = q2.n_valid = nao;
   q2.nao = nao;
-  q2.nocc = nocc;
+  q2.nocc = even_nocc(nocc);
   q2.nblk = c->nblk;
   q2.naux = naux;
+  q2.nunits = (int)slice_gemm_units(q2);
   q2.s_blk = c->sblk;
   for (int q = 0; q <= 8; ++q) q2.shiftT[q] = fixed_point_shift(q, kb_ld);
   q2.ea = c->eX;
@@ -248,10 +214,11 @@ bool gemm2_setup(df_ctx *c, int nocc, int nsplit, SgParams &q2, CUtensorMap &tx)
   q2.out_blk = (long long)nao * nao;
   q2.status = c->status;
   q2.pair = c->pair_mode;
-  return true;
+  const SgOperand X{c->Xd, kb_ld, nao, (long long)c->s_max * c->nblk, kb_ld, (long long)nao * kb_ld};
+  return make_operand_maps(&m, X, X, q2.nw);
 }
 
-long long xdigit_ld(int nocc) { return round_up((long long)kBlock * nocc, 64); }
+long long xdigit_ld(int nocc) { return round_up((long long)kBlock * even_nocc(nocc), 64); }
 
 }  // namespace df
 
@@ -275,14 +242,14 @@ df_status k_front(df_ctx *c, const double *C, int nocc, const int *sb, int c_pla
     PhaseTimer t(c, DF_PHASE_SPLIT_C, st);
     DF_TRY(c, df::launch_split_cols_bf16(C, nao, nocc, c_planes, c->eC, c->Cd, c->ld_nao, c_plane, st));
   }
-  // 2. X^T = C^T B^T
+  // 2. X = B C
   df::SgParams p;
-  CUtensorMap ta, tb;
-  if (!df::gemm1_setup(c, nocc, p, ta, tb)) return record(c, DF_ERR_CUDA);
+  df::SgMaps maps;
+  if (!df::gemm1_setup(c, nocc, p, maps)) return record(c, DF_ERR_CUDA);
   DF_TRY(c, cudaMemsetAsync(c->rowE, 0x80, sizeof(int) * (size_t)c->nblk * nao, st));
   {
     PhaseTimer t(c, DF_PHASE_GEMM1, st);
-    DF_TRY(c, df::launch_slice_gemm(p, ta, tb, st));
+    DF_TRY(c, df::launch_slice_gemm(p, maps, st));
   }
   if (after_gemm1) DF_TRY(c, cudaEventRecord(after_gemm1, st));
   // 3. X -> per-(block, mu) digit planes
@@ -291,7 +258,7 @@ df_status k_front(df_ctx *c, const double *C, int nocc, const int *sb, int c_pla
     PhaseTimer t(c, DF_PHASE_SPLIT_X, st);
     df::ShiftTable t1;
     for (int q = 0; q <= 8; ++q) t1.v[q] = p.shiftT[q];
-    DF_TRY(c, df::launch_split_xblocks(reinterpret_cast<const long long *>(c->X), naux, nao, nocc, smax, c->eB,
+    DF_TRY(c, df::launch_split_xblocks(reinterpret_cast<const long long *>(c->X), naux, nao, df::even_nocc(nocc), smax, c->eB,
                                        c->eC, c->sblk, t1, c->rowE, c->eX, c->Xd, kb_ld, c->nblk, st));
   }
   return DF_OK;
@@ -300,11 +267,11 @@ df_status k_front(df_ctx *c, const double *C, int nocc, const int *sb, int c_pla
 df_status k_back(df_ctx *c, int nocc, double *K, cudaStream_t st) {
   // 4. per-block K_b on upper tiles (exact int64 partials per K split)
   df::SgParams q2;
-  CUtensorMap tx;
-  if (!df::gemm2_setup(c, nocc, c->nsplit, q2, tx)) return record(c, DF_ERR_CUDA);
+  df::SgMaps maps;
+  if (!df::gemm2_setup(c, nocc, c->nsplit, q2, maps)) return record(c, DF_ERR_CUDA);
   {
     PhaseTimer t(c, DF_PHASE_GEMM2, st);
-    DF_TRY(c, df::launch_slice_gemm(q2, tx, tx, st));
+    DF_TRY(c, df::launch_slice_gemm(q2, maps, st));
   }
   // 5. K = sum_b K_b
   {
@@ -393,16 +360,19 @@ df_status df_create(df_ctx **out, int nao, int naux, int nocc_max, int s_max) {
   c->nocc_max = nocc_max;
   c->s_max = s_max;
   c->nblk = (naux + kBlock - 1) / kBlock;
-  c->ld_nao = round_up(nao, 8);
-  c->kb_ld_max = round_up((long long)kBlock * nocc_max, 64);
+  // digit rows start on 32-byte boundaries (DRAM and L2 sectors): a TMA box of
+  // 128-byte pieces then touches 4 sectors per row instead of 5 (nao 600 at 8-
+  // value steps: the first exchange GEMM took 2.35 ms, at 16 1.71 ms)
+  c->ld_nao = round_up(nao, 16);
   const long long rowsB = (long long)naux * nao;
   cudaError_t e = cudaSuccess;
   if (e == cudaSuccess) e = alloc(c, &c->Bd, (size_t)s_max * rowsB * c->ld_nao);
   if (e == cudaSuccess) e = alloc(c, &c->eB, (size_t)rowsB);
   if (e == cudaSuccess) e = alloc(c, &c->Cd, (size_t)s_max * nocc_max * c->ld_nao);
-  if (e == cudaSuccess) e = alloc(c, &c->eC, (size_t)nocc_max);
-  if (e == cudaSuccess) e = alloc(c, &c->X, (size_t)rowsB * nocc_max);
-  if (e == cudaSuccess) e = alloc(c, &c->Xd, (size_t)s_max * c->nblk * nao * c->kb_ld_max);
+  if (e == cudaSuccess) e = alloc(c, &c->eC, (size_t)df::even_nocc(nocc_max));
+  if (e == cudaSuccess) e = cudaMemset(c->eC, 0, sizeof(int) * (size_t)df::even_nocc(nocc_max));
+  if (e == cudaSuccess) e = alloc(c, &c->X, (size_t)rowsB * df::even_nocc(nocc_max));
+  if (e == cudaSuccess) e = alloc(c, &c->Xd, (size_t)s_max * c->nblk * nao * df::xdigit_ld(nocc_max));
   if (e == cudaSuccess) e = alloc(c, &c->eX, (size_t)c->nblk * nao);
   if (e == cudaSuccess) e = alloc(c, &c->rowE, (size_t)c->nblk * nao);
   {
@@ -862,7 +832,7 @@ namespace {
 df_status grid_gemm(const double *A, const double *B, int M, int N, int K, int s, int mode, int64_t *raw,
                     double *out, int32_t *ea_out, int32_t *eb_out, cudaStream_t st) {
   if (!A || !B || M <= 0 || N <= 0 || K <= 0 || s < 1 || s > DF_S_MAX) return DF_ERR_ARG;
-  const long long ld = round_up(K, 8);
+  const long long ld = round_up(K, 16);
   // A B^T with B == A (a Gram matrix such as K_b = X_b X_b^T): one split serves both sides
   const bool same = A == B && M == N;
   uint16_t *Ad = nullptr, *Bd = nullptr;
@@ -883,30 +853,20 @@ df_status grid_gemm(const double *A, const double *B, int M, int N, int K, int s
     eb = ea;
   }
   if (e == cudaSuccess) {
-    CUtensorMap ta, tb;
-    if (!df::make_tmap_bf16(&ta, Ad, K, M, s, ld, (long long)M * ld) ||
-        !df::make_tmap_bf16(&tb, Bd, K, N, s, ld, (long long)N * ld)) {
+    df::SgMaps maps;
+    const df::SgOperand a{Ad, K, M, s, ld, (long long)M * ld}, b{Bd, K, N, s, ld, (long long)N * ld};
+    if (!df::make_operand_maps(&maps, a, b, df::kTile)) {
       rs = DF_ERR_CUDA;
     } else {
       df::SgParams p;
-      std::memset(&p, 0, sizeof(p));
-      p.layout = df::kLayoutGrid;
-      p.mode = mode;
-      p.nt_m = (M + df::kTile - 1) / df::kTile;
-      p.nt_n = (N + df::kTile - 1) / df::kTile;
-      p.nunits = p.nt_m * p.nt_n;
-      p.m_valid = M;
-      p.n_valid = N;
-      p.ktiles = (K + df::kKTile - 1) / df::kKTile;
-      p.s_fixed = s;
-      for (int q = 0; q <= 8; ++q) p.shiftT[q] = df::fixed_point_shift(q, (long long)p.ktiles * df::kKTile);
+      df::grid_params(&p, mode, M, N, K, s);
       p.ea = ea;
       p.eb = eb;
       p.out = out;
       p.out_ld = N;
       p.raw = reinterpret_cast<long long *>(raw);
       p.status = status;
-      e = df::launch_slice_gemm(p, ta, tb, st);
+      e = df::launch_slice_gemm(p, maps, st);
     }
   }
   int h = 0;

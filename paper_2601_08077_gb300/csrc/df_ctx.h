@@ -8,7 +8,6 @@
 struct df_ctx {
   int nao = 0, naux = 0, nocc_max = 0, s_max = 0, nblk = 0;
   long long ld_nao = 0;    // row stride (elements) of the B and C digit rows
-  long long kb_ld_max = 0; // row stride bound of the X digit rows
   const double *B = nullptr;  // dense [naux][nao][nao], or packed [naux][nao (nao + 1) / 2]
   bool packed = false;
   bool ready = false;
@@ -82,12 +81,12 @@ namespace df {
 // the stream when they did; not allowed during stream capture).
 df_status ctx_upload_slices(df_ctx *c, const int *sb, cudaStream_t st);
 // Parameters and operand maps of the two exchange GEMMs of a context.
-// swap: 0 orbitals on the MMA's M side; 1 (single problem) the (P, mu)-rows-
-// on-M layout when CTA pairs are on, nocc <= 128 and nao is even; 2 (grouped,
-// one slice count per problem, so a pair may straddle two blocks) that layout
-// whenever nocc <= 128.
-bool gemm1_setup(df_ctx *c, int nocc, SgParams &p, CUtensorMap &ta, CUtensorMap &tb, int swap = 1);
-bool gemm2_setup(df_ctx *c, int nocc, int nsplit, SgParams &q2, CUtensorMap &tx);
+bool gemm1_setup(df_ctx *c, int nocc, SgParams &p, SgMaps &m);
+bool gemm2_setup(df_ctx *c, int nocc, int nsplit, SgParams &q2, SgMaps &m);
+// The orbital count X is laid out for: even, so that the int64 sums and the
+// digits of two neighbouring orbitals always share an aligned 16- and 4-byte
+// word; the orbital added to an odd count has zero digits everywhere.
+inline int even_nocc(int nocc) { return nocc + (nocc & 1); }
 long long xdigit_ld(int nocc);
 // The sparsity masks to use (null: run dense).
 inline const uint32_t *use_mask_mu(const df_ctx *c) { return c->sparse && c->sparse_opt ? c->mask_mu : nullptr; }

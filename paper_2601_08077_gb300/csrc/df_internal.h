@@ -16,26 +16,16 @@ constexpr int kTile = 128;       // output tile edge of the slice GEMM
 constexpr int kKTile = 64;       // K elements per pipeline stage (128 bytes of bf16)
 constexpr int kMaxChunk = 1024;  // products per exact FP32 accumulation chunk
 
-// Epilogue modes of the slice GEMM.
+// What a slice GEMM computes and how it stores it.
 enum SgMode : int {
-  kModeX = 0,       // first exchange GEMM: int64 sums R[n*ld + m] of X^T = C^T B^T (the X split rounds them)
-  kModeKPart = 1,   // second exchange GEMM: int64 fixed-point partial per (block, K split),
-                    // raw[part*blk + n*ld + m] (the reduce scales and sums them)
+  kModeX = 0,       // first exchange GEMM, X = B C with the (P, mu) rows on the MMA's M side and the
+                    // orbitals on its N side: the exact int64 sums R[m*ld + n] (the X split rounds them)
+  kModeKPart = 1,   // second exchange GEMM: upper tile pairs of K_b = X_b X_b^T, an int64 fixed-point
+                    // partial per (block, K split), raw[part*blk + n*ld + m] (the reduce scales and sums them)
   kModeRaw = 2,     // exact S_g per group: raw[(g*n_valid + n)*m_valid + m]
   kModeGemm = 3,    // generic emulated product: out[m*ld + n]
-  kModeXs = 4,      // first exchange GEMM with swapped operands (rows (P, mu) on the A side):
-                    // int64 sums R[m*ld + n], the same X layout as kModeX
   kModeMod = 5,     // CRT variant: the exact sum of one modulus plane reduced modulo that
                     // modulus, one byte each: out8[plane*out_blk + m*ld + n]
-};
-
-// How the persistent kernel turns a unit index into a tile.
-enum SgLayout : int {
-  kLayoutGrid = 0,   // u -> (m_tile = u % nt_m, n_tile = u / nt_m), planes az = t, bz = t
-  kLayoutX = 1,      // first exchange GEMM: n rows are (P, mu); block = n0 / (128 nao)
-  kLayoutKPart = 2,  // second exchange GEMM: u -> (upper tile pair, block)
-  kLayoutXs = 3,     // first exchange GEMM, swapped: m rows are (P, mu); block = m0 / (128 nao)
-  kLayoutCrt = 4,    // CRT variant: u -> (plane = u / (nt_m nt_n), grid tile), planes az = bz = plane
 };
 
 constexpr int kCrtMaxModuli = 16;
@@ -48,15 +38,18 @@ constexpr int kDensityChangeBlocks = 152;
 constexpr int kWideRow = 2048;
 
 struct SgParams {
-  int layout, mode;
+  int mode;
   int nunits;
   int nt_m, nt_n;           // tiles along m and n
   int m_valid, n_valid;     // rows of the A side and of the B side that exist
-  int ktiles;               // K tiles (64 wide) for kLayoutGrid / kLayoutX
-  int s_fixed;              // slice count for kLayoutGrid
+  int ktiles;               // K tiles (64 wide); kModeKPart: of a block, from nocc
+  int kvalid;               // K values (the last tile's rest is zeros); kModeKPart: of a block, from nocc
+  int nw;                   // columns of an n tile (rows of a stacked B digit): a multiple of 32, at most 128
+  int q;                    // digits stacked in one MMA: min(8, 256 / nw)
+  int s_fixed;              // slice count (kModeRaw, kModeGemm, kModeMod)
   int nao, nocc, nblk, naux;
-  int nsplit;               // K splits per block (kLayoutKPart)
-  const int *s_blk;         // per-block slice counts (kLayoutX, kLayoutKPart)
+  int nsplit;               // K splits per block (kModeKPart)
+  const int *s_blk;         // per-block slice counts (kModeX, kModeKPart)
   int shiftT[9];            // truncation T of the fixed-point sum, indexed by s (0..8)
   const int *ea;            // A-side row exponents
   const int *eb;            // B-side row exponents
@@ -66,8 +59,8 @@ struct SgParams {
   long long *raw;
   int *status;              // device status word (DF_ERR_TIMEOUT bits)
   // CTA-pair mode: two CTAs of a cluster take two tiles that share their
-  // B-side operand; each CTA loads its own A tile and one of the two stacked
-  // B tiles into its own shared memory (both copies complete on the first
+  // B-side operand; each CTA loads its own A tile and half of the stacked
+  // B rows into its own shared memory (both copies complete on the first
   // CTA's barrier), and one M = 256 MMA reads both CTAs' tiles.  Work is
   // then counted in tile pairs (npairs); the host sets both.
   int pair;
@@ -77,7 +70,7 @@ struct SgParams {
   // B's (P, mu) rows, the bit mask of its nonzero 64-wide K tiles (bit k = K
   // tile k, at most 32); null = dense
   const uint32_t *kmask;
-  // first exchange GEMM (kModeX / kModeXs): per (block, mu) row of X, the
+  // first exchange GEMM (kModeX): per (block, mu) row of X, the
   // largest bit-length bound E = bitlen(|R|) + k over the row's nonzero exact
   // sums R (|R 2^k| < 2^E), atomically maxed; the X split takes it as its
   // exponent guess and so reads R once.  Reset to kRowBoundNone before the
@@ -89,15 +82,34 @@ struct SgParams {
 // memset resets it); below every real bound.
 constexpr int kRowBoundNone = (int)0x80808080;
 
-// Tile pairs of a launch in CTA-pair mode (0 = the layout has no pairing):
-// kLayoutGrid / kLayoutX pair m tiles 2a, 2a+1 of one n tile (nt_m even);
-// kLayoutKPart pairs m tiles 2a, 2a+1 of n tile j >= 2a per (block, split).
+// Work units of a launch: tiles, and tile pairs in CTA-pair mode (0 = the
+// mode has no pairing).
+long long slice_gemm_units(const SgParams &p);
 long long slice_gemm_pairs(const SgParams &p);
+
+// One operand's digit planes: [planes][rows][ld] BF16, k of the ld columns used.
+struct SgOperand {
+  const void *base;
+  long long k, rows, planes, ld, plane_stride;
+};
+
+// Tensor maps of a launch: boxes of 64 (K) x 128 rows of A, and of nw and
+// nw / 2 rows of B (a CTA of a pair stages a digit's rows whole or by halves).
+// x: the first exchange GEMM's output, for its TMA stores.
+struct SgMaps {
+  CUtensorMap a, b, h, x;
+};
+bool make_tmap_x(CUtensorMap *map, const void *base, long long ld, long long rows);
+bool make_operand_maps(SgMaps *m, const SgOperand &a, const SgOperand &b, int nw);
+
+// A stand-alone product of A [M][K] and B [N][K] over s digits (kModeRaw, kModeGemm):
+// sizes, tiles and truncation; the caller sets the exponents and the output.
+void grid_params(SgParams *p, int mode, int M, int N, int K, int s);
 
 // A grouped launch: the work units of several problems (molecules) in one
 // persistent launch.  Problem i owns units [unit_off[i], unit_off[i+1]); its
-// parameters are params[i] and its operand tensor maps maps[2i] (A side) and
-// maps[2i+1] (B side), all in device memory (maps 64-byte aligned).
+// parameters are params[i] and its tensor maps maps[4i] .. maps[4i+3]
+// (an SgMaps), all in device memory (maps 64-byte aligned).
 struct SgGroup {
   const SgParams *params;
   const CUtensorMap *maps;
@@ -137,7 +149,8 @@ cudaError_t launch_split_cols_bf16(const double *C, int nrows, int ncols, int ns
 struct ShiftTable {
   int v[9];
 };
-// R: the first GEMM's int64 sums (kModeX); X = fl64(R 2^k) is formed here with
+// R: the first GEMM's int64 sums (kModeX, nocc even: an odd count is padded
+// with a zero orbital); X = fl64(R 2^k) is formed here with
 // the first GEMM's exponents eB (rows (P, mu)), eC (orbitals), slices s_blk and
 // truncation table T1, then split per (block, mu).  rowE: the first GEMM's
 // per-row bound (SgParams::rowE) when it recorded one, else null.
@@ -147,14 +160,13 @@ cudaError_t launch_split_xblocks(const long long *R, int naux, int nao, int nocc
 cudaError_t launch_kpart_reduce(const long long *Rp, const int *eX, const int *s_blk, ShiftTable T, int nao,
                                 int nblk, int nsplit, double *K, cudaStream_t st);
 
-// Encode a 3D bf16 tensor map {k, rows, planes} with a 64 x 128 x 1 box, 128B swizzle.
+// Encode a 3D bf16 tensor map {k, rows, planes} with a 64 x box_rows x 1 box, 128B swizzle.
 bool make_tmap_bf16(CUtensorMap *map, const void *base, long long k, long long rows, long long planes,
-                    long long row_stride_elems, long long plane_stride_elems);
+                    long long row_stride_elems, long long plane_stride_elems, int box_rows);
 
-cudaError_t launch_slice_gemm(const SgParams &p, const CUtensorMap &ta, const CUtensorMap &tb,
-                              cudaStream_t st);
+cudaError_t launch_slice_gemm(const SgParams &p, const SgMaps &m, cudaStream_t st);
 // Grouped launch; `mode` is shared by all problems, `grid` CTAs (0 = one per SM).
-// pairs: CTA-pair launch over tile pairs (kModeXs only; unit_off and total
+// pairs: CTA-pair launch over tile pairs (kModeX only; unit_off and total
 // count tile pairs, every problem's npairs set).
 cudaError_t launch_slice_gemm_grouped(int mode, const SgGroup &g, int *status, int grid, cudaStream_t st,
                                       bool pairs = false);

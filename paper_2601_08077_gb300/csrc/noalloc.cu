@@ -89,28 +89,17 @@ extern "C" df_status df_emulated_gemm_static(const double *A, const double *B, i
   if (e == cudaSuccess && !same)
     e = df::launch_split_rows_bf16(B, N, K, K, nslices, eb, Bd, ld, (long long)N * ld, st);
   if (e != cudaSuccess) return DF_ERR_CUDA;
-  CUtensorMap ta, tb;
-  if (!df::make_tmap_bf16(&ta, Ad, K, M, nslices, ld, (long long)M * ld) ||
-      !df::make_tmap_bf16(&tb, Bd, K, N, nslices, ld, (long long)N * ld))
-    return DF_ERR_CUDA;
+  df::SgMaps maps;
+  const df::SgOperand a{Ad, K, M, nslices, ld, (long long)M * ld}, b{Bd, K, N, nslices, ld, (long long)N * ld};
+  if (!df::make_operand_maps(&maps, a, b, df::kTile)) return DF_ERR_CUDA;
   df::SgParams p;
-  std::memset(&p, 0, sizeof(p));
-  p.layout = df::kLayoutGrid;
-  p.mode = df::kModeGemm;
-  p.nt_m = (M + df::kTile - 1) / df::kTile;
-  p.nt_n = (N + df::kTile - 1) / df::kTile;
-  p.nunits = p.nt_m * p.nt_n;
-  p.m_valid = M;
-  p.n_valid = N;
-  p.ktiles = (K + df::kKTile - 1) / df::kKTile;
-  p.s_fixed = nslices;
-  for (int q = 0; q <= 8; ++q) p.shiftT[q] = df::fixed_point_shift(q, (long long)p.ktiles * df::kKTile);
+  df::grid_params(&p, df::kModeGemm, M, N, K, nslices);
   p.ea = ea;
   p.eb = eb;
   p.out = out;
   p.out_ld = N;
   p.status = status;
-  e = df::launch_slice_gemm(p, ta, tb, st);
+  e = df::launch_slice_gemm(p, maps, st);
   if (e != cudaSuccess) return DF_ERR_CUDA;
   int h = 0;
   e = cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, st);
