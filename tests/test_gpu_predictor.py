@@ -36,6 +36,24 @@ def test_mlp_forward_and_gradients_match_oracle(df):
     assert np.max(np.abs(g - g_ref)) <= 1e-5 + 1e-4 * np.max(np.abs(g_ref))
 
 
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 8193])
+def test_mlp_gradients_at_tile_edges(df, n):
+    """Row tiles of 32 (one row, a ragged tile, more tiles than partial gradients): FP32 sums of n
+    terms of size |g|/n, so within n eps of them against FP64, and the same bits on every run."""
+    rng = np.random.default_rng(n)
+    theta = (M.init_params(3) + 0.05 * rng.standard_normal(M.N_PARAMS)).astype(np.float32)
+    X = rng.standard_normal((n, 16)).astype(np.float32)
+    y = rng.integers(0, 8, size=n)
+    net = df.MLP(theta)
+    Xg, yg = torch.from_numpy(X).cuda(), torch.from_numpy(y.astype(np.int32)).cuda()
+    g, loss = net.gradients(Xg, yg)
+    ref = M.gradients(theta.astype(np.float64), X.astype(np.float64), y)
+    assert abs(loss - M.loss(theta.astype(np.float64), X.astype(np.float64), y)) < 1e-5
+    assert np.max(np.abs(g - ref)) <= 1e-5 + 1e-4 * np.max(np.abs(ref))
+    g2, loss2 = net.gradients(Xg, yg)
+    assert np.array_equal(g, g2) and loss == loss2
+
+
 def test_adam_steps_match_oracle(df):
     """Three df_mlp_train_step calls against the oracle's Adam (beta 0.9 / 0.999, bias
     correction) on the oracle's FP64 gradients, element by element.  The first update is
