@@ -358,51 +358,6 @@ __global__ void density_change_final_kernel(const double *__restrict__ part, int
   }
 }
 
-// Sets *flag when some B_P is not exactly symmetric (a NaN counts as
-// asymmetric).  Block (x, y, P) with x <= y compares the 32 x 32 tile (x, y) of
-// B_P, staged in shared memory, with the transpose of tile (y, x).
-__global__ void __launch_bounds__(256) symmetry_check_kernel(const double *__restrict__ B, int nao,
-                                                             int *__restrict__ flag) {
-  const int bi = blockIdx.x, bj = blockIdx.y;
-  if (bi > bj) return;
-  __shared__ double t[32][33];
-  const double *BP = B + (long long)blockIdx.z * nao * nao;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int r = ty; r < 32; r += 8) {
-    const int i = bi * 32 + r, j = bj * 32 + tx;
-    if (i < nao && j < nao) t[r][tx] = BP[(long long)i * nao + j];
-  }
-  __syncthreads();
-  bool bad = false;
-  for (int r = ty; r < 32; r += 8) {
-    const int i = bj * 32 + r, j = bi * 32 + tx;  // B[i][j] must equal B[j][i] = t[tx][r]
-    if (i < nao && j < nao && !(BP[(long long)i * nao + j] == t[tx][r])) bad = true;
-  }
-  if (__any_sync(0xffffffffu, bad) && tx == 0) atomicOr(flag, 1);
-}
-
-// Per mu: bit c set when some B_P mu nu, nu in [64c, 64c + 64), is nonzero.
-// One CTA per mu, over every P (one pass over B at setup).
-__global__ void __launch_bounds__(256) pair_mask_kernel(const double *__restrict__ B, int naux, int nao,
-                                                        uint32_t *__restrict__ mask_mu) {
-  const int mu = blockIdx.x;
-  uint32_t bits = 0u;
-  const long long n2 = (long long)nao * nao;
-  for (int P = 0; P < naux; ++P) {
-    const double *row = B + (long long)P * n2 + (long long)mu * nao;
-    for (int nu = threadIdx.x; nu < nao; nu += blockDim.x)
-      if (__ldg(row + nu) != 0.0) bits |= 1u << (nu >> 6);
-  }
-  bits = __reduce_or_sync(0xffffffffu, bits);
-  __shared__ uint32_t red[8];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = bits;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) bits |= red[w];
-    mask_mu[mu] = bits;
-  }
-}
-
 // Packed B: flag[k] = 1 when the packed pair k (of the upper triangle) is
 // nonzero in some B_P (one coalesced pass over B), then the per-mu masks
 // over all nu from the symmetric pair flags.
@@ -455,8 +410,7 @@ __global__ void tile_mask_kernel(const uint32_t *__restrict__ mask_mu, int nao, 
 
 constexpr int kEnergyBlocks = 296;
 
-cudaError_t launch_pair_masks_packed(const double *Bp, int naux, int nao, uint32_t *mask_mu, uint32_t *mask_tile,
-                                     cudaStream_t st) {
+cudaError_t launch_pair_masks_packed(const double *Bp, int naux, int nao, uint32_t *mask_mu, cudaStream_t st) {
   const long long npk = (long long)nao * (nao + 1) / 2;
   uint8_t *flag = nullptr;
   cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&flag), (size_t)npk, st);
@@ -465,12 +419,6 @@ cudaError_t launch_pair_masks_packed(const double *Bp, int naux, int nao, uint32
   e = cudaGetLastError();
   if (e == cudaSuccess) {
     mask_from_packed_flags_kernel<<<(nao + 127) / 128, 128, 0, st>>>(flag, nao, mask_mu);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) {
-    const long long rows = (long long)naux * nao;
-    const int ntiles = (int)((rows + kTile - 1) / kTile);
-    tile_mask_kernel<<<(ntiles + 255) / 256, 256, 0, st>>>(mask_mu, nao, rows, ntiles, mask_tile);
     e = cudaGetLastError();
   }
   cudaFreeAsync(flag, st);
@@ -483,24 +431,7 @@ cudaError_t launch_unpack(const double *Bp, int P0, int nP, int nao, double *out
   return cudaGetLastError();
 }
 
-cudaError_t launch_symmetry_check(const double *B, int naux, int nao, int *flag, cudaStream_t st) {
-  const int nt = (nao + 31) / 32;
-  cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  for (int p0 = 0; p0 < naux; p0 += 65535) {
-    const int np = naux - p0 < 65535 ? naux - p0 : 65535;
-    symmetry_check_kernel<<<dim3(nt, nt, np), 256, 0, st>>>(B + (long long)p0 * nao * nao, nao, flag);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-cudaError_t launch_pair_masks(const double *B, int naux, int nao, uint32_t *mask_mu, uint32_t *mask_tile,
-                              cudaStream_t st) {
-  pair_mask_kernel<<<nao, 256, 0, st>>>(B, naux, nao, mask_mu);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+cudaError_t launch_tile_masks(const uint32_t *mask_mu, int naux, int nao, uint32_t *mask_tile, cudaStream_t st) {
   const long long rows = (long long)naux * nao;
   const int ntiles = (int)((rows + kTile - 1) / kTile);
   tile_mask_kernel<<<(ntiles + 255) / 256, 256, 0, st>>>(mask_mu, nao, rows, ntiles, mask_tile);

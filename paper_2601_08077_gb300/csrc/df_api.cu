@@ -560,37 +560,36 @@ df_status setup_common(df_ctx *c, const double *B_dev, const int *perm_host, boo
     c->bstats = nullptr;
   }
   c->ready = false;
-  // rho and J read the upper triangle of each B_P: a dense B_P must be exactly symmetric
-  if (!packed) {
-    int h = 0;
-    DF_TRY(c, df::launch_symmetry_check(B_dev, c->naux, c->nao, c->status, st));
-    DF_TRY(c, cudaMemcpyAsync(&h, c->status, sizeof(int), cudaMemcpyDeviceToHost, st));
-    DF_TRY(c, cudaStreamSynchronize(st));
-    DF_TRY(c, cudaMemsetAsync(c->status, 0, sizeof(int), st));
-    if (h) return record(c, DF_ERR_ARG);
-  }
   const long long rows = (long long)c->naux * c->nao;
-  if (packed)
+  const int ntiles = (int)((rows + df::kTile - 1) / df::kTile);
+  // block sparsity of a screened B (Section 2.1): exact zero chunks of the AO pairs
+  const bool masks = c->nao <= 32 * df::kKTile;
+  if (masks && !c->mask_mu) DF_TRY(c, cudaMalloc(&c->mask_mu, sizeof(uint32_t) * c->nao));
+  if (masks && !c->mask_tile) DF_TRY(c, cudaMalloc(&c->mask_tile, sizeof(uint32_t) * ntiles));
+  int h = 0;
+  if (packed) {
     DF_TRY(c, df::launch_split_rows_packed(B_dev, c->naux, c->nao, c->s_max, c->eB, c->Bd, c->ld_nao,
                                            rows * c->ld_nao, c->perm, st));
-  else
-    DF_TRY(c, df::launch_split_rows_bf16(B_dev, rows, c->nao, c->nao, c->s_max, c->eB, c->Bd, c->ld_nao,
-                                         rows * c->ld_nao, st, c->perm, c->nao));
-  // block sparsity of a screened B (Section 2.1): exact zero chunks of the AO pairs
+    if (masks) DF_TRY(c, df::launch_pair_masks_packed(B_dev, c->naux, c->nao, c->mask_mu, st));
+  } else {
+    // rho and J read the upper triangle of each B_P: a dense B_P must be exactly
+    // symmetric (checked in the same pass, through the status word)
+    DF_TRY(c, df::launch_setup_rows(B_dev, c->naux, c->nao, c->s_max, c->eB, c->Bd, c->ld_nao, rows * c->ld_nao,
+                                    c->perm, masks ? c->mask_mu : nullptr, c->status, st));
+    DF_TRY(c, cudaMemcpyAsync(&h, c->status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    DF_TRY(c, cudaMemsetAsync(c->status, 0, sizeof(int), st));
+  }
   c->sparse = false;
   c->frac_ktiles = c->frac_chunks = 1.0;
-  if (c->nao <= 32 * df::kKTile) {
-    const int ntiles = (int)((rows + df::kTile - 1) / df::kTile);
-    if (!c->mask_mu) DF_TRY(c, cudaMalloc(&c->mask_mu, sizeof(uint32_t) * c->nao));
-    if (!c->mask_tile) DF_TRY(c, cudaMalloc(&c->mask_tile, sizeof(uint32_t) * ntiles));
-    if (packed)
-      DF_TRY(c, df::launch_pair_masks_packed(B_dev, c->naux, c->nao, c->mask_mu, c->mask_tile, st));
-    else
-      DF_TRY(c, df::launch_pair_masks(B_dev, c->naux, c->nao, c->mask_mu, c->mask_tile, st));
-    std::vector<uint32_t> mu(c->nao), tiles(ntiles);
+  std::vector<uint32_t> mu(c->nao), tiles(ntiles);
+  if (masks) {
+    DF_TRY(c, df::launch_tile_masks(c->mask_mu, c->naux, c->nao, c->mask_tile, st));
     DF_TRY(c, cudaMemcpyAsync(mu.data(), c->mask_mu, sizeof(uint32_t) * c->nao, cudaMemcpyDeviceToHost, st));
     DF_TRY(c, cudaMemcpyAsync(tiles.data(), c->mask_tile, sizeof(uint32_t) * ntiles, cudaMemcpyDeviceToHost, st));
-    DF_TRY(c, cudaStreamSynchronize(st));
+  }
+  DF_TRY(c, cudaStreamSynchronize(st));
+  if (h) return record(c, DF_ERR_ARG);
+  if (masks) {
     const int nk = (c->nao + df::kKTile - 1) / df::kKTile;
     long long on = 0, all = 0, kon = 0;
     for (int m = 0; m < c->nao; ++m)

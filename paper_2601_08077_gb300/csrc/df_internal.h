@@ -141,7 +141,14 @@ inline cudaError_t scratch_malloc(void **p, size_t bytes, cudaStream_t st) {
 // Kernel launchers (split.cu, slicegemm.cu, coulomb.cu).
 cudaError_t launch_split_rows_bf16(const double *A, long long rows, int cols, long long ld, int nslices,
                                    int *exps, uint16_t *digits, long long dld, long long plane_stride,
-                                   cudaStream_t st, const int *perm = nullptr, int group = 1);
+                                   cudaStream_t st);
+// Dense B [naux][nao][nao] at setup: *flag (zeroed first) set when some B_P is
+// not exactly symmetric, the digits of its rows (P' = perm[P] order), and
+// mask_mu (optional, nao <= 2048): per mu, bit c set when some B_P mu nu with
+// nu in [64c, 64c + 64) is nonzero.
+cudaError_t launch_setup_rows(const double *B, int naux, int nao, int nslices, int *exps, uint16_t *digits,
+                              long long dld, long long plane_stride, const int *perm, uint32_t *mask_mu, int *flag,
+                              cudaStream_t st);
 cudaError_t launch_split_rows_int8(const double *A, int rows, int cols, int ld, int nslices, int *exps,
                                    int8_t *digits, cudaStream_t st);
 cudaError_t launch_split_cols_bf16(const double *C, int nrows, int ncols, int nslices, int *exps,
@@ -193,20 +200,14 @@ cudaError_t launch_coulomb(const double *B, const double *rho, int naux, int nao
                            const uint32_t *mask_mu = nullptr, bool packed = false, int *work = nullptr,
                            int grid = 0);
 // The masks of a packed B (pair flags through stream-ordered scratch of nao (nao + 1) / 2 bytes).
-cudaError_t launch_pair_masks_packed(const double *Bp, int naux, int nao, uint32_t *mask_mu, uint32_t *mask_tile,
-                                     cudaStream_t st);
+cudaError_t launch_pair_masks_packed(const double *Bp, int naux, int nao, uint32_t *mask_mu, cudaStream_t st);
 // Dense B_P, P = P0 .. P0 + nP - 1, into out [nP][nao][nao] from a packed B.
 cudaError_t launch_unpack(const double *Bp, int P0, int nP, int nao, double *out, cudaStream_t st);
 // Digits of B from its packed layout (rows (P', mu) as launch_split_rows_bf16 writes them).
 cudaError_t launch_split_rows_packed(const double *Bp, int naux, int nao, int nslices, int *exps, uint16_t *digits,
                                      long long dld, long long plane_stride, const int *perm, cudaStream_t st);
-// Sets *flag (zeroed first) when some B_P of B [naux][nao][nao] is not exactly
-// symmetric.
-cudaError_t launch_symmetry_check(const double *B, int naux, int nao, int *flag, cudaStream_t st);
-// The masks of a screened B: mask_mu as above (nao <= 2048) and, per
-// 128-row tile of the (P, mu) rows, the OR of its rows' mu masks.
-cudaError_t launch_pair_masks(const double *B, int naux, int nao, uint32_t *mask_mu, uint32_t *mask_tile,
-                              cudaStream_t st);
+// Per 128-row tile of the (P, mu) rows, the OR of its rows' mu masks.
+cudaError_t launch_tile_masks(const uint32_t *mask_mu, int naux, int nao, uint32_t *mask_tile, cudaStream_t st);
 cudaError_t launch_energy(const double *D, const double *J, const double *K, const double *rho, int nao,
                           int naux, double *partials, double *E_dev, cudaStream_t st);
 

@@ -51,70 +51,141 @@ __device__ __forceinline__ uint64_t row_max_u64(uint64_t m) {
   return m;
 }
 
+// Digit t of the balanced expansion of N as an exact FP32 value, from
+// M = N + 128 (1 + 256 + ... + 256^6): the top digit is M >> 56, digit t >= 1
+// is byte 7-t of M minus 128.  The FP32 is built as (1.5 2^23 + byte) - (1.5
+// 2^23 + 128): one byte permute places the byte under the exponent bits and
+// one FP32 subtraction is exact, so its top 16 bits are the digit's BF16.
+__device__ __forceinline__ float digit_f32(long long M, int t) {
+  if (t == 0) return __int_as_float(0x4B400000 + (int)(M >> 56)) - 12582912.0f;
+  const uint32_t w = (7 - t) >= 4 ? (uint32_t)((unsigned long long)M >> 32) : (uint32_t)M;
+  return __int_as_float((int)__byte_perm(w, 0x4B400000u, 0x7640u | (uint32_t)((7 - t) & 3))) - 12583040.0f;
+}
+
+// BF16 of two FP32 digits (exact) packed low, high.
+__device__ __forceinline__ uint32_t bf16x2_of(float lo, float hi) {
+  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632u);
+}
+
+constexpr long long kDigitBias = 0x0080808080808080ll;  // 128 in each of the seven low bytes
+
+// Four consecutive values of a row from column c on (zeros past cols); 16-byte
+// loads when the row allows them.
+template <bool kVec2>
+__device__ __forceinline__ void load4(const double *__restrict__ row, int c, int cols, uint64_t (&v)[4]) {
+  if (kVec2 && c + 4 <= cols) {
+    const double2 a = __ldg(reinterpret_cast<const double2 *>(row + c));
+    const double2 b = __ldg(reinterpret_cast<const double2 *>(row + c + 2));
+    v[0] = (uint64_t)__double_as_longlong(a.x);
+    v[1] = (uint64_t)__double_as_longlong(a.y);
+    v[2] = (uint64_t)__double_as_longlong(b.x);
+    v[3] = (uint64_t)__double_as_longlong(b.y);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = c + i < cols ? (uint64_t)__double_as_longlong(__ldg(row + c + i)) : 0ull;
+  }
+}
+
+// Splits one row by TPR threads: its exponent, and s digits per value, four
+// columns per thread and step (8-byte stores into rows of a multiple of 8
+// digits, so columns past the row's end get zero digits).  nz (optional): the
+// 64-wide column chunks in which this thread saw a nonzero, for cols <= 2048.
+// The second pass reads the row from L1 or L2.
+template <int TPR, bool kVec2>
+__device__ __forceinline__ void split_row(const double *__restrict__ row, int cols, int lane, int nslices,
+                                          int *__restrict__ exp, uint16_t *__restrict__ drow, long long plane_stride,
+                                          uint32_t *nz) {
+  uint64_t m = 0;
+  uint32_t bits = 0u;
+#pragma unroll 4
+  for (int c = 4 * lane; c < cols; c += 4 * TPR) {
+    uint64_t v[4], any = 0;
+    load4<kVec2>(row, c, cols, v);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint64_t a = v[i] & 0x7FFFFFFFFFFFFFFFull;
+      m = a > m ? a : m;
+      any |= a;
+    }
+    if (nz && any) bits |= 1u << ((c >> 6) & 31);
+  }
+  if (nz) *nz = bits;
+  m = row_max_u64<TPR>(m);
+  const int e = exponent_from_max_bits_dev(m);
+  if (lane == 0) *exp = e;
+  for (int c = 4 * lane; c < cols; c += 4 * TPR) {
+    uint64_t v[4];
+    load4<kVec2>(row, c, cols, v);
+    long long M[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) M[i] = scaled_rne(v[i], e) + kDigitBias;
+#pragma unroll
+    for (int t = 0; t < kSMax; ++t)
+      if (t < nslices)
+        *reinterpret_cast<uint2 *>(drow + (long long)t * plane_stride + c) =
+            make_uint2(bf16x2_of(digit_f32(M[0], t), digit_f32(M[1], t)),
+                       bf16x2_of(digit_f32(M[2], t), digit_f32(M[3], t)));
+  }
+}
+
 // TPR threads per row (a warp, or the whole block for wide rows so that a
-// few hundred rows of tens of thousands of columns still fill the GPU); two
-// columns per thread per step (16-byte loads, 4-byte stores).
-template <int TPR>
+// few hundred rows of tens of thousands of columns still fill the GPU).
+template <int TPR, bool kVec2>
 __global__ void __launch_bounds__(256) split_rows_bf16_kernel(const double *__restrict__ A, long long rows,
                                                               int cols, long long ld, int nslices,
                                                               int *__restrict__ exps,
                                                               uint16_t *__restrict__ digits, long long dld,
-                                                              long long plane_stride, int vec2,
-                                                              const int *__restrict__ perm, int group) {
+                                                              long long plane_stride) {
   const int lane = threadIdx.x & (TPR - 1);
   const long long r = (long long)blockIdx.x * (blockDim.x / TPR) + (threadIdx.x / TPR);
   if (r >= rows) return;  // uniform over a row's threads (a whole block when TPR = 256)
-  // with a permutation, output row r = (P', j) reads input row (perm[P'], j), `group` rows per P
-  const long long src = perm ? (long long)perm[r / group] * group + (r % group) : r;
-  const double *row = A + src * ld;
-  uint64_t m = 0;
-  if (vec2) {
-    const double2 *row2 = reinterpret_cast<const double2 *>(row);
-    const int half = cols >> 1;
-    for (int c = lane; c < half; c += TPR) {
-      double2 v = __ldg(row2 + c);
-      uint64_t a = abs_bits(v.x), b = abs_bits(v.y);
-      m = a > m ? a : m;
-      m = b > m ? b : m;
+  split_row<TPR, kVec2>(A + r * ld, cols, lane, nslices, exps + r, digits + r * dld, plane_stride, nullptr);
+}
+
+// Everything df_setup reads a dense B for, in one kernel: a CTA takes 32 rows
+// of one B_P, compares them with the transposed tiles of B_P (an asymmetric B_P
+// or a NaN sets *flag), splits them (a warp per row; with a permutation, output
+// row (P', mu) reads input row (perm[P'], mu)), and ors each row's nonzero
+// 64-wide column chunks into mask_mu[mu] (null past 2048 columns).  B comes from
+// DRAM once: the transposed tiles and the second pass of a row are L2 and L1
+// hits.  As three kernels (check, split, masks: one CTA per mu walking all P)
+// the setup of 90 atoms (2.2 GB of B in, 3.3 GB of digits out) took 4.0 ms.
+template <bool kVec2>
+__global__ void __launch_bounds__(256) setup_rows_kernel(const double *__restrict__ B, int nao, int nslices,
+                                                         int *__restrict__ exps, uint16_t *__restrict__ digits,
+                                                         long long dld, long long plane_stride,
+                                                         const int *__restrict__ perm,
+                                                         uint32_t *__restrict__ mask_mu, int *__restrict__ flag) {
+  __shared__ double tile[32][33];
+  const int nt = (nao + 31) / 32;
+  const int Pq = blockIdx.x / nt, bi = blockIdx.x - Pq * nt;
+  const double *BP = B + (long long)(perm ? perm[Pq] : Pq) * nao * nao;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  bool bad = false;
+  for (int bj = bi; bj < nt; ++bj) {
+    for (int r = warp; r < 32; r += 8) {
+      const int i = bi * 32 + r, j = bj * 32 + lane;
+      if (i < nao && j < nao) tile[r][lane] = __ldg(BP + (long long)i * nao + j);
     }
-    if ((cols & 1) && lane == 0) {
-      uint64_t a = abs_bits(row[cols - 1]);
-      m = a > m ? a : m;
+    __syncthreads();
+    for (int r = warp; r < 32; r += 8) {
+      const int i = bj * 32 + r, j = bi * 32 + lane;  // B[i][j] must equal B[j][i] = tile[lane][r]
+      if (i < nao && j < nao && !(__ldg(BP + (long long)i * nao + j) == tile[lane][r])) bad = true;
     }
-  } else {
-    for (int c = lane; c < cols; c += TPR) {
-      uint64_t a = abs_bits(__ldg(row + c));
-      m = a > m ? a : m;
-    }
+    __syncthreads();
   }
-  m = row_max_u64<TPR>(m);
-  const int e = exponent_from_max_bits_dev(m);
-  if (lane == 0) exps[r] = e;
-  uint16_t *drow = digits + r * dld;
-  for (int c = 2 * lane; c < cols; c += 2 * TPR) {
-    int d0[kSMax], d1[kSMax];
-    uint64_t b0 = (uint64_t)__double_as_longlong(row[c]);
-    balanced_digits(scaled_rne(b0, e), d0);
-    bool two = c + 1 < cols;
-    if (two) {
-      uint64_t b1 = (uint64_t)__double_as_longlong(row[c + 1]);
-      balanced_digits(scaled_rne(b1, e), d1);
-    } else {
-#pragma unroll
-      for (int t = 0; t < kSMax; ++t) d1[t] = 0;
-    }
-#pragma unroll
-    for (int t = 0; t < kSMax; ++t) {
-      if (t < nslices) {
-        uint32_t pk = (uint32_t)int_to_bf16_bits(d0[t]) | ((uint32_t)int_to_bf16_bits(d1[t]) << 16);
-        uint16_t *dst = drow + (long long)t * plane_stride + c;
-        if (two && ((reinterpret_cast<uintptr_t>(dst) & 3) == 0)) {
-          *reinterpret_cast<uint32_t *>(dst) = pk;
-        } else {
-          dst[0] = (uint16_t)(pk & 0xFFFF);
-          if (two) dst[1] = (uint16_t)(pk >> 16);
-        }
-      }
+  if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(flag, 1);
+  for (int r = warp; r < 32; r += 8) {
+    const int mu = bi * 32 + r;
+    if (mu >= nao) break;  // the whole warp
+    const long long out = (long long)Pq * nao + mu;
+    uint32_t nz = 0u;
+    split_row<32, kVec2>(BP + (long long)mu * nao, nao, lane, nslices, exps + out, digits + out * dld, plane_stride,
+                         mask_mu ? &nz : nullptr);
+    if (mask_mu) {
+      nz = __reduce_or_sync(0xffffffffu, nz);
+      // the mask only gains bits: an old value at worst costs an atomic
+      if (lane == 0 && (nz & ~*reinterpret_cast<volatile uint32_t *>(mask_mu + mu))) atomicOr(mask_mu + mu, nz);
     }
   }
 }
@@ -243,22 +314,6 @@ constexpr int kSplitXThreads = 256;
 constexpr int kSplitXMinBlocks = 6;  // 40 registers: six rows in flight per SM (four at 51 measured slower)
 constexpr int kP1 = 4;  // loads in flight per thread in the first pass (8 measured slower)
 
-// Digit t of the balanced expansion of N as an exact FP32 value, from
-// M = N + 128 (1 + 256 + ... + 256^6): the top digit is M >> 56, digit t >= 1
-// is byte 7-t of M minus 128.  The FP32 is built as (1.5 2^23 + byte) - (1.5
-// 2^23 + 128): one byte permute places the byte under the exponent bits and
-// one FP32 subtraction is exact, so its top 16 bits are the digit's BF16.
-__device__ __forceinline__ float digit_f32(long long M, int t) {
-  if (t == 0) return __int_as_float(0x4B400000 + (int)(M >> 56)) - 12582912.0f;
-  const uint32_t w = (7 - t) >= 4 ? (uint32_t)((unsigned long long)M >> 32) : (uint32_t)M;
-  return __int_as_float((int)__byte_perm(w, 0x4B400000u, 0x7640u | (uint32_t)((7 - t) & 3))) - 12583040.0f;
-}
-
-// BF16 of two FP32 digits (exact) packed low, high.
-__device__ __forceinline__ uint32_t bf16x2_of(float lo, float hi) {
-  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632u);
-}
-
 struct XScale {
   const int *eB, *eC;  // (P, mu) row and orbital exponents of the first GEMM
   const int *s_blk;     // slices per block
@@ -333,7 +388,6 @@ __global__ void __launch_bounds__(kSplitXThreads, kSplitXMinBlocks) split_xblock
     constexpr bool keys = mode == 1, tb = mode == 2;
     if ((nocc & 1) == 0) {
       const int hp = nocc >> 1;
-      constexpr long long kBias = 0x0080808080808080ll;  // 128 in each of the seven low bytes
       constexpr int kU = 2;                                // pairs per thread per iteration (4 measured slower)
       for (int q0 = threadIdx.x; 2 * q0 < kpad; q0 += kU * blockDim.x) {
         longlong2 v[kU];
@@ -356,7 +410,7 @@ __global__ void __launch_bounds__(kSplitXThreads, kSplitXMinBlocks) split_xblock
           const int q = q0 + r * blockDim.x;
           const int k = 2 * q;
           if (k >= kpad) continue;
-          long long M0 = kBias, M1 = kBias;
+          long long M0 = kDigitBias, M1 = kDigitBias;
           if (kq[r] >= 0) {
             const int i = k - kq[r] * nocc;
             const int kp = eP[kq[r]];
@@ -531,19 +585,27 @@ __global__ void kpart_reduce_kernel(const long long *__restrict__ Rp, const int 
 
 cudaError_t launch_split_rows_bf16(const double *A, long long rows, int cols, long long ld, int nslices,
                                    int *exps, uint16_t *digits, long long dld, long long plane_stride,
-                                   cudaStream_t st, const int *perm, int group) {
+                                   cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
-  const int vec2 = ((ld & 1) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0) ? 1 : 0;
-  const int g = group > 0 ? group : 1;
-  if (cols >= kWideRow) {
-    split_rows_bf16_kernel<256><<<(unsigned)rows, 256, 0, st>>>(A, rows, cols, ld, nslices, exps, digits, dld,
-                                                                 plane_stride, vec2, perm, g);
-  } else {
-    const int wpb = 8;
-    dim3 grid((unsigned)((rows + wpb - 1) / wpb));
-    split_rows_bf16_kernel<32><<<grid, 32 * wpb, 0, st>>>(A, rows, cols, ld, nslices, exps, digits, dld,
-                                                         plane_stride, vec2, perm, g);
-  }
+  const bool vec2 = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  const bool wide = cols >= kWideRow;
+  const unsigned grid = (unsigned)(wide ? rows : (rows + 7) / 8);
+  auto kern = wide ? (vec2 ? split_rows_bf16_kernel<256, true> : split_rows_bf16_kernel<256, false>)
+                   : (vec2 ? split_rows_bf16_kernel<32, true> : split_rows_bf16_kernel<32, false>);
+  kern<<<grid, 256, 0, st>>>(A, rows, cols, ld, nslices, exps, digits, dld, plane_stride);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_setup_rows(const double *B, int naux, int nao, int nslices, int *exps, uint16_t *digits,
+                              long long dld, long long plane_stride, const int *perm, uint32_t *mask_mu, int *flag,
+                              cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), st);
+  if (e == cudaSuccess && mask_mu) e = cudaMemsetAsync(mask_mu, 0, sizeof(uint32_t) * nao, st);
+  if (e != cudaSuccess) return e;
+  const bool vec2 = (nao & 1) == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
+  auto kern = vec2 ? setup_rows_kernel<true> : setup_rows_kernel<false>;
+  kern<<<(unsigned)naux * (unsigned)((nao + 31) / 32), 256, 0, st>>>(B, nao, nslices, exps, digits, dld,
+                                                                      plane_stride, perm, mask_mu, flag);
   return cudaGetLastError();
 }
 

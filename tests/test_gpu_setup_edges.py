@@ -1,0 +1,71 @@
+"""df_setup's one pass over a dense B at the edges of its 32-row strips: the
+symmetry check (one ulp off, or a NaN, anywhere), the digits of every row (K at
+3 slices equals the oracle's emulation bit for bit, with and without an order of
+the auxiliary functions) and the 64-wide chunk masks (the fractions worked out
+from B)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import df_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def df():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2601_08077_gb300 import build, df as dfmod
+    build.build_all()
+    return dfmod
+
+
+def _tensor(seed, naux, nao):
+    rng = np.random.default_rng(seed)
+    B = rng.standard_normal((naux, nao, nao)) * np.exp2(rng.integers(-6, 1, (naux, nao, 1)))
+    return np.triu(B) + np.triu(B, 1).transpose(0, 2, 1)
+
+
+@pytest.mark.parametrize("nao", [1, 31, 32, 33, 64, 65, 130])
+def test_setup_checks_symmetry_everywhere(df, nao):
+    B = _tensor(nao, 3, nao)
+    ctx = df.Context(nao, 3, 1, 2)
+    ctx.setup(torch.from_numpy(B).cuda())
+    spots = {(0, nao - 1), (nao - 1, 0), (nao // 2, nao - 1), (min(31, nao - 1), min(32, nao - 1))}
+    for i, j in spots:
+        if i != j:
+            bad = B.copy()
+            bad[2, i, j] = np.nextafter(bad[2, i, j], 10.0)
+            with pytest.raises(df.DFError) as e:
+                ctx.setup(torch.from_numpy(bad).cuda())
+            assert e.value.status == -1
+    bad = B.copy()
+    bad[1, nao - 1, nao - 1] = np.nan
+    with pytest.raises(df.DFError) as e:
+        ctx.setup(torch.from_numpy(bad).cuda())
+    assert e.value.status == -1
+
+
+@pytest.mark.parametrize("naux,nao", [(2, 3), (130, 33), (5, 64), (4, 97)])
+def test_setup_digits_and_masks(df, naux, nao):
+    B = _tensor(7 * nao, naux, nao)
+    pair = np.random.default_rng(nao).random((nao, nao)) < 0.05  # a screened B
+    pair = pair | pair.T | np.eye(nao, dtype=bool)
+    C = np.random.default_rng(1).standard_normal((nao, 5))
+    perm = np.random.default_rng(2).permutation(naux)
+    for T, order in ((B, None), (np.where(pair, B, 0.0), None), (B, perm)):
+        ctx = df.Context(nao, naux, 5, 3)
+        ctx.setup(torch.from_numpy(T).cuda(), perm=order)
+        K, _ = ctx.build_K(torch.from_numpy(C).cuda(), 3)
+        ref = O.emulated_exchange(T if order is None else T[order], C, 3)
+        assert np.array_equal(K.cpu().numpy(), ref)
+        on = (T != 0).any(0)
+        nk = (nao + 63) // 64
+        chunk = np.array([[on[m, 64 * k:64 * k + 64].any() for k in range(nk)] for m in range(nao)])
+        upper = [chunk[m, k] for m in range(nao) for k in range(m // 64, nk)]
+        rows = np.tile(chunk, (naux, 1))
+        tiles = [rows[r:r + 128].any(0).sum() for r in range(0, naux * nao, 128)]
+        kt, ch = ctx.sparsity()
+        assert ch == pytest.approx(np.mean(upper), abs=1e-12)
+        assert kt == pytest.approx(sum(tiles) / (len(tiles) * nk), abs=1e-12)
