@@ -160,7 +160,7 @@ struct ShiftTable {
 // with a zero orbital); X = fl64(R 2^k) is formed here with
 // the first GEMM's exponents eB (rows (P, mu)), eC (orbitals), slices s_blk and
 // truncation table T1, then split per (block, mu).  rowE: the first GEMM's
-// per-row bound (SgParams::rowE) when it recorded one, else null.
+// per-row bound (SgParams::rowE).
 cudaError_t launch_split_xblocks(const long long *R, int naux, int nao, int nocc, int nslices, const int *eB,
                                  const int *eC, const int *s_blk, const ShiftTable &T1, const int *rowE, int *eX,
                                  uint16_t *Xd, long long kb_ld, int nblk, cudaStream_t st);

@@ -16,7 +16,6 @@
 #include "df_internal.h"
 
 #include <climits>
-#include <type_traits>
 
 namespace df {
 
@@ -290,29 +289,32 @@ __global__ void split_cols_bf16_kernel(const double *__restrict__ C, int nrows, 
   }
 }
 
-// One CTA per (block b, row mu) of X [naux][nao][nocc]: the row of the second
-// exchange GEMM is X_b[mu, (P_local, i)], length nP*nocc, padded with zero
-// digits up to a multiple of 64, one exponent per (block, mu).
+// The X split.  One CTA per (block b, row mu) of X [naux][nao][nocc] (nocc even):
+// the row of the second exchange GEMM is X_b[mu, (P_local, i)], length nP*nocc,
+// padded with zero digits up to a multiple of 64, one exponent per (block, mu).
 //
 // The first exchange GEMM leaves X as its exact int64 fixed-point sums R
 // (Section 3.2's recombination before the final rounding); this kernel takes
 // X = fl64(R 2^k), k = -14 - 8(s_b - 1) + T(s_b) + eC[i] + eB[(P, mu)], the
 // one rounding of the emulated product, and splits it.  (Doing the rounding
-// here keeps the GEMM's epilogue short; it measured 18% faster that way.)
-// The row's exponent needs its largest |X| (exact magnitude keys).  When the
-// first GEMM recorded its bound E for the row (rowE), the exponent is E or
-// E + 1, so one pass writes the digits with E while it takes the keys, and
-// only a row whose exact exponent differs (about one in a hundred) is read
-// a second time; R is read once.  Without the bound, a first pass takes the
-// keys and a second re-reads the row (256 KB at most, mostly from DRAM) for
-// the digits.  Two consecutive orbitals per thread (16-byte loads, 4-byte
-// stores) when nocc is even.
-template <int M>
-using Mode = std::integral_constant<int, M>;  // digits_pass: 0 digits, 1 and keys, 2 and threshold bits
-
+// here keeps the GEMM's epilogue short.)
+//
+// The row's exponent needs its largest |X|.  The first GEMM recorded a bound g
+// of it (the largest bitlen(|R|) + k of the row, rowE), so the exponent is g, or
+// g + 1 when some |X| reaches 127/128 2^g.  The fast pass reads R once and
+// writes the digits with e = g: N = RNE(X 2^(63-g)) is a left shift of R, after
+// its rounding to 53 bits where it has more (kRound), for all but the elements
+// far below the row's largest.  On the way it keeps the largest |N| (its top 31
+// bits), which tells whether the bound is attained (|N| >= 2^62) and whether it
+// is reached (|N| >= 127 2^56, to within one unit of the 31 bits), and whether a
+// shift lost bits.  A row that is reached (about one in a hundred) or whose
+// bound is not the row's takes the exact path (split_x_exact): it costs time
+// only.
+//
+// The pass is bound by its integer instructions: with an exact key per element,
+// a division per pair and plane offsets computed for a run-time slice count it
+// took about 75 an element (120 atoms, 5 slices: 608 us for 2.4 GB).
 constexpr int kSplitXThreads = 256;
-constexpr int kSplitXMinBlocks = 6;  // 40 registers: six rows in flight per SM (four at 51 measured slower)
-constexpr int kP1 = 4;  // loads in flight per thread in the first pass (8 measured slower)
 
 struct XScale {
   const int *eB, *eC;  // (P, mu) row and orbital exponents of the first GEMM
@@ -320,240 +322,199 @@ struct XScale {
   ShiftTable T;         // truncation of the first GEMM's fixed-point sum, by s
 };
 
-__global__ void __launch_bounds__(kSplitXThreads, kSplitXMinBlocks) split_xblocks_kernel(const long long *__restrict__ R, int naux,
-                                                                       int nao, int nocc, int nslices, XScale xs,
-                                                                       const int *__restrict__ rowE,
-                                                                       int *__restrict__ eX,
-                                                                       uint16_t *__restrict__ Xd, long long kb_ld,
-                                                                       int nblk) {
+// One row of X as the split sees it: element (pl, i) is r[pl pstride + i] 2^(eP[pl] + eI[i]).
+struct XRow {
+  const long long *r;
+  long long pstride;
+  const int *eP, *eI;  // shared memory
+  int nP, nocc, kpad;
+};
+
+// R to 53 bits, ties to even, for |R| < 2^61.
+__device__ __forceinline__ long long round53(long long R) {
+  const int hi = (int)(R >> 32);
+  const uint32_t a = (uint32_t)(hi ^ (hi >> 31));  // |R|'s (or |R| - 1's) high word
+  if (a >= (1u << 21)) {
+    const int sh = 11 - __clz((int)a);  // bits to drop; exact powers of two have none set
+    const long long lsb = (R >> sh) & 1;
+    R += ((1ll << sh) >> 1) - 1 + lsb;
+    R &= ~((1ll << sh) - 1);
+  }
+  return R;
+}
+
+// RNE(R 2^-r) for r >= 1, |R| < 2^61.
+__device__ __forceinline__ long long rne_down(long long R, int r) {
+  if (r >= 63) return 0;
+  return (R + ((1ll << (r - 1)) - 1) + ((R >> r) & 1)) >> r;
+}
+
+// Exact path of a row: the exact magnitude keys of its elements (bit length +
+// scale, then the normalised mantissa; rounding is monotone, so only the
+// winning element is rounded), the exponent they give, then the digits.
+// Returns the exponent.
+__device__ __noinline__ int split_x_exact(const XRow x, int nslices, uint16_t *dst, long long plane) {
+  __shared__ uint64_t red[kSplitXThreads / 32];
+  __shared__ int redE[kSplitXThreads / 32];
+  __shared__ int e_sh;
+  const int klen = x.nP * x.nocc;
+  int bE = INT_MIN;
+  uint64_t bM = 0;
+  for (int k = threadIdx.x; k < klen; k += kSplitXThreads) {
+    const int pl = k / x.nocc, i = k - pl * x.nocc;
+    const long long r = x.r[pl * x.pstride + i];
+    if (r == 0) continue;
+    int E;
+    uint64_t M;
+    mag_key(r, x.eP[pl] + x.eI[i], E, M);
+    if (E > bE || (E == bE && M > bM)) {
+      bE = E;
+      bM = M;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const int E2 = __shfl_xor_sync(0xffffffffu, bE, o);
+    const uint64_t M2 = __shfl_xor_sync(0xffffffffu, bM, o);
+    if (E2 > bE || (E2 == bE && M2 > bM)) {
+      bE = E2;
+      bM = M2;
+    }
+  }
+  if ((threadIdx.x & 31) == 0) {
+    redE[threadIdx.x >> 5] = bE;
+    red[threadIdx.x >> 5] = bM;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kSplitXThreads / 32; ++w)
+      if (redE[w] > bE || (redE[w] == bE && red[w] > bM)) {
+        bE = redE[w];
+        bM = red[w];
+      }
+    // the row's largest |X| is the rounding of its largest exact magnitude
+    const uint64_t top = bE == INT_MIN ? 0ull : abs_bits(ldexp_i64((long long)(bM >> 1), bE - 63));
+    e_sh = exponent_from_max_bits_dev(top);
+  }
+  __syncthreads();
+  const int e = e_sh;
+  for (int k = threadIdx.x; k < x.kpad; k += kSplitXThreads) {
+    int d[kSMax];
+    long long N = 0;  // zero digits in the padding
+    if (k < klen) {
+      const int pl = k / x.nocc, i = k - pl * x.nocc;
+      N = scaled_rne_i64(x.r[pl * x.pstride + i], x.eP[pl] + x.eI[i], e);
+    }
+    balanced_digits(N, d);
+#pragma unroll
+    for (int t = 0; t < kSMax; ++t)
+      if (t < nslices) dst[(long long)t * plane + k] = int_to_bf16_bits(d[t]);
+  }
+  return e;
+}
+
+// S: digit planes written; kRound: some |R| may have more than 53 bits.
+template <int S, bool kRound>
+__global__ void __launch_bounds__(kSplitXThreads, 5)
+    split_xblocks_kernel(const long long *__restrict__ R, int naux, int nao, int nocc, XScale xs,
+                         const int *__restrict__ rowE, int *__restrict__ eX, uint16_t *__restrict__ Xd,
+                         long long kb_ld, int nblk) {
   extern __shared__ int sh_e[];  // [kBlock] (P, mu) exponents + base, then [nocc] orbital exponents
+  __shared__ int sh_top, sh_lost;
   const int mu = blockIdx.x;
   const int b = blockIdx.y;
   const int p0 = b * kBlock;
   const int nP = min(kBlock, naux - p0);
-  const int klen = nP * nocc;
-  const int kpad = (klen + 63) / 64 * 64;
-  __shared__ uint64_t red[kSplitXThreads / 32];
-  __shared__ int redE[kSplitXThreads / 32];
-  __shared__ int e_sh;
   int *eP = sh_e;
   int *eI = sh_e + kBlock;
   {
     const int s1 = xs.s_blk[b];
     const int kbase = -14 - 8 * (s1 - 1) + xs.T.v[s1];
-    for (int q = threadIdx.x; q < nP; q += blockDim.x) eP[q] = kbase + xs.eB[(long long)(p0 + q) * nao + mu];
-    for (int q = threadIdx.x; q < nocc; q += blockDim.x) eI[q] = xs.eC[q];
+    for (int q = threadIdx.x; q < nP; q += kSplitXThreads) eP[q] = kbase + xs.eB[(long long)(p0 + q) * nao + mu];
+    for (int q = threadIdx.x; q < nocc; q += kSplitXThreads) eI[q] = xs.eC[q];
+    if (threadIdx.x == 0) sh_top = sh_lost = 0;
   }
+  const int g = __ldg(rowE + b * nao + mu);
   __syncthreads();
   const long long plane = (long long)nblk * nao * kb_ld;
   uint16_t *dst = Xd + ((long long)b * nao + mu) * kb_ld;
   const long long *row0 = R + ((long long)p0 * nao + mu) * nocc;  // element (pl, i) at row0[pl nao nocc + i]
   const long long pstride = (long long)nao * nocc;
-
-  // largest magnitude key (E, M) of the row seen by this thread; E = INT_MIN marks "none yet"
-  int bE = INT_MIN;
-  uint64_t bM = 0;
-  auto take = [&](long long r, int k) {
-    if (r == 0) return;
-    int E;
-    uint64_t M;
-    mag_key(r, k, E, M);
-    if (E > bE || (E == bE && M > bM)) {
-      bE = E;
-      bM = M;
-    }
-  };
-
-  // With the first GEMM's bound g (the largest bitlen(|R|) + k of the row):
-  // whether some element reaches 127/128 2^g once rounded to FP64 (only an
-  // element with bitlen(|R|) + k == g can: its normalised mantissa M must
-  // round to at least 127 2^46 on 53 bits, i.e. M >= 127 2^57 - 2^10, the tie
-  // going to the even 127 2^46), and whether the bound holds (no element above
-  // g, some element at g).  Bits: 1 reaches, 2 above g, 4 at g.
-  constexpr uint64_t kTopM = 0xFDFFFFFFFFFFFC00ull;
-  int tbits = 0;
-  auto thr = [&](long long r, int k, int g) {
-    if (r == 0) return;
-    const uint64_t u = r < 0 ? (uint64_t)(-(r + 1)) + 1ull : (uint64_t)r;
-    const int lz = __clzll((long long)u);
-    const int E = 64 - lz + k;
-    tbits |= (E > g ? 2 : 0) | (E == g ? (4 | ((u << lz) >= kTopM ? 1 : 0)) : 0);
-  };
-
-  // The digits of the whole row (zero digits in the padding) with exponent e;
-  // mode 1 takes the magnitude keys of the row's elements on the way, mode 2
-  // the threshold bits against the bound g (= e).
-  auto digits_pass = [&](int e, auto mode_c) {
-    constexpr int mode = decltype(mode_c)::value;
-    constexpr bool keys = mode == 1, tb = mode == 2;
-    if ((nocc & 1) == 0) {
-      const int hp = nocc >> 1;
-      constexpr int kU = 2;                                // pairs per thread per iteration (4 measured slower)
-      for (int q0 = threadIdx.x; 2 * q0 < kpad; q0 += kU * blockDim.x) {
-        longlong2 v[kU];
-        int kq[kU];
+  const int total = nP * (nocc >> 1);                    // pairs of neighbouring orbitals
+  const int pairs = (nP * nocc + 63) / 64 * 32;          // and with the padding
+  // far from the ends of the FP64 range: no |X| near 2^g overflows, and what
+  // fl64 would flush to zero is below half a unit of N
+  if (g > -900 && g < 1000) {
+    const int hp = nocc >> 1;
+    int pl = threadIdx.x / hp, ih = threadIdx.x - pl * hp;  // pair (pl, 2 ih)
+    const int dpl = kSplitXThreads / hp, dih = kSplitXThreads - dpl * hp;
+    uint32_t *out = reinterpret_cast<uint32_t *>(dst);
+    const long long pl2 = plane >> 1;
+    const int base = 63 - g;
+    int top = 0, lost = 0;
+    constexpr int kU = 2;  // pairs per thread in flight
+    for (int q0 = threadIdx.x; q0 < pairs; q0 += kU * kSplitXThreads) {
+      longlong2 v[kU];
+      int sx[kU], sy[kU];
 #pragma unroll
-        for (int r = 0; r < kU; ++r) {
-          const int q = q0 + r * blockDim.x;
-          const int k = 2 * q;
-          v[r] = make_longlong2(0, 0);  // N = 0 (padding) gives zero digits
-          kq[r] = -1;
-          if (k < klen) {
-            const int pl = q / hp;
-            const int i = k - pl * nocc;
-            v[r] = *reinterpret_cast<const longlong2 *>(row0 + pl * pstride + i);
-            kq[r] = pl;
-          }
+      for (int r = 0; r < kU; ++r) {
+        v[r] = make_longlong2(0, 0);  // N = 0 (padding) gives zero digits
+        sx[r] = sy[r] = 0;
+        if (q0 + r * kSplitXThreads < total) {
+          v[r] = *reinterpret_cast<const longlong2 *>(row0 + pl * pstride + 2 * ih);
+          const int2 e2 = *reinterpret_cast<const int2 *>(eI + 2 * ih);
+          sx[r] = base + eP[pl] + e2.x;
+          sy[r] = base + eP[pl] + e2.y;
         }
-#pragma unroll
-        for (int r = 0; r < kU; ++r) {
-          const int q = q0 + r * blockDim.x;
-          const int k = 2 * q;
-          if (k >= kpad) continue;
-          long long M0 = kDigitBias, M1 = kDigitBias;
-          if (kq[r] >= 0) {
-            const int i = k - kq[r] * nocc;
-            const int kp = eP[kq[r]];
-            if (keys) {
-              take(v[r].x, kp + eI[i]);
-              take(v[r].y, kp + eI[i + 1]);
-            }
-            if (tb) {
-              thr(v[r].x, kp + eI[i], e);
-              thr(v[r].y, kp + eI[i + 1], e);
-            }
-            M0 += scaled_rne_i64(v[r].x, kp + eI[i], e);
-            M1 += scaled_rne_i64(v[r].y, kp + eI[i + 1], e);
-          }
-#pragma unroll
-          for (int t = 0; t < kSMax; ++t)
-            if (t < nslices)
-              *reinterpret_cast<uint32_t *>(dst + (long long)t * plane + k) =
-                  bf16x2_of(digit_f32(M0, t), digit_f32(M1, t));
+        ih += dih;
+        pl += dpl;
+        if (ih >= hp) {
+          ih -= hp;
+          ++pl;
         }
       }
-    } else {
-      for (int k = threadIdx.x; k < kpad; k += blockDim.x) {
-        int d[kSMax];
-        if (k < klen) {
-          const int pl = k / nocc;
-          const int i = k - pl * nocc;
-          const long long r = row0[pl * pstride + i];
-          if (keys) take(r, eP[pl] + eI[i]);
-          if (tb) thr(r, eP[pl] + eI[i], e);
-          balanced_digits(scaled_rne_i64(r, eP[pl] + eI[i], e), d);
+      auto fixed = [&](long long r, int sh) -> long long {
+        if (kRound) r = round53(r);
+        const int hi = (int)(r >> 32);
+        if ((unsigned)sh < 32u) {
+          lost |= (hi >> (31 - sh)) ^ (hi >> 31);  // bits that the shift pushes out
+          r <<= sh;
+        } else if (sh < 0) {
+          r = rne_down(r, -sh);
         } else {
-#pragma unroll
-          for (int t = 0; t < kSMax; ++t) d[t] = 0;
+          lost |= sh > 62 ? (int)(r != 0) : (int)((r >> (63 - sh)) != (r >> 63));
+          r = sh > 62 ? 0 : r << sh;
         }
+        const int h = (int)(r >> 32);
+        top = max(top, h ^ (h >> 31));
+        return r + kDigitBias;
+      };
 #pragma unroll
-        for (int t = 0; t < kSMax; ++t)
-          if (t < nslices) dst[(long long)t * plane + k] = int_to_bf16_bits(d[t]);
+      for (int r = 0; r < kU; ++r) {
+        const int q = q0 + r * kSplitXThreads;
+        if (q >= pairs) break;
+        const long long M0 = fixed(v[r].x, sx[r]), M1 = fixed(v[r].y, sy[r]);
+#pragma unroll
+        for (int t = 0; t < S; ++t) out[q + t * pl2] = bf16x2_of(digit_f32(M0, t), digit_f32(M1, t));
       }
     }
-  };
-
-  // The row's exponent from the keys of all threads: e_sh (every thread reads it after the barrier).
-  auto reduce_keys = [&]() {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const int E2 = __shfl_xor_sync(0xffffffffu, bE, o);
-      const uint64_t M2 = __shfl_xor_sync(0xffffffffu, bM, o);
-      if (E2 > bE || (E2 == bE && M2 > bM)) {
-        bE = E2;
-        bM = M2;
-      }
-    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    lost = __reduce_or_sync(0xffffffffu, lost);
     if ((threadIdx.x & 31) == 0) {
-      redE[threadIdx.x >> 5] = bE;
-      red[threadIdx.x >> 5] = bM;
+      atomicMax(&sh_top, top);
+      if (lost) atomicOr(&sh_lost, lost);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-        if (redE[w] > bE || (redE[w] == bE && red[w] > bM)) {
-          bE = redE[w];
-          bM = red[w];
-        }
-      // the row's largest |X| is the rounding of its largest exact magnitude
-      const uint64_t top = bE == INT_MIN ? 0ull : abs_bits(ldexp_i64((long long)(bM >> 1), bE - 63));
-      e_sh = exponent_from_max_bits_dev(top);
-      eX[b * nao + mu] = e_sh;
+    // attained, and not within one unit of the 31 bits of 127/128 2^g
+    if (sh_lost == 0 && sh_top >= (1 << 30) && sh_top < (127 << 24) - 1) {
+      if (threadIdx.x == 0) eX[b * nao + mu] = g;
+      return;
     }
-    __syncthreads();
-  };
-
-  const int g = rowE ? __ldg(rowE + b * nao + mu) : kRowBoundNone;
-  if (rowE && g != kRowBoundNone && g > -1000 && g < 1000) {
-    // One read of R: the row's largest |X| lies in [2^(g-1), 2^g] for the first
-    // GEMM's bound g, so its exponent is g, or g + 1 when some element reaches
-    // 127/128 2^g: digits with g and the threshold bits on the way, a second
-    // pass only for a row that reaches it (far from the FP64 range's ends, so
-    // that no element near 2^g is flushed).  Should the bound not hold, the
-    // exact keys decide, as below.
-    digits_pass(g, Mode<2>{});
-    __shared__ int tsh;
-    if (threadIdx.x == 0) tsh = 0;
-    __syncthreads();
-    const int wb = __reduce_or_sync(0xffffffffu, tbits);
-    if ((threadIdx.x & 31) == 0 && wb) atomicOr(&tsh, wb);
-    __syncthreads();
-    const int bits = tsh;
-    if ((bits & 6) == 4) {
-      const int e = (bits & 1) ? g + 1 : g;
-      if (threadIdx.x == 0) eX[b * nao + mu] = e;
-      if (e != g) digits_pass(e, Mode<0>{});
-    } else {
-      digits_pass(g, Mode<1>{});
-      reduce_keys();
-      if (e_sh != g) digits_pass(e_sh, Mode<0>{});
-    }
-  } else if (rowE) {
-    // an all-zero row (or a bound near the FP64 range's ends): the exact keys
-    // on the way, a second pass if the exponent differs from the guess
-    const int e0 = g == kRowBoundNone ? exponent_from_max_bits_dev(0ull) : g;
-    digits_pass(e0, Mode<1>{});
-    reduce_keys();
-    if (e_sh != e0) digits_pass(e_sh, Mode<0>{});
-  } else {
-    // two passes: the keys (four loads in flight per thread), then the digits
-    if ((nocc & 1) == 0) {
-      const int hp = nocc >> 1;
-      const int total = nP * hp;
-      for (int q0 = threadIdx.x; q0 < total; q0 += kP1 * blockDim.x) {
-        longlong2 v[kP1];
-        int kp[kP1], ki[kP1];
-#pragma unroll
-        for (int r = 0; r < kP1; ++r) {
-          const int q = q0 + r * blockDim.x;
-          if (q < total) {
-            const int pl = q / hp;
-            const int i = 2 * (q - pl * hp);
-            v[r] = *reinterpret_cast<const longlong2 *>(row0 + pl * pstride + i);
-            kp[r] = eP[pl];
-            ki[r] = i;
-          } else {
-            v[r] = make_longlong2(0, 0);
-            kp[r] = 0;
-            ki[r] = 0;
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < kP1; ++r) {
-          take(v[r].x, kp[r] + eI[ki[r]]);
-          take(v[r].y, kp[r] + eI[ki[r] + 1]);
-        }
-      }
-    } else {
-      for (int k = threadIdx.x; k < klen; k += blockDim.x) {
-        const int pl = k / nocc;
-        const int i = k - pl * nocc;
-        take(row0[pl * pstride + i], eP[pl] + eI[i]);
-      }
-    }
-    reduce_keys();
-    digits_pass(e_sh, Mode<0>{});
+    __syncthreads();  // every thread has read the verdict
   }
+  const XRow x{row0, pstride, eP, eI, nP, nocc, 2 * pairs};
+  const int e = split_x_exact(x, S, dst, plane);
+  if (threadIdx.x == 0) eX[b * nao + mu] = e;
 }
 
 // K[mu][nu] = sum_b fl( 2^(eX[b,mu] + eX[b,nu] - 14 - 8(s_b - 1) + T(s_b)) * sum_sp R[b,sp] ),
@@ -636,17 +597,25 @@ cudaError_t launch_split_cols_bf16(const double *C, int nrows, int ncols, int ns
 cudaError_t launch_split_xblocks(const long long *R, int naux, int nao, int nocc, int nslices, const int *eB,
                                  const int *eC, const int *s_blk, const ShiftTable &T1, const int *rowE,
                                  int *eX, uint16_t *Xd, long long kb_ld, int nblk, cudaStream_t st) {
+  using Kern = void (*)(const long long *, int, int, int, XScale, const int *, int *, uint16_t *, long long, int);
+  // up to 4 slices a sum of nao products has at most 53 bits (2^(8(s-1) + 14) nao (1 + 2/256 + ...)) for
+  // nao <= 2^14
+  static const Kern exact[4] = {split_xblocks_kernel<1, false>, split_xblocks_kernel<2, false>,
+                                split_xblocks_kernel<3, false>, split_xblocks_kernel<4, false>};
+  static const Kern rounded[kSMax] = {split_xblocks_kernel<1, true>, split_xblocks_kernel<2, true>,
+                                      split_xblocks_kernel<3, true>, split_xblocks_kernel<4, true>,
+                                      split_xblocks_kernel<5, true>, split_xblocks_kernel<6, true>,
+                                      split_xblocks_kernel<7, true>, split_xblocks_kernel<8, true>};
+  if (nslices < 1 || nslices > kSMax || (nocc & 1)) return cudaErrorInvalidValue;
+  const Kern kern = nslices <= 4 && nao <= 16000 ? exact[nslices - 1] : rounded[nslices - 1];
   const size_t sm = sizeof(int) * (size_t)(kBlock + nocc);
-  static size_t attr = 48 * 1024;
-  if (sm > attr) {
-    cudaError_t e = cudaFuncSetAttribute(split_xblocks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (sm > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    attr = sm;
   }
   XScale xs{eB, eC, s_blk, T1};
   dim3 grid(nao, nblk);
-  split_xblocks_kernel<<<grid, kSplitXThreads, sm, st>>>(R, naux, nao, nocc, nslices, xs, rowE, eX, Xd, kb_ld,
-                                                         nblk);
+  kern<<<grid, kSplitXThreads, sm, st>>>(R, naux, nao, nocc, xs, rowE, eX, Xd, kb_ld, nblk);
   return cudaGetLastError();
 }
 
