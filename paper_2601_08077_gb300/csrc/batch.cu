@@ -131,13 +131,10 @@ df_status enqueue_K(df_batch *b, const double *const *C, const int *nocc, int s,
   for (int i = 0; i < n; ++i) {
     df_ctx *c = b->ctx[i];
     const long long c_plane = (long long)c->nocc_max * c->ld_nao;
-    if (df::launch_split_cols_bf16(C[i], c->nao, nocc[i], s, c->eC, c->Cd, c->ld_nao, c_plane, st) != cudaSuccess)
+    if (df::launch_split_cols_bf16(C[i], c->nao, nocc[i], s, c->eC, c->Cd, c->ld_nao, c_plane, st, c->rowE,
+                                   c->nblk * c->nao) != cudaSuccess)
       return DF_ERR_CUDA;
   }
-  for (int i = 0; i < n; ++i)
-    if (cudaMemsetAsync(b->ctx[i]->rowE, 0x80, sizeof(int) * (size_t)b->ctx[i]->nblk * b->ctx[i]->nao, st) !=
-        cudaSuccess)
-      return DF_ERR_CUDA;
   df::SgGroup g1{b->params1, b->maps1, b->off1, n, b->total1};
   if (df::launch_slice_gemm_grouped(df::kModeX, g1, b->status, 0, st, b->pairs1) !=
       cudaSuccess)

@@ -277,12 +277,42 @@ __global__ void __launch_bounds__(256, 5) coulomb_kernel(const double *__restric
   }
 }
 
-// Partial sums: [0] sum D.J, [1] sum rho.rho, [2] sum D.K, one triple per block.
-__global__ void __launch_bounds__(256) energy_partials_kernel(const double *__restrict__ D,
-                                                              const double *__restrict__ J,
-                                                              const double *__restrict__ K,
-                                                              const double *__restrict__ rho, long long n2,
-                                                              int naux, double *__restrict__ part) {
+// True in every thread of the last CTA of the grid to arrive here (each CTA's
+// global writes before it are visible to that CTA); it also resets the ticket
+// for the next launch.
+__device__ __forceinline__ bool last_block(unsigned *ticket) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (last) *ticket = 0u;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// Sum of the values of a 256-thread block, in thread 0 (fixed order).
+__device__ __forceinline__ double block_sum(double v, double *red) {
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < 8; ++w) s += red[w];
+  __syncthreads();
+  return s;
+}
+
+// E[0] = 1/2 sum D.J, E[1] = 1/2 sum rho.rho, E[2] = -1/2 sum D.K: partial sums
+// per block, added by the last block to finish (thread t takes blocks t, t + 256,
+// ..., then the block sum: the same order on every run).  A second launch whose
+// one thread walked 296 partials took 54 us of an SCF step of 204 (20 atoms).
+__global__ void __launch_bounds__(256) energy_kernel(const double *__restrict__ D, const double *__restrict__ J,
+                                                     const double *__restrict__ K, const double *__restrict__ rho,
+                                                     long long n2, int naux, double *__restrict__ part,
+                                                     unsigned *__restrict__ ticket, double *__restrict__ E) {
   double a = 0.0, b = 0.0, c = 0.0;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += stride) {
@@ -293,69 +323,55 @@ __global__ void __launch_bounds__(256) energy_partials_kernel(const double *__re
   if (rho)
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < naux; i += stride)
       b = fma(rho[i], rho[i], b);
-  a = warp_sum(a);
-  b = warp_sum(b);
-  c = warp_sum(c);
-  __shared__ double red[3][8];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) {
-    red[0][warp] = a;
-    red[1][warp] = b;
-    red[2][warp] = c;
-  }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += red[threadIdx.x][w];
-    part[blockIdx.x * 3 + threadIdx.x] = s;
-  }
-}
-
-__global__ void energy_final_kernel(const double *__restrict__ part, int nblocks, double *__restrict__ E) {
+  __shared__ double red[8];
+  a = block_sum(a, red);
+  b = block_sum(b, red);
+  c = block_sum(c, red);
   if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0, c = 0.0;
-    for (int i = 0; i < nblocks; ++i) {
-      a += part[3 * i];
-      b += part[3 * i + 1];
-      c += part[3 * i + 2];
-    }
+    part[blockIdx.x * 3] = a;
+    part[blockIdx.x * 3 + 1] = b;
+    part[blockIdx.x * 3 + 2] = c;
+  }
+  if (!last_block(ticket)) return;
+  a = b = c = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) {
+    a += __ldcg(part + 3 * i);
+    b += __ldcg(part + 3 * i + 1);
+    c += __ldcg(part + 3 * i + 2);
+  }
+  a = block_sum(a, red);
+  b = block_sum(b, red);
+  c = block_sum(c, red);
+  if (threadIdx.x == 0) {
     E[0] = 0.5 * a;
     E[1] = 0.5 * b;
     E[2] = -0.5 * c;
   }
 }
 
-// Partial sums of (D - D_prev)^2 per block; D_prev == nullptr: no previous density.
-__global__ void __launch_bounds__(256) density_change_kernel(const double *__restrict__ D,
-                                                             const double *__restrict__ Dprev, long long n2,
-                                                             double *__restrict__ part) {
+// *out = ||D - D_prev||_F (1 when there is no previous density), D_prev = D, in
+// one pass; the last block adds the partial sums.
+__global__ void __launch_bounds__(256) density_change_kernel(const double *__restrict__ D, double *__restrict__ Dprev,
+                                                             bool have_prev, long long n2,
+                                                             double *__restrict__ part,
+                                                             unsigned *__restrict__ ticket,
+                                                             double *__restrict__ out) {
   double a = 0.0;
-  if (Dprev) {
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += stride) {
-      const double d = D[i] - Dprev[i];
-      a = fma(d, d, a);
-    }
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += stride) {
+    const double v = D[i];
+    const double d = have_prev ? v - Dprev[i] : 0.0;
+    Dprev[i] = v;
+    a = fma(d, d, a);
   }
-  a = warp_sum(a);
   __shared__ double red[8];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += red[w];
-    part[blockIdx.x] = s;
-  }
-}
-
-// ||D - D_prev||_F from the partials, or 1 when there is no previous density.
-__global__ void density_change_final_kernel(const double *__restrict__ part, int nblocks, bool have_prev,
-                                            double *__restrict__ out) {
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < nblocks; ++i) s += part[i];
-    *out = have_prev ? sqrt(s) : 1.0;
-  }
+  a = block_sum(a, red);
+  if (threadIdx.x == 0) part[blockIdx.x] = a;
+  if (!last_block(ticket)) return;
+  a = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) a += __ldcg(part + i);
+  a = block_sum(a, red);
+  if (threadIdx.x == 0) *out = have_prev ? sqrt(a) : 1.0;
 }
 
 // Packed B: flag[k] = 1 when the packed pair k (of the upper triangle) is
@@ -439,14 +455,9 @@ cudaError_t launch_tile_masks(const uint32_t *mask_mu, int naux, int nao, uint32
 }
 
 cudaError_t launch_density_change(const double *D, double *Dprev, bool have_prev, long long n2, double *part,
-                                  double *out, cudaStream_t st) {
-  density_change_kernel<<<kDensityChangeBlocks, 256, 0, st>>>(D, have_prev ? Dprev : nullptr, n2, part);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  density_change_final_kernel<<<1, 32, 0, st>>>(part, kDensityChangeBlocks, have_prev, out);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return cudaMemcpyAsync(Dprev, D, sizeof(double) * n2, cudaMemcpyDeviceToDevice, st);
+                                  unsigned *ticket, double *out, cudaStream_t st) {
+  density_change_kernel<<<kDensityChangeBlocks, 256, 0, st>>>(D, Dprev, have_prev, n2, part, ticket, out);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, double *rho, cudaStream_t st,
@@ -488,11 +499,8 @@ cudaError_t launch_coulomb(const double *B, const double *rho, int naux, int nao
 }
 
 cudaError_t launch_energy(const double *D, const double *J, const double *K, const double *rho, int nao, int naux,
-                          double *partials, double *E_dev, cudaStream_t st) {
-  energy_partials_kernel<<<kEnergyBlocks, 256, 0, st>>>(D, J, K, rho, (long long)nao * nao, naux, partials);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  energy_final_kernel<<<1, 32, 0, st>>>(partials, kEnergyBlocks, E_dev);
+                          double *partials, unsigned *ticket, double *E_dev, cudaStream_t st) {
+  energy_kernel<<<kEnergyBlocks, 256, 0, st>>>(D, J, K, rho, (long long)nao * nao, naux, partials, ticket, E_dev);
   return cudaGetLastError();
 }
 

@@ -240,13 +240,13 @@ df_status k_front(df_ctx *c, const double *C, int nocc, const int *sb, int c_pla
   const long long c_plane = (long long)c->nocc_max * c->ld_nao;
   {
     PhaseTimer t(c, DF_PHASE_SPLIT_C, st);
-    DF_TRY(c, df::launch_split_cols_bf16(C, nao, nocc, c_planes, c->eC, c->Cd, c->ld_nao, c_plane, st));
+    DF_TRY(c, df::launch_split_cols_bf16(C, nao, nocc, c_planes, c->eC, c->Cd, c->ld_nao, c_plane, st, c->rowE,
+                                         c->nblk * nao));
   }
   // 2. X = B C
   df::SgParams p;
   df::SgMaps maps;
   if (!df::gemm1_setup(c, nocc, p, maps)) return record(c, DF_ERR_CUDA);
-  DF_TRY(c, cudaMemsetAsync(c->rowE, 0x80, sizeof(int) * (size_t)c->nblk * nao, st));
   {
     PhaseTimer t(c, DF_PHASE_GEMM1, st);
     DF_TRY(c, df::launch_slice_gemm(p, maps, st));
@@ -411,6 +411,8 @@ df_status df_create(df_ctx **out, int nao, int naux, int nocc_max, int s_max) {
   if (e == cudaSuccess) e = alloc(c, &c->Dprev, (size_t)nao * nao);
   if (e == cudaSuccess) e = alloc(c, &c->dD, (size_t)1);
   if (e == cudaSuccess) e = alloc(c, &c->dD_part, (size_t)df::kDensityChangeBlocks);
+  if (e == cudaSuccess) e = alloc(c, &c->tickets, (size_t)2);
+  if (e == cudaSuccess) e = cudaMemset(c->tickets, 0, 2 * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void **>(&c->sblk_host), sizeof(int) * c->nblk);
   if (e == cudaSuccess) e = cudaMemset(c->status, 0, sizeof(int));
   if (e == cudaSuccess) {
@@ -452,6 +454,7 @@ void df_destroy(df_ctx *c) {
   cudaFree(c->Dprev);
   cudaFree(c->dD);
   cudaFree(c->dD_part);
+  cudaFree(c->tickets);
   cudaFree(c->lF);
   cudaFree(c->lprobs);
   cudaFree(c->lpick);
@@ -632,7 +635,7 @@ df_status df_build_J(df_ctx *c, const double *D, double *J, double *rho, void *s
   if (rho && rho != c->rho)
     DF_TRY(c, cudaMemcpyAsync(c->rho, rho, sizeof(double) * c->naux, cudaMemcpyDeviceToDevice, st));
   // the density change since the last Coulomb build (an input of the learned slice counts)
-  DF_TRY(c, df::launch_density_change(D, c->Dprev, c->have_Dprev, (long long)c->nao * c->nao, c->dD_part, c->dD, st));
+  DF_TRY(c, df::launch_density_change(D, c->Dprev, c->have_Dprev, (long long)c->nao * c->nao, c->dD_part, c->tickets, c->dD, st));
   c->have_Dprev = true;
   return DF_OK;
 }
@@ -701,7 +704,7 @@ df_status df_build_JK(df_ctx *c, const double *D, const double *C, int nocc, int
   DF_TRY(c, cudaStreamWaitEvent(st, c->jk_join, 0));
   r = df::k_back(c, nocc, K, st);
   if (r != DF_OK) return r;
-  DF_TRY(c, df::launch_density_change(D, c->Dprev, c->have_Dprev, (long long)c->nao * c->nao, c->dD_part, c->dD, st));
+  DF_TRY(c, df::launch_density_change(D, c->Dprev, c->have_Dprev, (long long)c->nao * c->nao, c->dD_part, c->tickets, c->dD, st));
   c->have_Dprev = true;
   fill_stats(stats, c, sb, level);
   return DF_OK;
@@ -748,7 +751,7 @@ df_status df_energy(df_ctx *c, const double *D, const double *J, const double *K
   const double *r = rho ? rho : c->rho;
   {
     PhaseTimer t(c, DF_PHASE_ENERGY, st);
-    DF_TRY(c, df::launch_energy(D, J, K, r, c->nao, c->naux, c->epart, c->E, st));
+    DF_TRY(c, df::launch_energy(D, J, K, r, c->nao, c->naux, c->epart, c->tickets + 1, c->E, st));
   }
   DF_TRY(c, cudaMemcpyAsync(E_host, c->E, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
   DF_TRY(c, cudaStreamSynchronize(st));

@@ -64,6 +64,7 @@ struct df_ctx {
   double *Dprev = nullptr;   // [nao][nao] the density of the last df_build_J
   double *dD = nullptr;      // device scalar ||D - D_prev||_F (1 before any previous density)
   double *dD_part = nullptr; // partial sums of the reduction
+  unsigned *tickets = nullptr; // finished-block counters of the density-change and energy reductions
   bool have_Dprev = false;
   // learned slice counts (df_set_predictor; the network's kernels live in mlp.cu)
   df_mlp *pred = nullptr;
@@ -106,7 +107,8 @@ int level_count(const df_ctx *c, int level);
 // context's current level, checked against the level's error bound.
 df_status build_K_learned(df_ctx *c, const double *C, int nocc, double *K, df_kstats *stats, cudaStream_t st);
 // Launch of ||D - D_prev||_F into c->dD (1 when there is no previous density)
-// and the copy D -> D_prev (coulomb.cu).
+// and the copy D -> D_prev (coulomb.cu).  ticket: a zeroed word that counts the
+// launch's finished blocks and is zero again afterwards.
 cudaError_t launch_density_change(const double *D, double *Dprev, bool have_prev, long long n2, double *part,
-                                  double *out, cudaStream_t st);
+                                  unsigned *ticket, double *out, cudaStream_t st);
 }  // namespace df

@@ -152,7 +152,8 @@ cudaError_t launch_setup_rows(const double *B, int naux, int nao, int nslices, i
 cudaError_t launch_split_rows_int8(const double *A, int rows, int cols, int ld, int nslices, int *exps,
                                    int8_t *digits, cudaStream_t st);
 cudaError_t launch_split_cols_bf16(const double *C, int nrows, int ncols, int nslices, int *exps,
-                                   uint16_t *digits, long long dld, long long plane_stride, cudaStream_t st);
+                                   uint16_t *digits, long long dld, long long plane_stride, cudaStream_t st,
+                                   int *reset = nullptr, int nreset = 0);
 struct ShiftTable {
   int v[9];
 };
@@ -209,6 +210,6 @@ cudaError_t launch_split_rows_packed(const double *Bp, int naux, int nao, int ns
 // Per 128-row tile of the (P, mu) rows, the OR of its rows' mu masks.
 cudaError_t launch_tile_masks(const uint32_t *mask_mu, int naux, int nao, uint32_t *mask_tile, cudaStream_t st);
 cudaError_t launch_energy(const double *D, const double *J, const double *K, const double *rho, int nao,
-                          int naux, double *partials, double *E_dev, cudaStream_t st);
+                          int naux, double *partials, unsigned *ticket, double *E_dev, cudaStream_t st);
 
 }  // namespace df

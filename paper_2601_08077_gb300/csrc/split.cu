@@ -266,27 +266,68 @@ __global__ void split_rows_int8_kernel(const double *__restrict__ A, int rows, i
   }
 }
 
-// One warp per column c of C [nrows][ncols]: digits go to [t][c][r] (K-major).
-__global__ void split_cols_bf16_kernel(const double *__restrict__ C, int nrows, int ncols, int nslices,
-                                       int *__restrict__ exps, uint16_t *__restrict__ digits, long long dld,
-                                       long long plane_stride) {
-  const int lane = threadIdx.x & 31;
-  const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (c >= ncols) return;
+// C [nrows][ncols] by columns: digits go to [t][c][r] (K-major).  A CTA takes 8
+// columns with 512 threads, a warp 4 rows x 8 columns at a time (64-byte pieces
+// of C's rows); all its loads are in flight before the first is used, and the
+// values stay in registers between the maximum and the digits (up to 8 per
+// thread, 512 rows; further rows are read again).  A warp per column walked them
+// in two dependent passes (250 columns of 1200: 29 us).
+// reset (optional): nreset words set to kRowBoundNone on the way, the row bounds
+// that the first exchange GEMM is about to raise.
+constexpr int kColsT = 512;
+constexpr int kColsHeld = 8;
+__global__ void __launch_bounds__(kColsT) split_cols_bf16_kernel(const double *__restrict__ C, int nrows, int ncols,
+                                                                 int nslices, int *__restrict__ exps,
+                                                                 uint16_t *__restrict__ digits, long long dld,
+                                                                 long long plane_stride, int *__restrict__ reset,
+                                                                 int nreset) {
+  for (int i = blockIdx.x * kColsT + threadIdx.x; i < nreset; i += gridDim.x * kColsT) reset[i] = kRowBoundNone;
+  const int c = blockIdx.x * 8 + (threadIdx.x & 7);
+  const int r0 = threadIdx.x >> 3;
+  constexpr int step = kColsT / 8;
+  const bool col = c < ncols;
+  uint64_t held[kColsHeld];
   uint64_t m = 0;
-  for (int r = lane; r < nrows; r += 32) {
-    uint64_t a = abs_bits(C[(long long)r * ncols + c]);
+#pragma unroll
+  for (int k = 0; k < kColsHeld; ++k) {
+    const int r = r0 + k * step;
+    held[k] = col && r < nrows ? (uint64_t)__double_as_longlong(__ldg(C + (long long)r * ncols + c)) : 0ull;
+  }
+#pragma unroll
+  for (int k = 0; k < kColsHeld; ++k) {
+    const uint64_t a = held[k] & 0x7FFFFFFFFFFFFFFFull;
     m = a > m ? a : m;
   }
-  m = warp_max_u64(m);
-  const int e = exponent_from_max_bits_dev(m);
-  if (lane == 0) exps[c] = e;
-  for (int r = lane; r < nrows; r += 32) {
-    int d[kSMax];
-    balanced_digits(scaled_rne((uint64_t)__double_as_longlong(C[(long long)r * ncols + c]), e), d);
-    for (int t = 0; t < nslices; ++t)
-      digits[(long long)t * plane_stride + (long long)c * dld + r] = int_to_bf16_bits(d[t]);
+  for (int r = r0 + kColsHeld * step; col && r < nrows; r += step) {
+    const uint64_t a = abs_bits(__ldg(C + (long long)r * ncols + c));
+    m = a > m ? a : m;
   }
+#pragma unroll
+  for (int o = 8; o < 32; o <<= 1) {
+    const uint64_t w = __shfl_xor_sync(0xffffffffu, m, o);
+    m = w > m ? w : m;
+  }
+  __shared__ uint64_t red[kColsT / 32][8];
+  if ((threadIdx.x & 31) < 8) red[threadIdx.x >> 5][threadIdx.x & 7] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kColsT / 32; ++w) m = red[w][threadIdx.x & 7] > m ? red[w][threadIdx.x & 7] : m;
+  if (!col) return;
+  const int e = exponent_from_max_bits_dev(m);
+  if (r0 == 0) exps[c] = e;
+  uint16_t *out = digits + (long long)c * dld;
+  auto put = [&](uint64_t bits, int r) {
+    int d[kSMax];
+    balanced_digits(scaled_rne(bits, e), d);
+#pragma unroll
+    for (int t = 0; t < kSMax; ++t)
+      if (t < nslices) out[(long long)t * plane_stride + r] = int_to_bf16_bits(d[t]);
+  };
+#pragma unroll
+  for (int k = 0; k < kColsHeld; ++k)
+    if (r0 + k * step < nrows) put(held[k], r0 + k * step);
+  for (int r = r0 + kColsHeld * step; r < nrows; r += step)
+    put((uint64_t)__double_as_longlong(__ldg(C + (long long)r * ncols + c)), r);
 }
 
 // The X split.  One CTA per (block b, row mu) of X [naux][nao][nocc] (nocc even):
@@ -520,26 +561,49 @@ __global__ void __launch_bounds__(kSplitXThreads, 5)
 // K[mu][nu] = sum_b fl( 2^(eX[b,mu] + eX[b,nu] - 14 - 8(s_b - 1) + T(s_b)) * sum_sp R[b,sp] ),
 // blocks in order (FP64), where R[b,sp][hi][lo] are the exact int64 partials of
 // the second exchange GEMM (lower block-triangle, transposed) and the sum over
-// the K splits of a block is exact.
-__global__ void kpart_reduce_kernel(const long long *__restrict__ Rp, const int *__restrict__ eX,
-                                    const int *__restrict__ s_blk, ShiftTable shiftT, int nao, int nblk, int nsplit,
-                                    double *__restrict__ K) {
-  const int nu = blockIdx.x * blockDim.x + threadIdx.x;
-  const int mu = blockIdx.y;
-  if (nu >= nao) return;
-  const int hi = mu > nu ? mu : nu;
-  const int lo = mu > nu ? nu : mu;
-  const long long off = (long long)hi * nao + lo;
+// the K splits of a block is exact.  A CTA takes a 32 x 8 tile of the lower
+// triangle (rows hi, columns lo, so the partials are read along rows), four
+// blocks' partials in flight, and writes both halves of K, the upper one through
+// shared memory.  (One thread per element of the whole square read half of the
+// partials column by column: 240 atoms 153 us.)
+__global__ void __launch_bounds__(256) kpart_reduce_kernel(const long long *__restrict__ Rp,
+                                                           const int *__restrict__ eX,
+                                                           const int *__restrict__ s_blk, ShiftTable shiftT, int nao,
+                                                           int nblk, int nsplit, double *__restrict__ K) {
+  const int lo0 = blockIdx.x * 32, hi0 = blockIdx.y * 8;
+  if (lo0 > hi0 + 7) return;  // above the diagonal
+  const int lo = lo0 + (threadIdx.x & 31), hi = hi0 + (threadIdx.x >> 5);
   const long long bs = (long long)nao * nao;
   double acc = 0.0;
-  for (int b = 0; b < nblk; ++b) {
-    long long R = 0;
-    for (int sp = 0; sp < nsplit; ++sp) R += Rp[((long long)b * nsplit + sp) * bs + off];
-    const int s = s_blk[b];
-    const int k = eX[b * nao + mu] + eX[b * nao + nu] - 14 - 8 * (s - 1) + shiftT.v[s];
-    acc += ldexp_i64(R, k);
+  if (hi < nao && lo <= hi) {
+    const long long *src = Rp + (long long)hi * nao + lo;
+    constexpr int kU = 4;
+    for (int b0 = 0; b0 < nblk; b0 += kU) {
+      long long R[kU];
+      int k[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int b = b0 + u;
+        R[u] = 0;
+        k[u] = 0;
+        if (b < nblk) {
+          const int s = __ldg(s_blk + b);
+          k[u] = __ldg(eX + b * nao + hi) + __ldg(eX + b * nao + lo) - 14 - 8 * (s - 1) + shiftT.v[s];
+#pragma unroll 4
+          for (int sp = 0; sp < nsplit; ++sp) R[u] += __ldg(src + ((long long)b * nsplit + sp) * bs);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+        if (b0 + u < nblk) acc += ldexp_i64(R[u], k[u]);
+    }
+    K[(long long)hi * nao + lo] = acc;
   }
-  K[(long long)mu * nao + nu] = acc;
+  __shared__ double t[32][9];
+  t[threadIdx.x & 31][threadIdx.x >> 5] = acc;
+  __syncthreads();
+  const int row = lo0 + (threadIdx.x >> 3), col = hi0 + (threadIdx.x & 7);
+  if (row < nao && col < nao && row < col) K[(long long)row * nao + col] = t[threadIdx.x >> 3][threadIdx.x & 7];
 }
 
 }  // namespace
@@ -587,10 +651,11 @@ cudaError_t launch_split_rows_int8(const double *A, int rows, int cols, int ld, 
 }
 
 cudaError_t launch_split_cols_bf16(const double *C, int nrows, int ncols, int nslices, int *exps,
-                                   uint16_t *digits, long long dld, long long plane_stride, cudaStream_t st) {
+                                   uint16_t *digits, long long dld, long long plane_stride, cudaStream_t st,
+                                   int *reset, int nreset) {
   if (ncols <= 0) return cudaSuccess;
-  split_cols_bf16_kernel<<<(ncols + 7) / 8, 256, 0, st>>>(C, nrows, ncols, nslices, exps, digits, dld,
-                                                          plane_stride);
+  split_cols_bf16_kernel<<<(ncols + 7) / 8, kColsT, 0, st>>>(C, nrows, ncols, nslices, exps, digits, dld,
+                                                             plane_stride, reset, nreset);
   return cudaGetLastError();
 }
 
@@ -621,8 +686,8 @@ cudaError_t launch_split_xblocks(const long long *R, int naux, int nao, int nocc
 
 cudaError_t launch_kpart_reduce(const long long *Rp, const int *eX, const int *s_blk, ShiftTable shiftT, int nao,
                                 int nblk, int nsplit, double *K, cudaStream_t st) {
-  dim3 grid((nao + 127) / 128, nao);
-  kpart_reduce_kernel<<<grid, 128, 0, st>>>(Rp, eX, s_blk, shiftT, nao, nblk, nsplit, K);
+  dim3 grid((nao + 31) / 32, (nao + 7) / 8);
+  kpart_reduce_kernel<<<grid, 256, 0, st>>>(Rp, eX, s_blk, shiftT, nao, nblk, nsplit, K);
   return cudaGetLastError();
 }
 
