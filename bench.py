@@ -36,9 +36,7 @@ import numpy as np  # noqa: E402
 
 METRIC = "DF K-build effective FP64 TFLOP/s, INT8-adaptive vs native FP64, max|dK|<=1e-10"
 UNIT = "TFLOP/s"
-LAUNCHES_PER_STEP = 11     # rho, coulomb, 2 density-change kernels, split C, GEMM1, split X, GEMM2, reduce,
-                           # 2 energy kernels
-FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
+LAUNCHES_PER_STEP = 7      # split C, GEMM1 (with rho), split X, GEMM2 (with J), reduce, density change, energy
 
 
 def parse():
@@ -62,7 +60,7 @@ def parse():
                     help="keep only the first N 128-function auxiliary blocks of the workload (a smaller case of "
                          "the same kernels, for profiling); 0 keeps them all")
     ap.add_argument("--jk-overlap", type=int, choices=[0, 1, 2, 3, 4], default=4,
-                    help="CTAs per SM of rho and J beside the X split in the J + K build (df_build_JK); "
+                    help="1..4 (alike) run rho and J beside the exchange GEMMs in the J + K build (df_build_JK); "
                          "0 runs J, then K, in one stream")
     ap.add_argument("--cluster-pairs", type=int, choices=[0, 1, 2], default=1,
                     help="slice GEMMs on CTA pairs (cta_group::2): 0 never, 1 the first GEMM, 2 both GEMMs")
@@ -679,8 +677,8 @@ def main():
     ms = shard.max_over_ranks(ms, dev)
     ctx.sync_status()
 
-    # the exchange build alone (INT8 slices): in the timed step the X split shares
-    # the SMs with rho and J, so its phase time there is not the K build's
+    # the exchange build alone (INT8 slices): in the timed step the GEMMs share
+    # the SMs with rho and J, so their phase times there are not the K build's
     nk = max(1, min(10, args.steps))
     torch.cuda.synchronize()
     ctx.phase_times()
@@ -757,9 +755,9 @@ def main():
                    "slice_count": "fixed for every step (5 = Table 1 level 2's count, the first level meeting "
                                   "max|dK| <= 1e-10 max|K|)" if s == 5 else "fixed for every step", "l2": "inputs larger than L2 (B %.1f GB)" % (B_bytes / 1e9),
                    "cluster_pairs": args.cluster_pairs,
-                   "jk_overlap": ("J, then K, in one stream (df_build_JK; a block-sparse B runs its masked "
-                                  "kernels in order)" if sparsity[1] < 1.0 else
-                                  "rho and J on %d CTAs per SM beside the X split (df_build_JK)" % args.jk_overlap)
+                   "jk_overlap": ("J, then K, in one stream (df_build_JK; a B of mostly zero chunks runs its "
+                                  "masked kernels in order)" if sparsity[1] < 0.5 else
+                                  "rho and J by spare warps of the exchange GEMMs (df_build_JK)")
                                  if args.jk_overlap else "J, then K, in one stream",
                    "parallelism": "replicas" if world > 1 else "single"},
         "e2e": {"value": FK / (ms_e2e * 1e-3) / 1e12 * world, "unit": UNIT, "h2d_bytes_per_step": h2d,
@@ -775,8 +773,8 @@ def main():
         "fp64_native": {"k_build_ms": ms_fp64, "tflops": FK / (ms_fp64 * 1e-3) / 1e12,
                         "speedup_of_int8": ms_fp64 / ms_k},
         "phases_ms_per_step": {k: v[0] / args.steps for k, v in phases.items()},
-        "phases_note": "CUDA-event intervals per phase; rho and J run beside the X split (df_build_JK), "
-                       "so those three intervals overlap" if args.jk_overlap else "phases in one stream, in order",
+        "phases_note": "CUDA-event intervals per phase; rho and J run inside gemm1 and gemm2 (df_build_JK)"
+                       if args.jk_overlap else "phases in one stream, in order",
         "k_build_tflops": FK / (ms_k * 1e-3) / 1e12,
         "k_build_alone": {"ms": ms_k, "builds": nk,
                           "phases_ms": {k: v[0] / nk for k, v in k_phases.items() if v[1]}},

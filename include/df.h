@@ -143,16 +143,13 @@ df_status df_build_K(df_ctx *ctx, const double *C_dev, int nocc, int nslices, do
  * df_build_J(ctx, D_dev, J_dev, rho_dev, stream) followed by
  * df_build_K(ctx, C_dev, nocc, nslices, K_dev, stats, stream), with the same
  * arguments, ownership and errors.  For an emulated count (1..8, or -1 at a
- * level that runs slices) the FP64 rho and J kernels run on an internal
- * high-priority stream of the context, forked from `stream` after the first
- * exchange GEMM and joined back before the second: they share the SMs with
- * the X split (rho and J are bound by GB300's FP64 pipe, the X split by HBM
- * and integer work), from short grids of a few CTAs per SM
- * (DF_OPT_JK_OVERLAP).  Native FP64 (0), the learned counts (-2 at a level
- * above 0), a block-sparse B (df_sparsity below 1, with DF_OPT_SPARSE on) and
- * DF_OPT_JK_OVERLAP = 0 run the two builds in order in `stream`.  Calls on
- * one context must not overlap (they share the internal stream and its work
- * counters). */
+ * level that runs slices) spare warps of the two exchange GEMMs run the FP64
+ * passes, rho beside the first and J beside the second: rho and J stream B
+ * through the FP64 pipe, which the GEMMs leave idle.  Native FP64 (0), the
+ * learned counts (-2 at a level above 0), a B of mostly zero chunks
+ * (df_sparsity's frac_chunks below 1/2) and DF_OPT_JK_OVERLAP = 0 run the two
+ * builds one after the other.  All of it is in `stream`.  Calls on one context
+ * must not overlap (they share its work counters). */
 df_status df_build_JK(df_ctx *ctx, const double *D_dev, const double *C_dev, int nocc, int nslices,
                       double *J_dev, double *rho_dev, double *K_dev, df_kstats *stats, void *stream);
 
@@ -406,8 +403,8 @@ int64_t df_workspace_bytes(const df_ctx *ctx);
  * counts the surviving pairs as N_scr).  At setup the library records, per mu,
  * which 64-wide chunks of nu hold a nonzero B_P mu nu for some P; when some
  * chunk is zero (and nao <= 2048) the first exchange GEMM runs only the
- * nonzero 64-wide K tiles of each 128-row tile of B's (P, mu) rows, and rho
- * and J skip the zero chunks.  Skipped terms are exact zeros: every result is
+ * nonzero 64-wide K tiles of each 128-row tile of B's (P, mu) rows, and, when
+ * most chunks are zero, rho and J skip them.  Skipped terms are exact zeros: every result is
  * the one of the dense build.  frac_ktiles: nonzero K tiles / all of the first
  * GEMM's row tiles; frac_chunks: nonzero (mu, chunk) pairs of the upper
  * triangle / all.  Both 1 for a B without zero chunks.  DF_ERR_STATE before
@@ -432,9 +429,8 @@ df_status df_sparsity(const df_ctx *ctx, double *frac_ktiles, double *frac_chunk
 /* DF_OPT_SPARSE — whether the builds use the block sparsity of a screened B
  * (df_sparsity): 1 (default) when df_setup found zero chunks, 0 never. */
 #define DF_OPT_SPARSE 2
-/* DF_OPT_JK_OVERLAP — CTAs per SM of the rho and J kernels that df_build_JK
- * runs beside the X split: 1..4 (default 4, the fastest at 240 atoms), 0 = no
- * overlap (J, then K, in the caller's stream). */
+/* DF_OPT_JK_OVERLAP — whether df_build_JK runs rho and J beside the exchange
+ * GEMMs: 1..4 (all alike; default 4) yes, 0 no (J, then K). */
 #define DF_OPT_JK_OVERLAP 3
 df_status df_set_option(df_ctx *ctx, int option, int value);
 

@@ -131,8 +131,11 @@ df_status enqueue_K(df_batch *b, const double *const *C, const int *nocc, int s,
   for (int i = 0; i < n; ++i) {
     df_ctx *c = b->ctx[i];
     const long long c_plane = (long long)c->nocc_max * c->ld_nao;
-    if (df::launch_split_cols_bf16(C[i], c->nao, nocc[i], s, c->eC, c->Cd, c->ld_nao, c_plane, st, c->rowE,
-                                   c->nblk * c->nao) != cudaSuccess)
+    df::ColsExtra extra{};
+    extra.reset = c->rowE;
+    extra.nreset = c->nblk * c->nao;
+    if (df::launch_split_cols_bf16(C[i], c->nao, nocc[i], s, c->eC, c->Cd, c->ld_nao, c_plane, st, extra) !=
+        cudaSuccess)
       return DF_ERR_CUDA;
   }
   df::SgGroup g1{b->params1, b->maps1, b->off1, n, b->total1};
@@ -147,7 +150,7 @@ df_status enqueue_K(df_batch *b, const double *const *C, const int *nocc, int s,
     for (int q = 0; q <= 8; ++q) t1.v[q] = df::fixed_point_shift(q, k1);
     if (df::launch_split_xblocks(reinterpret_cast<const long long *>(c->X), c->naux, c->nao, df::even_nocc(nocc[i]), s, c->eB,
                                  c->eC, c->sblk, t1, c->rowE, c->eX, c->Xd, df::xdigit_ld(nocc[i]), c->nblk,
-                                 b->side[i % df_batch::kFan]) != cudaSuccess)
+                                 df::RhoParts{}, b->side[i % df_batch::kFan]) != cudaSuccess)
       return DF_ERR_CUDA;
   }
   if (join(b, st) != cudaSuccess) return DF_ERR_CUDA;
@@ -300,7 +303,8 @@ df_status df_batch_build_J(df_batch *b, const double *const *D, double *const *J
       df_ctx *c = b->ctx[i];
       cudaStream_t si = b->side[i % df_batch::kFan];
       const uint32_t *mk = df::use_mask_mu(c);
-      if (df::launch_rho(c->B, D[i], c->naux, c->nao, c->rho, si, mk, c->packed, nullptr, 0, c->sparse) != cudaSuccess) return DF_ERR_CUDA;
+      if (df::launch_rho(c->B, D[i], c->naux, c->nao, c->rho, nullptr, si, mk, c->packed, c->rows) != cudaSuccess)
+        return DF_ERR_CUDA;
       if (df::launch_coulomb(c->B, c->rho, c->naux, c->nao, J[i], si, mk, c->packed) != cudaSuccess)
         return DF_ERR_CUDA;
     }

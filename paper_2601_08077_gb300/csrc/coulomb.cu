@@ -27,124 +27,6 @@ namespace df {
 
 namespace {
 
-// Start of row mu in a packed upper triangle of order nao.
-__device__ __forceinline__ long long packed_row(int mu, int nao) {
-  return (long long)mu * nao - (long long)mu * (mu - 1) / 2;
-}
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Work items of a launch: with a null counter the CTA takes its own index
-// once; otherwise the CTAs of a short grid (a few per SM, sharing the SMs
-// with another kernel) take items from the counter until they run out.  The
-// value is uniform over the CTA.
-__device__ __forceinline__ int take_item(int *work, int *slot) {
-  if (threadIdx.x == 0) *slot = atomicAdd(work, 1);
-  __syncthreads();
-  const int v = *slot;
-  __syncthreads();
-  return v;
-}
-
-// The strictly upper elements of B_P in row-pair order: pair q < nao/2 is
-// row q from nu = q + 1 followed by row nao-1-q from nu = nao-q (nao - 1
-// elements together, so every pair has the same length); for odd nao the
-// middle row, q = nao/2, comes last alone.  Thread t of the CTA takes the
-// elements t, t + 256, t + 512, ...: each warp reads 32 consecutive values of
-// one row, and no thread has a per-row tail.
-struct PairStream {
-  int q, e;       // the current element: offset e in pair q
-  int nao, L;     // L = nao - 1, the length of a full pair
-  __device__ __forceinline__ void init(int j0, int n) {
-    nao = n;
-    L = n - 1;
-    q = j0 / L;
-    e = j0 - q * L;
-  }
-  __device__ __forceinline__ bool valid() const {
-    return 2 * q + 1 < nao || (2 * q + 1 == nao && e < nao - 1 - q);
-  }
-  // (mu, nu), nu > mu, of the current element
-  __device__ __forceinline__ void at(int &mu, int &nu) const {
-    if (e < nao - 1 - q) {
-      mu = q;
-      nu = q + 1 + e;
-    } else {
-      mu = nao - 1 - q;
-      nu = e + 1;
-    }
-  }
-  __device__ __forceinline__ void advance(int step) {
-    e += step;
-    while (e >= L) {
-      e -= L;
-      ++q;
-    }
-  }
-};
-
-// rho_P for one P by one CTA of 256 threads:
-//   rho_P = sum_mu B_P mu mu D_mu mu + 2 sum_{mu < nu} B_P mu nu D_mu nu.
-// The diagonal terms are spread over the threads; the strictly upper ones
-// stream in row-pair order (PairStream), eight loads ahead of their FMAs (a
-// ring of registers, FMAs in stream order), so that a few CTAs per SM keep
-// enough bytes in flight to share the SM with another kernel.
-template <bool kPacked>
-__device__ __forceinline__ void rho_one(const double *__restrict__ B, const double *__restrict__ D, int nao,
-                                        double *__restrict__ rho, int P, double *red) {
-  constexpr int kQ = 8;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const double *BP = B + (long long)P * (kPacked ? (long long)nao * (nao + 1) / 2 : (long long)nao * nao);
-  auto badr = [&](int mu, int nu) -> const double * {
-    return kPacked ? BP + packed_row(mu, nao) + (nu - mu) : BP + (long long)mu * nao + nu;
-  };
-  double dia = 0.0;
-  for (int mu = tid; mu < nao; mu += 256) dia = fma(__ldg(badr(mu, mu)), __ldg(D + (long long)mu * nao + mu), dia);
-  double off = 0.0;
-  const long long total = (long long)nao * (nao - 1) / 2;
-  if (total > tid) {
-    PairStream ps;
-    ps.init(tid, nao);
-    double bq[kQ], dq[kQ];
-    auto fill = [&](int k) {
-      bq[k] = 0.0;
-      dq[k] = 0.0;
-      if (ps.valid()) {
-        int mu, nu;
-        ps.at(mu, nu);
-        bq[k] = __ldg(badr(mu, nu));
-        dq[k] = __ldg(D + (long long)mu * nao + nu);
-      }
-      ps.advance(256);
-    };
-#pragma unroll
-    for (int k = 0; k < kQ; ++k) fill(k);
-    const long long mine = (total - tid + 255) / 256;
-    const int rounds = (int)((mine + kQ - 1) / kQ);
-    for (int r = 0; r < rounds; ++r) {
-#pragma unroll
-      for (int k = 0; k < kQ; ++k) {
-        off = fma(bq[k], dq[k], off);
-        fill(k);
-      }
-    }
-  }
-  double v = 2.0 * off + dia;
-  v = warp_sum(v);
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  if (tid == 0) {
-    double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += red[w];
-    rho[P] = t;
-  }
-  __syncthreads();
-}
-
 // rho_P for a B with zero 64-wide chunks (a Schwarz-screened B), row by row:
 // warp w takes rows mu = w, w + 8, ...; lanes stride nu > mu.  With masks a
 // warp skips each 32-wide window whose chunks are all zero as a whole (no
@@ -154,8 +36,8 @@ __device__ __forceinline__ void rho_one(const double *__restrict__ B, const doub
 // element of the triangle to skip the zero ones.
 template <bool kPacked>
 __device__ __forceinline__ void rho_one_rows(const double *__restrict__ B, const double *__restrict__ D, int nao,
-                                             double *__restrict__ rho, const uint32_t *__restrict__ mask_mu, int P,
-                                             double *red) {
+                                             double *__restrict__ rho, double *__restrict__ rho2,
+                                             const uint32_t *__restrict__ mask_mu, int P, double *red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const double *BP = B + (long long)P * (kPacked ? (long long)nao * (nao + 1) / 2 : (long long)nao * nao);
   double off = 0.0, dia = 0.0;
@@ -183,98 +65,60 @@ __device__ __forceinline__ void rho_one_rows(const double *__restrict__ B, const
     double t = 0.0;
     for (int w = 0; w < 8; ++w) t += red[w];
     rho[P] = t;
+    if (rho2) rho2[P] = t;
   }
-  __syncthreads();
 }
 
-// One CTA per P (work == null), or a short grid taking P from the counter.
-// kRows: the row-by-row order of a B with zero chunks (masks optional).  At
-// most 48 registers, like the J kernel.
-template <bool kPacked, bool kRows>
-__global__ void __launch_bounds__(256, 5) rho_kernel(const double *__restrict__ B, const double *__restrict__ D,
-                                                     int naux, int nao, double *__restrict__ rho,
-                                                     const uint32_t *__restrict__ mask_mu, int *__restrict__ work) {
+// rho in the row-by-row order of a B with zero chunks, one CTA per P; rho2
+// (optional): a second copy.
+template <bool kPacked>
+__global__ void __launch_bounds__(256) rho_rows_kernel(const double *__restrict__ B, const double *__restrict__ D,
+                                                       int nao, double *__restrict__ rho, double *__restrict__ rho2,
+                                                       const uint32_t *__restrict__ mask_mu) {
   __shared__ double red[8];
-  __shared__ int slot;
-  if (!work) {
-    if (kRows)
-      rho_one_rows<kPacked>(B, D, nao, rho, mask_mu, blockIdx.x, red);
-    else
-      rho_one<kPacked>(B, D, nao, rho, blockIdx.x, red);
-    return;
-  }
-  for (;;) {
-    const int P = take_item(work, &slot);
-    if (P >= naux) break;
-    if (kRows)
-      rho_one_rows<kPacked>(B, D, nao, rho, mask_mu, P, red);
-    else
-      rho_one<kPacked>(B, D, nao, rho, P, red);
+  rho_one_rows<kPacked>(B, D, nao, rho, rho2, mask_mu, blockIdx.x, red);
+}
+
+// rho in row-pair order, one CTA per P: its 8 warps are the 8 parts.
+template <bool kPacked>
+__global__ void __launch_bounds__(256, 4) rho_kernel(const double *__restrict__ B, const double *__restrict__ D,
+                                                     int naux, int nao, double *__restrict__ rho,
+                                                     double *__restrict__ rho2) {
+  __shared__ double part[8];
+  double v[1];
+  rho_part<kPacked, 1, 8>(B, D, naux, nao, blockIdx.x, threadIdx.x >> 5, v);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v[0];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += part[w];
+    rho[blockIdx.x] = t;
+    if (rho2) rho2[blockIdx.x] = t;
   }
 }
 
 // J_mn = sum_P B_Pmn rho_P over the upper triangle, written to both halves.
-// Item (x, y) takes elements x*256 .. of the row pair (y, nao-1-y): row y from
-// column y, then row nao-1-y from its diagonal (nao + 1 elements per pair, one
-// row alone in the middle when nao is odd), so every item has the same work.
-// Each element's sum runs over P in ascending order, one FMA per P, with
-// eight loads of B ahead of their FMAs.
-template <bool kPacked>
-__device__ __forceinline__ void coulomb_one(const double *__restrict__ B, const double *srho, int naux, int nao,
-                                            double *__restrict__ J, const uint32_t *__restrict__ mask_mu, int x,
-                                            int y) {
-  const int m0 = y, m1 = nao - 1 - m0;
-  const int len0 = nao - m0, len1 = m1 > m0 ? nao - m1 : 0;
-  const int e = x * blockDim.x + threadIdx.x;
-  if (e >= len0 + len1) return;
-  const int mu = e < len0 ? m0 : m1;
-  const int nu = e < len0 ? m0 + e : m1 + (e - len0);
-  const long long off = kPacked ? packed_row(mu, nao) + (nu - mu) : (long long)mu * nao + nu;
-  const long long stride = kPacked ? (long long)nao * (nao + 1) / 2 : (long long)nao * nao;
-  const long long jmn = (long long)mu * nao + nu;
-  if (mask_mu && !((__ldg(mask_mu + mu) >> (nu >> 6)) & 1u)) {
-    // a screened pair: B_P mu nu = 0 for every P
-    J[jmn] = 0.0;
-    J[(long long)nu * nao + mu] = 0.0;
-    return;
-  }
-  const double *bp = B + off;
-  double acc = 0.0;
-  int P = 0;
-  for (; P + 8 <= naux; P += 8) {
-    double b[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) b[q] = __ldg(bp + (P + q) * stride);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) acc = fma(b[q], srho[P + q], acc);
-  }
-  for (; P < naux; ++P) acc = fma(__ldg(bp + P * stride), srho[P], acc);
-  J[jmn] = acc;
-  J[(long long)nu * nao + mu] = acc;
-}
-
-// Grid (gx, gy) of items (work == null), or a short grid taking item
-// x + gx y from the counter.  At most 48 registers, so that a short grid of a
-// few CTAs per SM leaves room for the X split's CTAs.
+// CTA (x, y) takes elements x*256 .. of the row pair (y, nao-1-y), so every CTA
+// has the same work.  Each element's sum runs over P in ascending order, one FMA
+// per P, with eight loads of B ahead of their FMAs.
 template <bool kPacked>
 __global__ void __launch_bounds__(256, 5) coulomb_kernel(const double *__restrict__ B,
                                                          const double *__restrict__ rho, int naux, int nao,
                                                          double *__restrict__ J,
-                                                         const uint32_t *__restrict__ mask_mu,
-                                                         int *__restrict__ work, int gx, int nitems) {
+                                                         const uint32_t *__restrict__ mask_mu) {
   extern __shared__ double srho[];
-  __shared__ int slot;
   for (int i = threadIdx.x; i < naux; i += blockDim.x) srho[i] = rho[i];
   __syncthreads();
-  if (!work) {
-    coulomb_one<kPacked>(B, srho, naux, nao, J, mask_mu, blockIdx.x, blockIdx.y);
-    return;
+  int mu, nu;
+  if (!pair_element(nao, blockIdx.y, blockIdx.x * 256 + threadIdx.x, mu, nu)) return;
+  double acc = 0.0;  // a screened pair: B_P mu nu = 0 for every P
+  if (!mask_mu || ((__ldg(mask_mu + mu) >> (nu >> 6)) & 1u)) {
+    const long long off = kPacked ? packed_row(mu, nao) + (nu - mu) : (long long)mu * nao + nu;
+    const long long stride = kPacked ? (long long)nao * (nao + 1) / 2 : (long long)nao * nao;
+    acc = coulomb_sum<8>(B + off, stride, srho, naux);
   }
-  for (;;) {
-    const int it = take_item(work, &slot);
-    if (it >= nitems) break;
-    coulomb_one<kPacked>(B, srho, naux, nao, J, mask_mu, it % gx, it / gx);
-  }
+  J[(long long)mu * nao + nu] = acc;
+  J[(long long)nu * nao + mu] = acc;
 }
 
 // True in every thread of the last CTA of the grid to arrive here (each CTA's
@@ -460,26 +304,54 @@ cudaError_t launch_density_change(const double *D, double *Dprev, bool have_prev
   return cudaGetLastError();
 }
 
-cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, double *rho, cudaStream_t st,
-                       const uint32_t *mask_mu, bool packed, int *work, int grid, bool rows) {
-  const unsigned g = work ? (unsigned)grid : (unsigned)naux;
-  rows = rows || mask_mu;
-  if (packed) {
-    if (rows)
-      rho_kernel<true, true><<<g, 256, 0, st>>>(B, D, naux, nao, rho, mask_mu, work);
+CoulombWork rho_work(const double *B, const double *D, int naux, int nao, bool packed, double *part, int *work) {
+  CoulombWork w{};
+  w.kind = 1;
+  w.naux = naux;
+  w.nao = nao;
+  w.packed = packed;
+  // 912 spare warps (6 on each of 152 SMs): as many functions at once (one load
+  // of D serves the group) as leave every warp an item
+  w.group = naux >= 456 && nao <= 16384 ? 4 : 1;
+  w.nitems = 8 * ((naux + w.group - 1) / w.group);
+  w.B = B;
+  w.D = D;
+  w.part = part;
+  w.work = work;
+  return w;
+}
+
+CoulombWork coulomb_work_of(const double *B, const double *rho, int naux, int nao, bool packed, double *J, int *work) {
+  CoulombWork w{};
+  w.kind = 2;
+  w.naux = naux;
+  w.nao = nao;
+  w.packed = packed;
+  w.nitems = (nao + 1 + 31) / 32 * ((nao + 1) / 2);
+  w.B = B;
+  w.rho = rho;
+  w.J = J;
+  w.work = work;
+  return w;
+}
+
+cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, double *rho, double *rho2,
+                       cudaStream_t st, const uint32_t *mask_mu, bool packed, bool rows) {
+  if (rows || mask_mu) {
+    if (packed)
+      rho_rows_kernel<true><<<(unsigned)naux, 256, 0, st>>>(B, D, nao, rho, rho2, mask_mu);
     else
-      rho_kernel<true, false><<<g, 256, 0, st>>>(B, D, naux, nao, rho, nullptr, work);
+      rho_rows_kernel<false><<<(unsigned)naux, 256, 0, st>>>(B, D, nao, rho, rho2, mask_mu);
+  } else if (packed) {
+    rho_kernel<true><<<(unsigned)naux, 256, 0, st>>>(B, D, naux, nao, rho, rho2);
   } else {
-    if (rows)
-      rho_kernel<false, true><<<g, 256, 0, st>>>(B, D, naux, nao, rho, mask_mu, work);
-    else
-      rho_kernel<false, false><<<g, 256, 0, st>>>(B, D, naux, nao, rho, nullptr, work);
+    rho_kernel<false><<<(unsigned)naux, 256, 0, st>>>(B, D, naux, nao, rho, rho2);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_coulomb(const double *B, const double *rho, int naux, int nao, double *J, cudaStream_t st,
-                           const uint32_t *mask_mu, bool packed, int *work, int grid) {
+                           const uint32_t *mask_mu, bool packed) {
   const size_t sm = (size_t)naux * sizeof(double);
   static size_t attr = 48 * 1024;
   if (sm > attr) {
@@ -489,12 +361,11 @@ cudaError_t launch_coulomb(const double *B, const double *rho, int naux, int nao
     if (e != cudaSuccess) return e;
     attr = sm;
   }
-  const int gx = (nao + 1 + 255) / 256, gy = (nao + 1) / 2;
-  const dim3 g = work ? dim3((unsigned)grid) : dim3(gx, gy);
+  const dim3 g((nao + 1 + 255) / 256, (nao + 1) / 2);
   if (packed)
-    coulomb_kernel<true><<<g, 256, sm, st>>>(B, rho, naux, nao, J, mask_mu, work, gx, gx * gy);
+    coulomb_kernel<true><<<g, 256, sm, st>>>(B, rho, naux, nao, J, mask_mu);
   else
-    coulomb_kernel<false><<<g, 256, sm, st>>>(B, rho, naux, nao, J, mask_mu, work, gx, gx * gy);
+    coulomb_kernel<false><<<g, 256, sm, st>>>(B, rho, naux, nao, J, mask_mu);
   return cudaGetLastError();
 }
 

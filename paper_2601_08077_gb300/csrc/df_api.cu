@@ -225,7 +225,7 @@ long long xdigit_ld(int nocc) { return round_up((long long)kBlock * even_nocc(no
 namespace df {
 
 df_status k_front(df_ctx *c, const double *C, int nocc, const int *sb, int c_planes, cudaStream_t st,
-                  cudaEvent_t after_gemm1) {
+                  const CoulombWork *cw, const RhoParts &rp) {
   int smax = 0;
   for (int b = 0; b < c->nblk; ++b) {
     if (sb[b] < 1 || sb[b] > c->s_max) return record(c, DF_ERR_ARG);
@@ -240,8 +240,14 @@ df_status k_front(df_ctx *c, const double *C, int nocc, const int *sb, int c_pla
   const long long c_plane = (long long)c->nocc_max * c->ld_nao;
   {
     PhaseTimer t(c, DF_PHASE_SPLIT_C, st);
-    DF_TRY(c, df::launch_split_cols_bf16(C, nao, nocc, c_planes, c->eC, c->Cd, c->ld_nao, c_plane, st, c->rowE,
-                                         c->nblk * nao));
+    df::ColsExtra extra{};
+    extra.reset = c->rowE;
+    extra.nreset = c->nblk * nao;
+    if (cw) {
+      extra.zero = c->jk_work;
+      extra.nzero = 2;
+    }
+    DF_TRY(c, df::launch_split_cols_bf16(C, nao, nocc, c_planes, c->eC, c->Cd, c->ld_nao, c_plane, st, extra));
   }
   // 2. X = B C
   df::SgParams p;
@@ -249,9 +255,8 @@ df_status k_front(df_ctx *c, const double *C, int nocc, const int *sb, int c_pla
   if (!df::gemm1_setup(c, nocc, p, maps)) return record(c, DF_ERR_CUDA);
   {
     PhaseTimer t(c, DF_PHASE_GEMM1, st);
-    DF_TRY(c, df::launch_slice_gemm(p, maps, st));
+    DF_TRY(c, df::launch_slice_gemm(p, maps, st, cw));
   }
-  if (after_gemm1) DF_TRY(c, cudaEventRecord(after_gemm1, st));
   // 3. X -> per-(block, mu) digit planes
   const long long kb_ld = df::xdigit_ld(nocc);
   {
@@ -259,19 +264,19 @@ df_status k_front(df_ctx *c, const double *C, int nocc, const int *sb, int c_pla
     df::ShiftTable t1;
     for (int q = 0; q <= 8; ++q) t1.v[q] = p.shiftT[q];
     DF_TRY(c, df::launch_split_xblocks(reinterpret_cast<const long long *>(c->X), naux, nao, df::even_nocc(nocc), smax, c->eB,
-                                       c->eC, c->sblk, t1, c->rowE, c->eX, c->Xd, kb_ld, c->nblk, st));
+                                       c->eC, c->sblk, t1, c->rowE, c->eX, c->Xd, kb_ld, c->nblk, rp, st));
   }
   return DF_OK;
 }
 
-df_status k_back(df_ctx *c, int nocc, double *K, cudaStream_t st) {
+df_status k_back(df_ctx *c, int nocc, double *K, cudaStream_t st, const CoulombWork *cw) {
   // 4. per-block K_b on upper tiles (exact int64 partials per K split)
   df::SgParams q2;
   df::SgMaps maps;
   if (!df::gemm2_setup(c, nocc, c->nsplit, q2, maps)) return record(c, DF_ERR_CUDA);
   {
     PhaseTimer t(c, DF_PHASE_GEMM2, st);
-    DF_TRY(c, df::launch_slice_gemm(q2, maps, st));
+    DF_TRY(c, df::launch_slice_gemm(q2, maps, st, cw));
   }
   // 5. K = sum_b K_b
   {
@@ -404,6 +409,7 @@ df_status df_create(df_ctx **out, int nao, int naux, int nocc_max, int s_max) {
   if (e == cudaSuccess) e = alloc(c, &c->Rp, (size_t)c->nblk * c->nsplit * nao * nao);
   if (e == cudaSuccess) e = alloc(c, &c->rho, (size_t)naux);
   if (e == cudaSuccess) e = alloc(c, &c->jk_work, (size_t)2);
+  if (e == cudaSuccess) e = alloc(c, &c->rho_part, (size_t)8 * naux);
   if (e == cudaSuccess) e = alloc(c, &c->epart, (size_t)3 * 296);
   if (e == cudaSuccess) e = alloc(c, &c->E, (size_t)4);
   if (e == cudaSuccess) e = alloc(c, &c->sblk, (size_t)c->nblk);
@@ -444,9 +450,7 @@ void df_destroy(df_ctx *c) {
   cudaFree(c->Rp);
   cudaFree(c->rho);
   cudaFree(c->jk_work);
-  if (c->jk_stream) cudaStreamDestroy(c->jk_stream);
-  if (c->jk_fork) cudaEventDestroy(c->jk_fork);
-  if (c->jk_join) cudaEventDestroy(c->jk_join);
+  cudaFree(c->rho_part);
   cudaFree(c->epart);
   cudaFree(c->E);
   cudaFree(c->sblk);
@@ -582,7 +586,7 @@ df_status setup_common(df_ctx *c, const double *B_dev, const int *perm_host, boo
     DF_TRY(c, cudaMemcpyAsync(&h, c->status, sizeof(int), cudaMemcpyDeviceToHost, st));
     DF_TRY(c, cudaMemsetAsync(c->status, 0, sizeof(int), st));
   }
-  c->sparse = false;
+  c->sparse = c->rows = false;
   c->frac_ktiles = c->frac_chunks = 1.0;
   std::vector<uint32_t> mu(c->nao), tiles(ntiles);
   if (masks) {
@@ -604,6 +608,10 @@ df_status setup_common(df_ctx *c, const double *B_dev, const int *perm_host, boo
     c->frac_chunks = all ? (double)on / all : 1.0;
     c->frac_ktiles = (double)kon / ((double)ntiles * nk);
     c->sparse = on < all;
+    // rho and J skip chunks only where most are zero: the row order and the mask
+    // tests cost more than a few skipped chunks save (90-atom cube, 2 % zero: rho
+    // 502 us in row order, ~230 in row-pair order)
+    c->rows = 2 * on < all;
   }
   c->ready = true;
   return DF_OK;
@@ -626,34 +634,18 @@ df_status df_build_J(df_ctx *c, const double *D, double *J, double *rho, void *s
   double *r = rho ? rho : c->rho;
   {
     PhaseTimer t(c, DF_PHASE_RHO, st);
-    DF_TRY(c, df::launch_rho(c->B, D, c->naux, c->nao, r, st, df::use_mask_mu(c), c->packed, nullptr, 0, c->sparse));
+    DF_TRY(c, df::launch_rho(c->B, D, c->naux, c->nao, r, r == c->rho ? nullptr : c->rho, st, df::use_mask_mu(c),
+                             c->packed, c->rows));
   }
   {
     PhaseTimer t(c, DF_PHASE_COULOMB, st);
     DF_TRY(c, df::launch_coulomb(c->B, r, c->naux, c->nao, J, st, df::use_mask_mu(c), c->packed));
   }
-  if (rho && rho != c->rho)
-    DF_TRY(c, cudaMemcpyAsync(c->rho, rho, sizeof(double) * c->naux, cudaMemcpyDeviceToDevice, st));
   // the density change since the last Coulomb build (an input of the learned slice counts)
   DF_TRY(c, df::launch_density_change(D, c->Dprev, c->have_Dprev, (long long)c->nao * c->nao, c->dD_part, c->tickets, c->dD, st));
   c->have_Dprev = true;
   return DF_OK;
 }
-
-namespace {
-
-// The internal stream and events of df_build_JK (created on first use).
-df_status jk_streams(df_ctx *c) {
-  if (c->jk_stream) return DF_OK;
-  int lo = 0, hi = 0;
-  DF_TRY(c, cudaDeviceGetStreamPriorityRange(&lo, &hi));
-  DF_TRY(c, cudaStreamCreateWithPriority(&c->jk_stream, cudaStreamNonBlocking, hi));
-  DF_TRY(c, cudaEventCreateWithFlags(&c->jk_fork, cudaEventDisableTiming));
-  DF_TRY(c, cudaEventCreateWithFlags(&c->jk_join, cudaEventDisableTiming));
-  return DF_OK;
-}
-
-}  // namespace
 
 df_status df_build_JK(df_ctx *c, const double *D, const double *C, int nocc, int nslices, double *J, double *rho,
                       double *K, df_kstats *stats, void *stream) {
@@ -666,43 +658,26 @@ df_status df_build_JK(df_ctx *c, const double *D, const double *C, int nocc, int
     s = df::level_count(c, level);
   }
   if (s > c->s_max) return record(c, DF_ERR_ARG);
-  // the native FP64 build, the learned counts, a block-sparse B (whose
-  // masked kernels take more registers than an SM shared with the X split
-  // leaves) and the no-overlap option run the two builds one after the other
-  if (c->jk_ctas == 0 || s == 0 || (nslices == -2 && c->level > 0) || df::use_mask_mu(c)) {
+  // the native FP64 build, the learned counts, a B of mostly zero chunks (its
+  // masked kernels) and the no-overlap option run the two builds one after the
+  // other
+  if (c->jk_ctas == 0 || s == 0 || (nslices == -2 && c->level > 0) || c->rows) {
     df_status r = df_build_J(c, D, J, rho, stream);
     return r == DF_OK ? df_build_K(c, C, nocc, nslices, K, stats, stream) : r;
   }
-  df_status r = jk_streams(c);
-  if (r != DF_OK) return r;
-  cudaStream_t st = as_stream(stream), side = c->jk_stream;
+  cudaStream_t st = as_stream(stream);
   int sb[4096];
   if (c->nblk > 4096) return record(c, DF_ERR_ARG);
   for (int b = 0; b < c->nblk; ++b) sb[b] = s;
-  // the exchange front (C split, first GEMM, X split) in the caller's stream;
-  // the Coulomb build forks after the first GEMM, whose persistent grid fills
-  // every SM, and runs beside the X split: rho and J are bound by the FP64
-  // pipe, the X split by HBM and integer work, so they share the SMs
-  r = df::k_front(c, C, nocc, sb, 0, st, c->jk_fork);
-  if (r != DF_OK) return r;
-  DF_TRY(c, cudaStreamWaitEvent(side, c->jk_fork, 0));
+  // rho and J stream B through the FP64 pipe, which the exchange GEMMs leave
+  // idle: their spare warps run rho beside the first GEMM and J beside the
+  // second
   double *rr = rho ? rho : c->rho;
-  const int grid = c->jk_ctas * (c->nsm > 0 ? c->nsm : 1);
-  DF_TRY(c, cudaMemsetAsync(c->jk_work, 0, 2 * sizeof(int), side));
-  {
-    PhaseTimer t(c, DF_PHASE_RHO, side);
-    DF_TRY(c, df::launch_rho(c->B, D, c->naux, c->nao, rr, side, nullptr, c->packed, c->jk_work, grid, c->sparse));
-  }
-  {
-    PhaseTimer t(c, DF_PHASE_COULOMB, side);
-    DF_TRY(c, df::launch_coulomb(c->B, rr, c->naux, c->nao, J, side, nullptr, c->packed, c->jk_work + 1, grid));
-  }
-  if (rho && rho != c->rho)
-    DF_TRY(c, cudaMemcpyAsync(c->rho, rho, sizeof(double) * c->naux, cudaMemcpyDeviceToDevice, side));
-  DF_TRY(c, cudaEventRecord(c->jk_join, side));
-  // the second GEMM's persistent grid waits for whole SMs: join first
-  DF_TRY(c, cudaStreamWaitEvent(st, c->jk_join, 0));
-  r = df::k_back(c, nocc, K, st);
+  const df::CoulombWork w1 = df::rho_work(c->B, D, c->naux, c->nao, c->packed, c->rho_part, c->jk_work);
+  const df::RhoParts rp{c->rho_part, rr, rr == c->rho ? nullptr : c->rho, c->naux};
+  const df::CoulombWork w2 = df::coulomb_work_of(c->B, rr, c->naux, c->nao, c->packed, J, c->jk_work + 1);
+  df_status r = df::k_front(c, C, nocc, sb, 0, st, &w1, rp);
+  if (r == DF_OK) r = df::k_back(c, nocc, K, st, &w2);
   if (r != DF_OK) return r;
   DF_TRY(c, df::launch_density_change(D, c->Dprev, c->have_Dprev, (long long)c->nao * c->nao, c->dD_part, c->tickets, c->dD, st));
   c->have_Dprev = true;

@@ -22,14 +22,12 @@ struct df_ctx {
   long long *Rp = nullptr;  // int64 partials of the second GEMM [nblk][nsplit][nao][nao]
   int nsplit = 1;
   double *rho = nullptr;
-  // df_build_JK: rho and J on a high-priority internal stream beside the X
-  // split, from short grids of jk_ctas CTAs per SM taking items from the two
-  // counters jk_work (0: everything in the caller's stream, in order)
+  // df_build_JK: rho and J by the spare warps of the two exchange GEMMs, their
+  // items from the two counters jk_work (jk_ctas 0: separate kernels, in order)
   int *jk_work = nullptr;
+  double *rho_part = nullptr;  // [8][naux]
   int jk_ctas = 4;
   int nsm = 0;
-  cudaStream_t jk_stream = nullptr;
-  cudaEvent_t jk_fork = nullptr, jk_join = nullptr;
   double *epart = nullptr;
   double *E = nullptr;
   int *sblk = nullptr;      // device per-block slice counts
@@ -42,6 +40,7 @@ struct df_ctx {
   uint32_t *mask_mu = nullptr;
   uint32_t *mask_tile = nullptr;
   bool sparse = false;
+  bool rows = false;  // most chunks are zero: rho in row order, and rho and J with the masks
   int sparse_opt = 1;        // DF_OPT_SPARSE: 0 never use the masks, 1 when some chunk is zero
   double frac_ktiles = 1.0;  // nonzero K tiles of the first GEMM's row tiles
   double frac_chunks = 1.0;  // nonzero (mu, 64-wide nu chunk) pairs of the upper triangle
@@ -90,16 +89,18 @@ bool gemm2_setup(df_ctx *c, int nocc, int nsplit, SgParams &q2, SgMaps &m);
 inline int even_nocc(int nocc) { return nocc + (nocc & 1); }
 long long xdigit_ld(int nocc);
 // The sparsity masks to use (null: run dense).
-inline const uint32_t *use_mask_mu(const df_ctx *c) { return c->sparse && c->sparse_opt ? c->mask_mu : nullptr; }
+inline const uint32_t *use_mask_mu(const df_ctx *c) { return c->rows && c->sparse_opt ? c->mask_mu : nullptr; }
 inline const uint32_t *use_mask_tile(const df_ctx *c) { return c->sparse && c->sparse_opt ? c->mask_tile : nullptr; }
 // The two halves of an emulated exchange build with per-block counts sb:
 // the front uploads sb, splits C into c_planes digit planes (>= max sb), runs
 // the first GEMM and the X split; the back runs the second GEMM and the
 // reduce into K.  Both asynchronous on st.
-// after_gemm1 (optional): an event recorded in st right after the first GEMM.
+// cw (optional): a Coulomb pass run beside the half's GEMM (rho beside the
+// first, whose counter and J's the front zeroes and whose parts the X split adds
+// as rp says; J beside the second).
 df_status k_front(df_ctx *c, const double *C, int nocc, const int *sb, int c_planes, cudaStream_t st,
-                  cudaEvent_t after_gemm1 = nullptr);
-df_status k_back(df_ctx *c, int nocc, double *K, cudaStream_t st);
+                  const CoulombWork *cw = nullptr, const RhoParts &rp = RhoParts{});
+df_status k_back(df_ctx *c, int nocc, double *K, cudaStream_t st, const CoulombWork *cw = nullptr);
 // The slice count run at a Table 1 level under the context's controller
 // settings (0 = native FP64).
 int level_count(const df_ctx *c, int level);

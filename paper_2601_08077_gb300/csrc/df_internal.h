@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/df.h"
+#include "coulomb_dev.cuh"
 #include "df_device.cuh"
 
 namespace df {
@@ -151,9 +152,17 @@ cudaError_t launch_setup_rows(const double *B, int naux, int nao, int nslices, i
                               cudaStream_t st);
 cudaError_t launch_split_rows_int8(const double *A, int rows, int cols, int ld, int nslices, int *exps,
                                    int8_t *digits, cudaStream_t st);
+// What the C split does on the way for the kernels after it: `reset` words set to
+// kRowBoundNone, `zero` words set to 0.
+struct ColsExtra {
+  int *reset;
+  int nreset;
+  int *zero;
+  int nzero;
+};
 cudaError_t launch_split_cols_bf16(const double *C, int nrows, int ncols, int nslices, int *exps,
                                    uint16_t *digits, long long dld, long long plane_stride, cudaStream_t st,
-                                   int *reset = nullptr, int nreset = 0);
+                                   const ColsExtra &extra);
 struct ShiftTable {
   int v[9];
 };
@@ -161,10 +170,10 @@ struct ShiftTable {
 // with a zero orbital); X = fl64(R 2^k) is formed here with
 // the first GEMM's exponents eB (rows (P, mu)), eC (orbitals), slices s_blk and
 // truncation table T1, then split per (block, mu).  rowE: the first GEMM's
-// per-row bound (SgParams::rowE).
+// per-row bound (SgParams::rowE).  rp: parts of rho to add on the way (part null: none).
 cudaError_t launch_split_xblocks(const long long *R, int naux, int nao, int nocc, int nslices, const int *eB,
                                  const int *eC, const int *s_blk, const ShiftTable &T1, const int *rowE, int *eX,
-                                 uint16_t *Xd, long long kb_ld, int nblk, cudaStream_t st);
+                                 uint16_t *Xd, long long kb_ld, int nblk, const RhoParts &rp, cudaStream_t st);
 cudaError_t launch_kpart_reduce(const long long *Rp, const int *eX, const int *s_blk, ShiftTable T, int nao,
                                 int nblk, int nsplit, double *K, cudaStream_t st);
 
@@ -172,7 +181,8 @@ cudaError_t launch_kpart_reduce(const long long *Rp, const int *eX, const int *s
 bool make_tmap_bf16(CUtensorMap *map, const void *base, long long k, long long rows, long long planes,
                     long long row_stride_elems, long long plane_stride_elems, int box_rows);
 
-cudaError_t launch_slice_gemm(const SgParams &p, const SgMaps &m, cudaStream_t st);
+// cw (optional, the two exchange GEMMs): a Coulomb pass for the spare warps.
+cudaError_t launch_slice_gemm(const SgParams &p, const SgMaps &m, cudaStream_t st, const CoulombWork *cw = nullptr);
 // Grouped launch; `mode` is shared by all problems, `grid` CTAs (0 = one per SM).
 // pairs: CTA-pair launch over tile pairs (kModeX only; unit_off and total
 // count tile pairs, every problem's npairs set).
@@ -185,21 +195,21 @@ int slice_gemm_grid(int nunits);
 cudaError_t launch_wait_selftest(int *status, unsigned long long limit_ns, cudaStream_t st);
 int fixed_point_shift(int s, long long k);
 
+// rho_P for every P into rho (and rho2 if given), J from rho.
 // mask_mu (optional, block-sparse B): per mu, bit c set when some B_P mu nu
 // with nu in [64c, 64c + 64) is nonzero; null = dense.
 // packed: B holds per P the upper triangle row by row ([naux][nao (nao + 1) / 2]).
-// work (optional): a zeroed item counter; then `grid` CTAs take the items from
-// it (a short grid sharing the SMs with a concurrent kernel), else one CTA
-// per item.  Either way every rho_P and J_mn is summed in the same order.
-// rows: rho in the row-by-row order of a B with zero chunks (taken whenever
+// rows: rho in the row-by-row order of a B with many zero chunks (taken whenever
 // mask_mu is given), else in row-pair order; the order is the B's, so a
 // screened B gives the same bits with and without its masks.
-cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, double *rho, cudaStream_t st,
-                       const uint32_t *mask_mu = nullptr, bool packed = false, int *work = nullptr, int grid = 0,
-                       bool rows = false);
+cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, double *rho, double *rho2,
+                       cudaStream_t st, const uint32_t *mask_mu, bool packed, bool rows);
 cudaError_t launch_coulomb(const double *B, const double *rho, int naux, int nao, double *J, cudaStream_t st,
-                           const uint32_t *mask_mu = nullptr, bool packed = false, int *work = nullptr,
-                           int grid = 0);
+                           const uint32_t *mask_mu, bool packed);
+// The same passes as work for a slice GEMM's spare warps (row-pair order, no
+// masks): `work` is zeroed before the launch, part holds 8 naux doubles.
+CoulombWork rho_work(const double *B, const double *D, int naux, int nao, bool packed, double *part, int *work);
+CoulombWork coulomb_work_of(const double *B, const double *rho, int naux, int nao, bool packed, double *J, int *work);
 // The masks of a packed B (pair flags through stream-ordered scratch of nao (nao + 1) / 2 bytes).
 cudaError_t launch_pair_masks_packed(const double *Bp, int naux, int nao, uint32_t *mask_mu, cudaStream_t st);
 // Dense B_P, P = P0 .. P0 + nP - 1, into out [nP][nao][nao] from a packed B.

@@ -82,6 +82,7 @@ constexpr int kStageBytes = 3 * kTileBytes;           // A_t tile + up to 256 st
 constexpr int kStagesP = 6;
 constexpr int kStageBytesP = 2 * kTileBytes;
 constexpr int kThreads = 384;                         // 12 warps
+constexpr int kThreadsHelp = 512;                     // and 4 more spare warps for a Coulomb pass
 constexpr int kEpiWarp0 = 4;
 constexpr int kEpiWarps = 8;
 constexpr int kAccBufs = 2;
@@ -126,6 +127,10 @@ static_assert(smem_bytes(kModeX, true) <= 232448 && smem_bytes(kModeX, false) <=
 constexpr int kRegsLow = 64;
 constexpr int kRegsHigh = 216;
 static_assert(128 * kRegsLow + 256 * kRegsHigh <= kThreads * 168, "register split exceeds the launch's registers");
+// With the Coulomb warps: 256*56 + 256*200 = 65536 = 512 threads * 128 registers.
+constexpr int kRegsLowH = 56;
+constexpr int kRegsHighH = 200;
+static_assert(256 * kRegsLowH + 256 * kRegsHighH <= kThreadsHelp * 128, "register split exceeds the launch's registers");
 
 // Instruction descriptor of tcgen05.mma .kind::f16, BF16 x BF16 -> FP32, both
 // operands K-major (D fmt bits 4-5, A fmt 7-9, B fmt 10-12, N>>3 at 17-22,
@@ -826,11 +831,17 @@ __device__ __forceinline__ const SgParams &unit_params(const SgParams &p, const 
   return g.params[lo];
 }
 
-template <int kMode, bool kGrouped, bool kPair>
-__global__ void __launch_bounds__(kThreads, 1)
+// kHelp: 512 threads, with warps 2, 3 and 12-15 running the Coulomb pass cw (rho
+// beside the first exchange GEMM, J beside the second).  The GEMMs leave the
+// FP64 pipe and, but for the first one at few orbitals, most of the DRAM rate
+// idle; the passes are bound by both, and run on their own or beside the X split
+// they were a quarter of a step.
+template <int kMode, bool kGrouped, bool kPair, bool kHelp>
+__global__ void __launch_bounds__(kHelp ? kThreadsHelp : kThreads, 1)
     slice_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                       const __grid_constant__ CUtensorMap tmap_h, const __grid_constant__ CUtensorMap tmap_x, const SgParams p,
-                      const SgGroup grp) {
+                      const SgGroup grp, const CoulombWork cw) {
+  constexpr int kRLow = kHelp ? kRegsLowH : kRegsLow, kRHigh = kHelp ? kRegsHighH : kRegsHigh;
   constexpr int NS = ring_stages(kMode, kPair);
   constexpr int SB = stage_bytes(kMode, kPair);
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -890,7 +901,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLow));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRLow));
     const bool lead = elect_one();
     uint32_t it = 0, st = 0, ph = 1;  // stages filled so far, ring position and the parity of its empty barrier
     bool ok = true, ready = false;
@@ -1001,7 +1012,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLow));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRLow));
     // pair, rank 1: rank 0's warp issues the MMAs of both CTAs
     if (!kPair || crank == 0) {
     // ------------------------------------------------------------ MMA issuer
@@ -1095,11 +1106,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
     }
-  } else if (warp < kEpiWarp0) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLow));
+  } else if (warp < kEpiWarp0 || warp >= kEpiWarp0 + kEpiWarps) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRLow));
+    if constexpr (kHelp) coulomb_work<kMode == kModeX ? 1 : 2>(cw);
   } else {
     // ------------------------------------------------------------ epilogue
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsHigh));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRHigh));
     const int quad = warp & 3;
     const int half = (warp - kEpiWarp0) >> 2;
     const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
@@ -1229,6 +1241,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (kMode == kModeX && lane == 0) tma_store_wait_all();
     __syncwarp();
+    // out of tiles: help with what is left of the Coulomb pass
+    if constexpr (kHelp) coulomb_work<kMode == kModeX ? 1 : 2>(cw);
   }
 
   tc_fence_before();
@@ -1364,26 +1378,29 @@ int slice_gemm_grid(int nunits) {
   return nunits < nsm ? nunits : nsm;
 }
 
-template <int kMode, bool kGrouped>
-cudaError_t launch_mode(const SgParams &p, const SgMaps &m, const SgGroup &g, int grid, cudaStream_t st) {
+template <int kMode, bool kGrouped, bool kHelp = false>
+cudaError_t launch_mode(const SgParams &p, const SgMaps &m, const SgGroup &g, int grid, cudaStream_t st,
+                        const CoulombWork &cw = CoulombWork{}) {
   constexpr int smem = smem_bytes(kMode, false);
+  auto kern = slice_gemm_kernel<kMode, kGrouped, false, kHelp>;
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(slice_gemm_kernel<kMode, kGrouped, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  slice_gemm_kernel<kMode, kGrouped, false><<<grid, kThreads, smem, st>>>(m.a, m.b, m.h, m.x, p, g);
+  kern<<<grid, kHelp ? kThreadsHelp : kThreads, smem, st>>>(m.a, m.b, m.h, m.x, p, g, cw);
   return cudaGetLastError();
 }
 
-// CTA-pair launch: clusters of two CTAs, as many clusters as fit at once
-// (at most one per tile pair), persistent over the tile pairs; grouped: the
-// tile pairs of several problems (g.total pairs, prefix table in pairs).
-template <int kMode, bool kGrouped = false>
-cudaError_t launch_pair(const SgParams &p, const SgMaps &m, cudaStream_t st, const SgGroup *grp = nullptr) {
-  auto kern = slice_gemm_kernel<kMode, kGrouped, true>;
+// CTA-pair launch: clusters of two CTAs, as many clusters as fit at once (at
+// most one per tile pair, unless a Coulomb pass wants every SM), persistent over
+// the tile pairs; grouped: the tile pairs of several problems (g.total pairs,
+// prefix table in pairs).
+template <int kMode, bool kGrouped = false, bool kHelp = false>
+cudaError_t launch_pair(const SgParams &p, const SgMaps &m, cudaStream_t st, const SgGroup *grp = nullptr,
+                        const CoulombWork &cw = CoulombWork{}) {
+  auto kern = slice_gemm_kernel<kMode, kGrouped, true, kHelp>;
   constexpr int smem = smem_bytes(kMode, true);
   static int max_clusters = 0;
   cudaLaunchConfig_t cfg;
@@ -1393,7 +1410,7 @@ cudaError_t launch_pair(const SgParams &p, const SgMaps &m, cudaStream_t st, con
   at[0].val.clusterDim.x = 2;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
-  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.blockDim = dim3(kHelp ? kThreadsHelp : kThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = at;
@@ -1410,12 +1427,12 @@ cudaError_t launch_pair(const SgParams &p, const SgMaps &m, cudaStream_t st, con
     max_clusters = n > 0 ? n : 1;
   }
   const int np = kGrouped ? grp->total : p.npairs;
-  const int nc = np < max_clusters ? np : max_clusters;
+  const int nc = np < max_clusters && !kHelp ? np : max_clusters;
   cfg.gridDim = dim3(2 * (unsigned)nc, 1, 1);
   SgGroup g;
   std::memset(&g, 0, sizeof(g));
   if (kGrouped) g = *grp;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, m.a, m.b, m.h, m.x, p, g);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, m.a, m.b, m.h, m.x, p, g, cw);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -1456,19 +1473,28 @@ static bool use_pairs(const SgParams &p) {
   return p.mode == kModeX || (p.mode == kModeKPart && (p.pair == 2 || p.nt_m >= 7));
 }
 
-cudaError_t launch_slice_gemm(const SgParams &p, const SgMaps &m, cudaStream_t st) {
+cudaError_t launch_slice_gemm(const SgParams &p, const SgMaps &m, cudaStream_t st, const CoulombWork *cw) {
   if (p.nunits <= 0) return cudaSuccess;
+  const bool help = cw && cw->kind && (p.mode == kModeX || p.mode == kModeKPart);
   if (use_pairs(p)) {
     const long long np = slice_gemm_pairs(p);
     if (np <= 0 || np > (1ll << 30)) return cudaErrorInvalidValue;
     SgParams q = p;
     q.npairs = (int)np;
-    if (p.mode == kModeX) return launch_pair<kModeX>(q, m, st);
     if (p.mode == kModeGemm) return launch_pair<kModeGemm>(q, m, st);
+    if (help)
+      return p.mode == kModeX ? launch_pair<kModeX, false, true>(q, m, st, nullptr, *cw)
+                              : launch_pair<kModeKPart, false, true>(q, m, st, nullptr, *cw);
+    if (p.mode == kModeX) return launch_pair<kModeX>(q, m, st);
     return launch_pair<kModeKPart>(q, m, st);
   }
   SgGroup g;
   std::memset(&g, 0, sizeof(g));
+  if (help) {
+    const int all = slice_gemm_grid(1 << 30);
+    return p.mode == kModeX ? launch_mode<kModeX, false, true>(p, m, g, all, st, *cw)
+                            : launch_mode<kModeKPart, false, true>(p, m, g, all, st, *cw);
+  }
   const int grid = slice_gemm_grid(p.nunits);
   switch (p.mode) {
     case kModeX: return launch_mode<kModeX, false>(p, m, g, grid, st);

@@ -272,16 +272,17 @@ __global__ void split_rows_int8_kernel(const double *__restrict__ A, int rows, i
 // values stay in registers between the maximum and the digits (up to 8 per
 // thread, 512 rows; further rows are read again).  A warp per column walked them
 // in two dependent passes (250 columns of 1200: 29 us).
-// reset (optional): nreset words set to kRowBoundNone on the way, the row bounds
-// that the first exchange GEMM is about to raise.
+// extra: words that the launches after it want set, the row bounds that the first
+// exchange GEMM raises and the counters of the Coulomb passes.
 constexpr int kColsT = 512;
 constexpr int kColsHeld = 8;
 __global__ void __launch_bounds__(kColsT) split_cols_bf16_kernel(const double *__restrict__ C, int nrows, int ncols,
                                                                  int nslices, int *__restrict__ exps,
                                                                  uint16_t *__restrict__ digits, long long dld,
-                                                                 long long plane_stride, int *__restrict__ reset,
-                                                                 int nreset) {
-  for (int i = blockIdx.x * kColsT + threadIdx.x; i < nreset; i += gridDim.x * kColsT) reset[i] = kRowBoundNone;
+                                                                 long long plane_stride, ColsExtra extra) {
+  const int me = blockIdx.x * kColsT + threadIdx.x, all = gridDim.x * kColsT;
+  for (int i = me; i < extra.nreset; i += all) extra.reset[i] = kRowBoundNone;
+  for (int i = me; i < extra.nzero; i += all) extra.zero[i] = 0;
   const int c = blockIdx.x * 8 + (threadIdx.x & 7);
   const int r0 = threadIdx.x >> 3;
   constexpr int step = kColsT / 8;
@@ -459,7 +460,8 @@ template <int S, bool kRound>
 __global__ void __launch_bounds__(kSplitXThreads, 5)
     split_xblocks_kernel(const long long *__restrict__ R, int naux, int nao, int nocc, XScale xs,
                          const int *__restrict__ rowE, int *__restrict__ eX, uint16_t *__restrict__ Xd,
-                         long long kb_ld, int nblk) {
+                         long long kb_ld, int nblk, RhoParts rp) {
+  if (rp.part && blockIdx.y == 0) rho_from_parts(rp, blockIdx.x * kSplitXThreads + threadIdx.x, gridDim.x * kSplitXThreads);
   extern __shared__ int sh_e[];  // [kBlock] (P, mu) exponents + base, then [nocc] orbital exponents
   __shared__ int sh_top, sh_lost;
   const int mu = blockIdx.x;
@@ -652,17 +654,19 @@ cudaError_t launch_split_rows_int8(const double *A, int rows, int cols, int ld, 
 
 cudaError_t launch_split_cols_bf16(const double *C, int nrows, int ncols, int nslices, int *exps,
                                    uint16_t *digits, long long dld, long long plane_stride, cudaStream_t st,
-                                   int *reset, int nreset) {
+                                   const ColsExtra &extra) {
   if (ncols <= 0) return cudaSuccess;
   split_cols_bf16_kernel<<<(ncols + 7) / 8, kColsT, 0, st>>>(C, nrows, ncols, nslices, exps, digits, dld,
-                                                             plane_stride, reset, nreset);
+                                                             plane_stride, extra);
   return cudaGetLastError();
 }
 
 cudaError_t launch_split_xblocks(const long long *R, int naux, int nao, int nocc, int nslices, const int *eB,
                                  const int *eC, const int *s_blk, const ShiftTable &T1, const int *rowE,
-                                 int *eX, uint16_t *Xd, long long kb_ld, int nblk, cudaStream_t st) {
-  using Kern = void (*)(const long long *, int, int, int, XScale, const int *, int *, uint16_t *, long long, int);
+                                 int *eX, uint16_t *Xd, long long kb_ld, int nblk, const RhoParts &rp,
+                                 cudaStream_t st) {
+  using Kern = void (*)(const long long *, int, int, int, XScale, const int *, int *, uint16_t *, long long, int,
+                        RhoParts);
   // up to 4 slices a sum of nao products has at most 53 bits (2^(8(s-1) + 14) nao (1 + 2/256 + ...)) for
   // nao <= 2^14
   static const Kern exact[4] = {split_xblocks_kernel<1, false>, split_xblocks_kernel<2, false>,
@@ -680,7 +684,7 @@ cudaError_t launch_split_xblocks(const long long *R, int naux, int nao, int nocc
   }
   XScale xs{eB, eC, s_blk, T1};
   dim3 grid(nao, nblk);
-  kern<<<grid, kSplitXThreads, sm, st>>>(R, naux, nao, nocc, xs, rowE, eX, Xd, kb_ld, nblk);
+  kern<<<grid, kSplitXThreads, sm, st>>>(R, naux, nao, nocc, xs, rowE, eX, Xd, kb_ld, nblk, rp);
   return cudaGetLastError();
 }
 

@@ -324,7 +324,7 @@ class Context:
         return K, st
 
     def build_JK(self, D, C, nslices: int, J=None, rho=None, K=None, stream=None):
-        """build_J(D) then build_K(C, nslices) in one call (rho and J beside the X split); (J, rho, K, stats)."""
+        """build_J(D) then build_K(C, nslices) in one call (rho and J beside the exchange GEMMs); (J, rho, K, stats)."""
         nocc = C.shape[1]
         if J is None:
             J = torch.empty((self.nao, self.nao), dtype=torch.float64, device=D.device)
@@ -377,7 +377,7 @@ class Context:
         _check(lib().df_set_option(self._h, OPT_SPARSE, 1 if on else 0), "df_set_option")
 
     def set_jk_overlap(self, ctas_per_sm: int):
-        """DF_OPT_JK_OVERLAP: CTAs per SM of rho and J beside the X split in build_JK (0 = in order)."""
+        """DF_OPT_JK_OVERLAP: rho and J beside the exchange GEMMs in build_JK (1..4 alike; 0 = in order)."""
         _check(lib().df_set_option(self._h, OPT_JK_OVERLAP, int(ctas_per_sm)), "df_set_option")
 
     def phase_times(self):

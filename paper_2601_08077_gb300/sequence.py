@@ -5,7 +5,7 @@ whose density differs from the converged D* by 0.1 10^-k (Frobenius).  The
 library's controller (df_adaptive_next: Table 1, monotone, iterations 0 and 1
 at level 4) picks each iteration's level from the relative change of the
 energy E_J + E_K; J and K of an iteration come from one df_build_JK call
-(rho and J beside the X split), at that level's count (mode "rule", ADAPTIVE), with per-block counts from the attached network
+(rho and J beside the exchange GEMMs), at that level's count (mode "rule", ADAPTIVE), with per-block counts from the attached network
 (mode "learned", LEARNED: prediction, fallback, check and recompute all in
 the library), or in native FP64 (mode "fp64").  Optionally every iteration's
 K and energy are compared with the native-FP64 build of the same density
