@@ -488,15 +488,17 @@ df_status df_mlp_create(df_mlp **out) {
   if (!out) return DF_ERR_ARG;
   df_mlp *m = new (std::nothrow) df_mlp();
   if (!m) return DF_ERR_OOM;
-  cudaError_t e = cudaMalloc(&m->P, sizeof(float) * kNParams);
-  if (e == cudaSuccess) e = cudaMalloc(&m->G, sizeof(float) * kNParams);
-  if (e == cudaSuccess) e = cudaMalloc(&m->m1, sizeof(float) * kNParams);
-  if (e == cudaSuccess) e = cudaMalloc(&m->m2, sizeof(float) * kNParams);
-  if (e == cudaSuccess) e = cudaMalloc(&m->loss, sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&m->part, sizeof(float) * (size_t)kMaxParts * kPart);
-  if (e == cudaSuccess) e = cudaMemset(m->P, 0, sizeof(float) * kNParams);
-  if (e == cudaSuccess) e = cudaMemset(m->m1, 0, sizeof(float) * kNParams);
-  if (e == cudaSuccess) e = cudaMemset(m->m2, 0, sizeof(float) * kNParams);
+  // one allocation: P, the two moments, G, the loss, the partial gradients
+  const size_t np = (kNParams + 63) / 64 * 64;
+  cudaError_t e = cudaMalloc(&m->P, sizeof(float) * (4 * np + 64 + (size_t)kMaxParts * kPart));
+  if (e == cudaSuccess) {
+    m->m1 = m->P + np;
+    m->m2 = m->P + 2 * np;
+    m->G = m->P + 3 * np;
+    m->loss = m->P + 4 * np;
+    m->part = m->loss + 64;
+  }
+  if (e == cudaSuccess) e = cudaMemset(m->P, 0, sizeof(float) * 3 * np);
   if (e != cudaSuccess) {
     df_mlp_destroy(m);
     return DF_ERR_CUDA;
@@ -508,11 +510,6 @@ df_status df_mlp_create(df_mlp **out) {
 void df_mlp_destroy(df_mlp *m) {
   if (!m) return;
   cudaFree(m->P);
-  cudaFree(m->G);
-  cudaFree(m->m1);
-  cudaFree(m->m2);
-  cudaFree(m->loss);
-  cudaFree(m->part);
   delete m;
 }
 
