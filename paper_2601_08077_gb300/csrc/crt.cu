@@ -19,7 +19,7 @@
 // The residues come from the balanced base-256 digits of A' (the digits of the
 // slice scheme): A' = sum_j b_j 256^j with signed bytes b_j, so A' mod m is
 // congruent to two 4-way signed byte dot products (dp4a) with the centred
-// weights 256^j mod m, a sum below 2^17 that one Barrett step reduces.  The
+// weights 256^j mod m, a sum of at most 2^17 that FP32 reduces exactly.  The
 // reconstruction accumulates sum_i y_i W_i (W_i the CRT weights) in 32-bit
 // limbs, estimates the quotient by M in FP32 and finishes in 128-bit integers.
 // No FP64 instruction is used: GB300's FP64 pipe is narrow.
@@ -36,8 +36,8 @@ struct CrtTab {
   int n;                            // moduli
   int q1;                           // q - 1
   int mod[kCrtMaxModuli];
-  uint32_t magic[kCrtMaxModuli];    // ceil(2^32 / m)
-  int off17[kCrtMaxModuli];         // a multiple of m >= 2^17
+  float modf[kCrtMaxModuli];
+  float inv[kCrtMaxModuli];         // 1 / m
   int wlo[kCrtMaxModuli];           // centred 256^j mod m, j = 0..3, one signed byte each
   int whi[kCrtMaxModuli];           // j = 4..7
   uint32_t W[kCrtMaxModuli][4];     // CRT weights (M/m_i) ((M/m_i)^-1 mod m_i), 32-bit limbs
@@ -100,8 +100,8 @@ bool make_tab(long long K, int n, CrtTab *t) {
   for (int i = 0; i < n; ++i) M *= (u128)t->mod[i];
   for (int i = 0; i < n; ++i) {
     const int m = t->mod[i];
-    t->magic[i] = (uint32_t)(0xFFFFFFFFu / (uint32_t)m + 1u);
-    t->off17[i] = ((1 << 17) + m - 1) / m * m;
+    t->modf[i] = (float)m;
+    t->inv[i] = 1.0f / (float)m;
     int lo = 0, hi = 0, w = 1 % m;
     for (int j = 0; j < 8; ++j) {
       const int c = w > m / 2 ? w - m : w;  // centred, in [-128, 127]
@@ -125,9 +125,9 @@ bool make_tab(long long K, int n, CrtTab *t) {
     for (int k = 0; k < 4; ++k) t->W[i][k] = (uint32_t)(Wi >> (32 * k));
   }
   for (int k = 0; k < 4; ++k) t->M[k] = (uint32_t)(M >> (32 * k));
-  // scale the FP32 estimate of V = sum y_i W_i < 2^12 M so it stays below 2^100
+  // scale the FP32 estimate of V = sum y_i W_i < 2^14 M so it stays below 2^100
   const int bl = bitlen128(M);
-  const int sc = bl + 12 > 100 ? bl + 12 - 100 : 0;
+  const int sc = bl + 14 > 100 ? bl + 14 - 100 : 0;
   for (int k = 0; k < 4; ++k) {
     const int ex = 32 * k - sc;
     t->f[k] = (ex >= -126 && ex <= 127) ? std::ldexp(1.0f, ex) : 0.0f;
@@ -198,17 +198,22 @@ __device__ __forceinline__ long long scaled_rne_q(uint64_t bits, int e, int q1) 
   return (bits >> 63) ? -N : N;
 }
 
-// Centred residue of the integer whose balanced digit words are (hi, lo):
-// S = sum_j b_j (256^j mod m) has |S| <= 8 128^2 = 2^17; S + off17 >= 0 is
-// reduced by a Barrett step (the high word of v ceil(2^32 / m) is floor(v / m)
-// or one more).
-__device__ __forceinline__ int residue(int lo, int hi, const CrtTab &t, int i) {
-  const int S = __dp4a(lo, t.wlo[i], __dp4a(hi, t.whi[i], 0));
-  const int m = t.mod[i];
-  const uint32_t v = (uint32_t)(S + t.off17[i]);
-  int r = (int)(v - __umulhi(v, t.magic[i]) * (uint32_t)m);
-  if (r < 0) r += m;
-  return r > (m >> 1) ? r - m : r;
+// Centred residue, as an exact FP32 value, of the integer whose balanced digit
+// words are (hi, lo), for an odd modulus: S = sum_j b_j (256^j mod m) has |S| <=
+// 8 128^2 = 2^17, so the dot products started at the bits of 1.5 2^23 leave the
+// FP32 1.5 2^23 + S; S - m rint(S / m) is then exact (S / m stays 1 / (2 m) > 2e-3
+// away from a tie, its FP32 error is below 1e-4).  Six instructions where an
+// integer Barrett step, the centring and the conversion to BF16 took 14.
+__device__ __forceinline__ float residue_odd(int lo, int hi, const CrtTab &t, int i) {
+  const float S = __int_as_float(__dp4a(lo, t.wlo[i], __dp4a(hi, t.whi[i], 0x4B400000))) - 12582912.0f;
+  const float q = fmaf(S, t.inv[i], 12582912.0f) - 12582912.0f;
+  return fmaf(-q, t.modf[i], S);
+}
+
+// The same for the modulus 256: the low digit, with 128 for -128.
+__device__ __forceinline__ float residue_256(int lo) {
+  const int b = (int)(signed char)(lo & 0xFF);
+  return (float)(b == -128 ? 128 : b);
 }
 
 // TPR threads per row (a warp, or the whole block for wide rows): exponent,
@@ -222,10 +227,20 @@ __global__ void __launch_bounds__(256)
   const long long r = (long long)blockIdx.x * (blockDim.x / TPR) + (threadIdx.x / TPR);
   if (r >= rows) return;  // uniform over a row's threads
   const double *row = A + r * ld;
+  const bool vec2 = (reinterpret_cast<uintptr_t>(row) & 15) == 0;
   uint64_t mx = 0;
-  for (int c = lane; c < cols; c += TPR) {
-    const uint64_t a = abs_bits(__ldg(row + c));
-    mx = a > mx ? a : mx;
+  if (vec2) {
+    for (int c = 2 * lane; c < cols; c += 2 * TPR) {
+      const double2 v = c + 1 < cols ? __ldg(reinterpret_cast<const double2 *>(row + c)) : make_double2(__ldg(row + c), 0.0);
+      const uint64_t a = abs_bits(v.x), b = abs_bits(v.y);
+      mx = a > mx ? a : mx;
+      mx = b > mx ? b : mx;
+    }
+  } else {
+    for (int c = lane; c < cols; c += TPR) {
+      const uint64_t a = abs_bits(__ldg(row + c));
+      mx = a > mx ? a : mx;
+    }
   }
   mx = row_max_u64<TPR>(mx);
   const int e = exponent_from_max_bits_dev(mx);
@@ -235,42 +250,59 @@ __global__ void __launch_bounds__(256)
   for (int c = 4 * lane; c < cols; c += 4 * TPR) {
     const int nv = cols - c < 4 ? cols - c : 4;
     int lo[4], hi[4];
+    double x[4];
+    if (vec2 && nv == 4) {
+      const double2 u = __ldg(reinterpret_cast<const double2 *>(row + c));
+      const double2 v = __ldg(reinterpret_cast<const double2 *>(row + c) + 1);
+      x[0] = u.x, x[1] = u.y, x[2] = v.x, x[3] = v.y;
+    } else {
+      for (int h = 0; h < 4; ++h) x[h] = h < nv ? __ldg(row + c + h) : 0.0;
+    }
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      const uint64_t b = h < nv ? (uint64_t)__double_as_longlong(row[c + h]) : 0ull;
+      const uint64_t b = (uint64_t)__double_as_longlong(x[h]);
       // balanced digits: byte j of Mg is b_j + 128 for j < 7, the top byte is b_7
       const long long Mg = scaled_rne_q(b, e, t.q1) + 0x0080808080808080ll;
       lo[h] = (int)((uint32_t)Mg ^ 0x80808080u);
       hi[h] = (int)((uint32_t)((unsigned long long)Mg >> 32) ^ 0x00808080u);
     }
-    for (int i = 0; i < t.n; ++i) {
-      uint32_t v[4];
+    // unrolled, so that the table entries are constant operands: indexed constant
+    // loads were the kernel's limit (their unit 71% busy)
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const int rr = residue(lo[h], hi[h], t, i);
-        v[h] = kInspect ? (uint32_t)(uint16_t)(int16_t)rr : (uint32_t)int_to_bf16_bits(rr);
-      }
+    for (int i = 0; i < kCrtMaxModuli; ++i) {
+      if (i >= t.n) break;
+      float res[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) res[h] = i == 0 ? residue_256(lo[h]) : residue_odd(lo[h], hi[h], t, i);
       uint16_t *dst = drow + (long long)i * pstride + c;
-      if (nv == 4 && ((reinterpret_cast<uintptr_t>(dst) & 7) == 0)) {
-        *reinterpret_cast<uint2 *>(dst) = make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
+      if (kInspect) {
+        for (int h = 0; h < nv; ++h) dst[h] = (uint16_t)(int16_t)(int)res[h];
+      } else if (nv == 4 && ((reinterpret_cast<uintptr_t>(dst) & 7) == 0)) {
+        // BF16 of an exact small integer: its FP32's upper half
+        *reinterpret_cast<uint2 *>(dst) = make_uint2(__byte_perm(__float_as_uint(res[0]), __float_as_uint(res[1]), 0x7632u),
+                                                     __byte_perm(__float_as_uint(res[2]), __float_as_uint(res[3]), 0x7632u));
       } else {
-        for (int h = 0; h < nv; ++h) dst[h] = (uint16_t)v[h];
+        for (int h = 0; h < nv; ++h) dst[h] = (uint16_t)(__float_as_uint(res[h]) >> 16);
       }
     }
   }
 }
 
-// P' from the residue bytes of one element, then fl64(P' 2^k).
-__device__ __forceinline__ double crt_value(const uint8_t *y, long long plane, const CrtTab &t, int k) {
-  uint64_t a0 = 0, a1 = 0, a2 = 0, a3 = 0;  // V = sum_j a_j 2^(32j), each a_j < 2^44
-  for (int i = 0; i < t.n; ++i) {
-    const uint64_t v = y[i * plane];
+// P' from the residue bytes of one element (nsplit K parts per modulus, added
+// here: the sum is congruent, at most 255 kModSplitMax), then fl64(P' 2^k).
+__device__ __forceinline__ double crt_value(const uint8_t *y, long long plane, int nsplit, const CrtTab &t, int k) {
+  uint64_t a0 = 0, a1 = 0, a2 = 0, a3 = 0;  // V = sum_j a_j 2^(32j), each a_j < 2^46
+#pragma unroll
+  for (int i = 0; i < kCrtMaxModuli; ++i) {  // unrolled: the weights are constant operands
+    if (i >= t.n) break;
+    uint64_t v = 0;
+    for (int s = 0; s < nsplit; ++s, y += plane) v += *y;
     a0 += v * t.W[i][0];
     a1 += v * t.W[i][1];
     a2 += v * t.W[i][2];
     a3 += v * t.W[i][3];
   }
-  // V / M < 4096; the FP32 estimate is within 1/64 of it, so floor is off by at most 1
+  // V / M < 2^14; the FP32 estimate is within 1/64 of it, so floor is off by at most 1
   const float vf = (float)a0 * t.f[0] + (float)a1 * t.f[1] + (float)a2 * t.f[2] + (float)a3 * t.f[3];
   const long long qe = (long long)__float2int_rd(vf * t.invM);
   // R = V - qe M in 128-bit two's complement (it lies in (-M, 2M))
@@ -299,14 +331,41 @@ __device__ __forceinline__ double crt_value(const uint8_t *y, long long plane, c
 }
 
 __global__ void __launch_bounds__(256)
-    crt_reconstruct_kernel(const uint8_t *__restrict__ Y, int M, int N, long long ldy, long long plane,
+    crt_reconstruct_kernel(const uint8_t *__restrict__ Y, int M, int N, long long ldy, long long plane, int nsplit,
                            const int *__restrict__ ea, const int *__restrict__ eb, const CrtTab t,
                            double *__restrict__ out, long long ldo) {
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
   const int ebn = eb[n];
   for (int m = blockIdx.y; m < M; m += gridDim.y)
-    out[(long long)m * ldo + n] = crt_value(Y + (long long)m * ldy + n, plane, t, ea[m] + ebn - 2 * t.q1);
+    out[(long long)m * ldo + n] = crt_value(Y + (long long)m * ldy + n, plane, nsplit, t, ea[m] + ebn - 2 * t.q1);
+}
+
+// The same for a Gram matrix, whose residues exist in the 128-wide tiles (i, j >= i):
+// a CTA takes 8 rows m0 .. of the columns n0 .. n0 + 31 >= m0 and writes them and
+// their transpose (64-byte pieces); a value is a chain of a few hundred integer
+// instructions, so the tile is one value per thread.
+__global__ void __launch_bounds__(256)
+    crt_reconstruct_sym_kernel(const uint8_t *__restrict__ Y, int N, long long ldy, long long plane, int nsplit,
+                               const int *__restrict__ ea, const CrtTab t, double *__restrict__ out, long long ldo) {
+  __shared__ double tile[32][9];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n0 = blockIdx.x * 32, n = n0 + lane;
+  const int en = n < N ? ea[n] : 0;
+  const int last = min(N, n0 + 32);
+  for (int m0 = blockIdx.y * 8; m0 < last; m0 += gridDim.y * 8) {
+    const int m = m0 + warp;
+    if (m < N && n < N) {
+      const double v = crt_value(Y + (long long)m * ldy + n, plane, nsplit, t, ea[m] + en - 2 * t.q1);
+      out[(long long)m * ldo + n] = v;
+      tile[lane][warp] = v;
+    }
+    if (m0 >= n0) continue;  // beside the diagonal both triangles are computed; m0 only grows
+    __syncthreads();
+    const int r = threadIdx.x >> 3, c = threadIdx.x & 7;  // m0 + c < n0 <= N - 1
+    if (n0 + r < N) out[(long long)(n0 + r) * ldo + m0 + c] = tile[r][c];
+    __syncthreads();
+  }
 }
 
 cudaError_t launch_crt_split(const double *A, long long rows, int cols, long long ld, const CrtTab &t, int *exps,
@@ -348,7 +407,12 @@ df_status crt_gemm(const double *A, const double *B, int M, int N, int K, int nm
   df_status rs = DF_OK;
   cudaError_t e = scratch_malloc((void **)&Ad, sizeof(uint16_t) * (size_t)nmod * M * ld, st);
   if (e == cudaSuccess && !same) e = scratch_malloc((void **)&Bd, sizeof(uint16_t) * (size_t)nmod * N * ld, st);
-  if (e == cudaSuccess) e = scratch_malloc((void **)&Y, (size_t)nmod * M * ldy, st);
+  // partial residues and the upper tiles alone serve the reconstruction; the
+  // inspection entry point returns whole products
+  SgParams p;
+  grid_params(&p, kModeMod, M, N, K, 1);  // shiftT[1] = 0: the sums are exact
+  plan_mod_gemm(&p, nmod, same && out, out != nullptr);
+  if (e == cudaSuccess) e = scratch_malloc((void **)&Y, (size_t)nmod * p.nsplit * M * ldy, st);
   if (e == cudaSuccess) e = scratch_malloc((void **)&ea, sizeof(int) * M, st);
   if (e == cudaSuccess && !same) e = scratch_malloc((void **)&eb, sizeof(int) * N, st);
   if (e == cudaSuccess) e = scratch_malloc((void **)&status, sizeof(int), st);
@@ -364,9 +428,6 @@ df_status crt_gemm(const double *A, const double *B, int M, int N, int K, int nm
     if (!make_operand_maps(&maps, a, b, kTile)) {
       rs = DF_ERR_CUDA;
     } else {
-      SgParams p;
-      grid_params(&p, kModeMod, M, N, K, 1);  // shiftT[1] = 0: the sums are exact
-      p.nunits *= nmod;
       p.out = reinterpret_cast<double *>(Y);
       p.out_ld = ldy;
       p.out_blk = (long long)M * ldy;
@@ -377,8 +438,14 @@ df_status crt_gemm(const double *A, const double *B, int M, int N, int K, int nm
     }
   }
   if (e == cudaSuccess && rs == DF_OK && out) {
-    const dim3 grid((unsigned)((N + 255) / 256), (unsigned)(M < 65535 ? M : 65535));
-    crt_reconstruct_kernel<<<grid, 256, 0, st>>>(Y, M, N, ldy, (long long)M * ldy, ea, ebx, t, out, N);
+    if (same) {
+      const unsigned nm = (unsigned)((N + 7) / 8);
+      const dim3 grid((unsigned)((N + 31) / 32), nm < 65535 ? nm : 65535);
+      crt_reconstruct_sym_kernel<<<grid, 256, 0, st>>>(Y, N, ldy, (long long)M * ldy, p.nsplit, ea, t, out, N);
+    } else {
+      const dim3 grid((unsigned)((N + 255) / 256), (unsigned)(M < 65535 ? M : 65535));
+      crt_reconstruct_kernel<<<grid, 256, 0, st>>>(Y, M, N, ldy, (long long)M * ldy, p.nsplit, ea, ebx, t, out, N);
+    }
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && rs == DF_OK && Y_user)

@@ -49,7 +49,8 @@ struct SgParams {
   int q;                    // digits stacked in one MMA: min(8, 256 / nw)
   int s_fixed;              // slice count (kModeRaw, kModeGemm, kModeMod)
   int nao, nocc, nblk, naux;
-  int nsplit;               // K splits per block (kModeKPart)
+  int nsplit;               // K splits per block (kModeKPart) or plane (kModeMod)
+  int sym;                  // kModeMod: A == B, only the tiles (i, j >= i) are formed
   const int *s_blk;         // per-block slice counts (kModeX, kModeKPart)
   int shiftT[9];            // truncation T of the fixed-point sum, indexed by s (0..8)
   const int *ea;            // A-side row exponents
@@ -106,6 +107,12 @@ bool make_operand_maps(SgMaps *m, const SgOperand &a, const SgOperand &b, int nw
 // A stand-alone product of A [M][K] and B [N][K] over s digits (kModeRaw, kModeGemm):
 // sizes, tiles and truncation; the caller sets the exponents and the output.
 void grid_params(SgParams *p, int mode, int M, int N, int K, int s);
+
+// CRT variant: the planes of a residue product, the upper tiles only (sym: A ==
+// B, whose products are symmetric) and, if the caller can add partial residues,
+// K splits, single tiles or CTA pairs.
+constexpr int kModSplitMax = 4;
+void plan_mod_gemm(SgParams *p, int planes, bool sym, bool split);
 
 // A grouped launch: the work units of several problems (molecules) in one
 // persistent launch.  Problem i owns units [unit_off[i], unit_off[i+1]); its

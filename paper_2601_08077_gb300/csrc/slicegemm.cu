@@ -518,13 +518,34 @@ __device__ __forceinline__ Unit decode_unit(const SgParams &p, int u, int rank) 
     }
     return kpart_unit(p, i, i + rem, u / npairs);
   } else if constexpr (kMode == kModeMod) {
-    // plane-major, so the B tile of a plane is reused from L2 by its m tiles
-    const int per = p.nt_m * p.nt_n;
-    const int plane = u / per, r = u % per;
-    Unit w = grid_unit(p, r % p.nt_m, r / p.nt_m);
+    // plane- and K-split-major, so the tiles of a plane's K range are reused from L2
+    const int na = kPair ? (p.nt_m + 1) / 2 : p.nt_m;
+    const int per = p.sym ? (kPair ? na * (p.nt_m - na + 1) : na * (na + 1) / 2) : na * p.nt_n;
+    const int ps = u / per, r = u % per;
+    int i, j;
+    if (p.sym) {
+      i = 0;
+      int rem = r;
+      while (rem >= p.nt_m - (kPair ? 2 * i : i)) {
+        rem -= p.nt_m - (kPair ? 2 * i : i);
+        ++i;
+      }
+      if (kPair) i = 2 * i;
+      j = i + rem;
+      i += rank;
+    } else {
+      i = kPair ? 2 * (r % na) + rank : r % na;
+      j = r / na;
+    }
+    Unit w = grid_unit(p, i, j);
+    const int plane = ps / p.nsplit, sp = ps - plane * p.nsplit;
     w.az0 = plane;
     w.bz0 = plane;
     w.blk = plane;
+    w.part = ps;
+    w.kt0 = p.ktiles * sp / p.nsplit;
+    w.ktiles = p.ktiles * (sp + 1) / p.nsplit - w.kt0;
+    if (sp + 1 < p.nsplit) w.ksteps_last = kKTile / 16;
     return w;
   } else {
     if (kPair) {
@@ -702,7 +723,7 @@ __device__ __forceinline__ void store_tile(const SgParams &p, const Unit &w, int
     const uint32_t magic = 0xFFFFFFFFu / (uint32_t)md + 1u;
     const int c24 = (int)((1u << 24) % (unsigned)md);
     const int off24 = (int)(((1u << 24) + (unsigned)md - 1u) / (unsigned)md * (unsigned)md);
-    uint8_t *out = reinterpret_cast<uint8_t *>(p.out) + (long long)w.blk * p.out_blk + (long long)m * p.out_ld + n0c;
+    uint8_t *out = reinterpret_cast<uint8_t *>(p.out) + (long long)w.part * p.out_blk + (long long)m * p.out_ld + n0c;
     if (n0c + 64 <= p.n_valid) {
 #pragma unroll
       for (int j8 = 0; j8 < 8; ++j8) {
@@ -1447,14 +1468,17 @@ static long long x_row_tiles(const SgParams &p, int rows) {
 long long slice_gemm_units(const SgParams &p) {
   if (p.mode == kModeX) return x_row_tiles(p, kTile) * p.nt_n;
   if (p.mode == kModeKPart) return (long long)p.nt_m * (p.nt_m + 1) / 2 * p.nblk * p.nsplit;
+  if (p.mode == kModeMod)
+    return (p.sym ? (long long)p.nt_m * (p.nt_m + 1) / 2 : (long long)p.nt_m * p.nt_n) * p.nblk * p.nsplit;
   return (long long)p.nt_m * p.nt_n;
 }
 
 long long slice_gemm_pairs(const SgParams &p) {
   if (p.mode == kModeX) return x_row_tiles(p, 2 * kTile) * p.nt_n;
   if (p.mode == kModeGemm) return (long long)((p.nt_m + 1) / 2) * p.nt_n;
-  if (p.mode != kModeKPart) return 0;
   const long long nt = p.nt_m, na = (nt + 1) / 2;
+  if (p.mode == kModeMod && !p.sym) return na * p.nt_n * p.nblk * p.nsplit;
+  if (p.mode != kModeKPart && p.mode != kModeMod) return 0;
   return na * (nt - na + 1) * p.nblk * p.nsplit;
 }
 
@@ -1468,9 +1492,35 @@ long long slice_gemm_pairs(const SgParams &p) {
 // when every pair has two tiles or there are tiles enough that one more row of
 // them does not matter.
 static bool use_pairs(const SgParams &p) {
+  if (p.mode == kModeMod) return p.pair != 0;
   if (p.mode == kModeGemm) return p.nt_m % 2 == 0 || p.nt_m >= 16;
   if (p.pair == 0) return false;
   return p.mode == kModeX || (p.mode == kModeKPart && (p.pair == 2 || p.nt_m >= 7));
+}
+
+void plan_mod_gemm(SgParams *p, int planes, bool sym, bool split) {
+  p->nblk = planes;
+  p->sym = sym ? 1 : 0;
+  const int sms = slice_gemm_grid(1 << 30);
+  double best = 0.0;
+  int best_pair = 0, best_n = 1;
+  for (int pair = 0; pair < 2; ++pair)
+    for (int n = 1; n <= (split ? kModSplitMax : 1); ++n) {
+      p->nsplit = n;
+      const long long workers = pair ? sms / 2 : sms;
+      const long long units = pair ? slice_gemm_pairs(*p) : slice_gemm_units(*p);
+      if (workers < 1 || (n > 1 && (p->ktiles / n < 16 || units > 8 * workers))) break;
+      const double waves = (double)((units + workers - 1) / workers);
+      const double cost = waves * ((double)((p->ktiles + n - 1) / n) * (pair ? 370.0 : 515.0) + 3000.0);
+      if (best == 0.0 || cost < 0.95 * best) {
+        best = cost;
+        best_pair = pair;
+        best_n = n;
+      }
+    }
+  p->nsplit = best_n;
+  p->pair = best_pair;
+  p->nunits = (int)slice_gemm_units(*p);
 }
 
 cudaError_t launch_slice_gemm(const SgParams &p, const SgMaps &m, cudaStream_t st, const CoulombWork *cw) {
@@ -1482,6 +1532,7 @@ cudaError_t launch_slice_gemm(const SgParams &p, const SgMaps &m, cudaStream_t s
     SgParams q = p;
     q.npairs = (int)np;
     if (p.mode == kModeGemm) return launch_pair<kModeGemm>(q, m, st);
+    if (p.mode == kModeMod) return launch_pair<kModeMod>(q, m, st);
     if (help)
       return p.mode == kModeX ? launch_pair<kModeX, false, true>(q, m, st, nullptr, *cw)
                               : launch_pair<kModeKPart, false, true>(q, m, st, nullptr, *cw);

@@ -112,6 +112,20 @@ def test_gram_product_shares_one_split(df, nmod):
     assert np.array_equal(out, out.T)
 
 
+@pytest.mark.parametrize("M,N,K,nmod", [(257, 0, 4200, 7), (129, 0, 9001, 12), (33, 0, 2050, 3), (384, 0, 1025, 2),
+                                        (130, 70, 4163, 16), (300, 129, 2112, 5)])
+def test_split_sums_and_upper_tiles(df, M, N, K, nmod):
+    # K in several parts whose residues the reconstruction adds, and (N = 0) the
+    # upper tiles of a Gram matrix only: one and several tile rows, an odd and an
+    # even count, ragged tiles and K, unaligned rows (odd K)
+    rng = np.random.default_rng(M + K + nmod)
+    A = _mat(rng, M, K, spread=4.0, zero_row=min(M - 1, 128))
+    B = _mat(rng, N, K, spread=2.0) if N else A
+    At = torch.from_numpy(A).cuda()
+    out = df.emulated_gemm_crt(At, torch.from_numpy(B).cuda() if N else At, nmod).cpu().numpy()
+    assert np.array_equal(out, CO.emulated_gemm_crt(A, B, nmod))
+
+
 @pytest.mark.parametrize("s", [3, 5])
 def test_slice_gram_product_shares_one_split(df, s):
     from oracle import df_oracle as O
