@@ -138,66 +138,6 @@ bool make_tab(long long K, int n, CrtTab *t) {
   return true;
 }
 
-__device__ __forceinline__ uint64_t abs_bits(double v) {
-  return (uint64_t)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
-}
-
-__device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t w = __shfl_xor_sync(0xffffffffu, v, o);
-    v = w > v ? w : v;
-  }
-  return v;
-}
-
-// Largest absolute bit pattern over the TPR threads of a row (a warp, or the
-// whole 256-thread block through shared memory).
-template <int TPR>
-__device__ __forceinline__ uint64_t row_max_u64(uint64_t m) {
-  m = warp_max_u64(m);
-  if (TPR > 32) {
-    __shared__ uint64_t part[TPR / 32];
-    const int w = (threadIdx.x & (TPR - 1)) >> 5;
-    if ((threadIdx.x & 31) == 0) part[w] = m;
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < TPR / 32; ++i) m = part[i] > m ? part[i] : m;
-  }
-  return m;
-}
-
-// RNE(v 2^(q1 - e)) as int64 for |v| < 127/128 2^e and q1 <= 62.  Integer-only.
-__device__ __forceinline__ long long scaled_rne_q(uint64_t bits, int e, int q1) {
-  int E = (int)((bits >> 52) & 0x7FF);
-  uint64_t m = bits & ((1ull << 52) - 1);
-  if (E == 0) {
-    if (m == 0) return 0;
-    E = 1;
-  } else {
-    m |= (1ull << 52);
-  }
-  // |v| 2^(q1 - e) = m 2^(E - 1075 + q1 - e)
-  const int sh = E - 1075 + q1 - e;
-  uint64_t n;
-  if (sh >= 0) {
-    n = m << sh;  // sh <= q1 - 53 by the headroom
-  } else {
-    const int k = -sh;
-    if (k >= 64) {
-      n = 0;
-    } else {
-      uint64_t q = m >> k;
-      const uint64_t rem = m & ((1ull << k) - 1);
-      const uint64_t half = 1ull << (k - 1);
-      if (rem > half || (rem == half && (q & 1))) q += 1;
-      n = q;
-    }
-  }
-  const long long N = (long long)n;
-  return (bits >> 63) ? -N : N;
-}
-
 // Centred residue, as an exact FP32 value, of the integer whose balanced digit
 // words are (hi, lo), for an odd modulus: S = sum_j b_j (256^j mod m) has |S| <=
 // 8 128^2 = 2^17, so the dot products started at the bits of 1.5 2^23 leave the
@@ -228,22 +168,18 @@ __global__ void __launch_bounds__(256)
   if (r >= rows) return;  // uniform over a row's threads
   const double *row = A + r * ld;
   const bool vec2 = (reinterpret_cast<uintptr_t>(row) & 15) == 0;
-  uint64_t mx = 0;
+  uint32_t mh = 0u;
+  auto bits = [&](int c) { return (uint64_t)__double_as_longlong(__ldg(row + c)); };
+  auto high = [&](double v) { return (uint32_t)__double2hiint(v) & 0x7FFFFFFFu; };
   if (vec2) {
     for (int c = 2 * lane; c < cols; c += 2 * TPR) {
       const double2 v = c + 1 < cols ? __ldg(reinterpret_cast<const double2 *>(row + c)) : make_double2(__ldg(row + c), 0.0);
-      const uint64_t a = abs_bits(v.x), b = abs_bits(v.y);
-      mx = a > mx ? a : mx;
-      mx = b > mx ? b : mx;
+      mh = max(mh, max(high(v.x), high(v.y)));
     }
   } else {
-    for (int c = lane; c < cols; c += TPR) {
-      const uint64_t a = abs_bits(__ldg(row + c));
-      mx = a > mx ? a : mx;
-    }
+    for (int c = lane; c < cols; c += TPR) mh = max(mh, high(__ldg(row + c)));
   }
-  mx = row_max_u64<TPR>(mx);
-  const int e = exponent_from_max_bits_dev(mx);
+  const int e = row_exponent<TPR>(mh, lane, cols, bits);
   if (lane == 0) exps[r] = e;
   uint16_t *drow = planes + r * dld;
   // four columns per lane per step: four independent chains per residue
@@ -262,7 +198,7 @@ __global__ void __launch_bounds__(256)
     for (int h = 0; h < 4; ++h) {
       const uint64_t b = (uint64_t)__double_as_longlong(x[h]);
       // balanced digits: byte j of Mg is b_j + 128 for j < 7, the top byte is b_7
-      const long long Mg = scaled_rne_q(b, e, t.q1) + 0x0080808080808080ll;
+      const long long Mg = scaled_rne(b, e, t.q1) + 0x0080808080808080ll;
       lo[h] = (int)((uint32_t)Mg ^ 0x80808080u);
       hi[h] = (int)((uint32_t)((unsigned long long)Mg >> 32) ^ 0x00808080u);
     }

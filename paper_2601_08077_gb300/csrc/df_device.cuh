@@ -28,35 +28,81 @@ __device__ inline int exponent_from_max_bits_dev(uint64_t bits) {
   return (E - 1023) + 1 + (m >= (127ull << 46) ? 1 : 0);
 }
 
-// N = RNE(v * 2^(63-e)) as int64, for |v| < 127/128 2^e.  Integer-only.
-__device__ inline long long scaled_rne(uint64_t bits, int e) {
-  int E = (int)((bits >> 52) & 0x7FF);
-  uint64_t m = bits & ((1ull << 52) - 1);
-  if (E == 0) {
-    if (m == 0) return 0;
-    E = 1;  // subnormal: value = m 2^(1-1075)
-  } else {
-    m |= (1ull << 52);
+// Shifts of 64 and more give zero (PTX clamps the amount; in C++ they are undefined).
+__device__ __forceinline__ uint64_t shr_clamped(uint64_t v, uint32_t k) {
+  uint64_t r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(k));
+  return r;
+}
+__device__ __forceinline__ uint64_t shl_clamped(uint64_t v, uint32_t k) {
+  uint64_t r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(k));
+  return r;
+}
+
+// N = RNE(v * 2^(q1-e)) as int64, for |v| < 127/128 2^e and q1 <= 63.
+// Integer-only, one path for every exponent: the significand at bits 62..10 moves right
+// by k = 10 - (E - 1075 + q1 - e), which the headroom keeps >= 0; `out` holds what
+// leaves it, so more than half (or half beside an odd quotient: the quotient's low
+// bit goes to the bit of `out` that is always clear) rounds up.
+__device__ __forceinline__ long long scaled_rne(uint64_t bits, int e, int q1 = 63) {
+  const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
+  const int E = (int)((hi >> 20) & 0x7FFu);
+  uint64_t m = ((uint64_t)((hi & 0xFFFFFu) | 0x100000u) << 42) | ((uint64_t)lo << 10);
+  uint32_t k = (uint32_t)(1085 - q1 + e - E);
+  if (E == 0) {  // zero, or subnormal (m 2^(1-1075)): its leading bit moves to bit 62
+    m &= (1ull << 62) - 1;
+    const int z = m ? __clzll((long long)m) - 1 : 0;
+    m <<= z;
+    k += (uint32_t)(z - 1);
   }
-  // |v| 2^(63-e) = m 2^(E - 1075 + 63 - e)
-  int sh = E - 1012 - e;
-  uint64_t n;
-  if (sh >= 0) {
-    n = m << sh;  // sh <= 10 by the headroom, so n < 2^63
-  } else {
-    int k = -sh;
-    if (k >= 64) {
-      n = 0;
-    } else {
-      uint64_t q = m >> k;
-      uint64_t rem = m & ((1ull << k) - 1);
-      uint64_t half = 1ull << (k - 1);
-      if (rem > half || (rem == half && (q & 1))) q += 1;
-      n = q;
+  uint64_t n = shr_clamped(m, k);
+  const uint64_t out = shl_clamped(m, 64u - k) | (n & 1ull);
+  n += out > (1ull << 63) ? 1ull : 0ull;
+  return (hi >> 31) ? -(long long)n : (long long)n;
+}
+
+// Largest value over the TPR threads of a row (TPR = 32: one warp; TPR = 256: the
+// whole block, through shared memory).
+__device__ __forceinline__ uint32_t warp_max(uint32_t v) { return __reduce_max_sync(0xffffffffu, v); }
+__device__ __forceinline__ uint64_t warp_max(uint64_t v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const uint64_t w = __shfl_xor_sync(0xffffffffu, v, o);
+    v = w > v ? w : v;
+  }
+  return v;
+}
+template <int TPR, typename T>
+__device__ __forceinline__ T row_max(T m) {
+  m = warp_max(m);
+  if (TPR > 32) {
+    __shared__ T part[TPR / 32];
+    const int w = (threadIdx.x & (TPR - 1)) >> 5;
+    if ((threadIdx.x & 31) == 0) part[w] = m;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < TPR / 32; ++i) m = part[i] > m ? part[i] : m;
+  }
+  return m;
+}
+
+// Row exponent of the values of a row: mh is this thread's largest high word
+// (without the sign).  The high words settle it unless all are below the
+// normal range, when the row is read again (bits(c): |value c|'s bits).
+template <int TPR, typename Bits>
+__device__ __forceinline__ int row_exponent(uint32_t mh, int lane, int cols, Bits bits) {
+  mh = row_max<TPR>(mh);
+  uint64_t m = (uint64_t)mh << 32;
+  if (mh < 0x00100000u) {  // uniform over the row's threads
+    m = 0;
+    for (int c = lane; c < cols; c += TPR) {
+      const uint64_t a = bits(c) & 0x7FFFFFFFFFFFFFFFull;
+      m = a > m ? a : m;
     }
+    m = row_max<TPR>(m);
   }
-  long long N = (long long)n;
-  return (bits >> 63) ? -N : N;
+  return exponent_from_max_bits_dev(m);
 }
 
 // Balanced digits of N: d[7..1] in [-128,127] from the bottom, d[0] the rest.

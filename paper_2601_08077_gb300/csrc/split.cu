@@ -25,31 +25,6 @@ __device__ __forceinline__ uint64_t abs_bits(double v) {
   return (uint64_t)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
 }
 
-__device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    uint64_t w = __shfl_xor_sync(0xffffffffu, v, o);
-    v = w > v ? w : v;
-  }
-  return v;
-}
-
-// Largest absolute bit pattern over the TPR threads of a row (TPR = 32: one
-// warp; TPR = 256: the whole block, through shared memory).
-template <int TPR>
-__device__ __forceinline__ uint64_t row_max_u64(uint64_t m) {
-  m = warp_max_u64(m);
-  if (TPR > 32) {
-    __shared__ uint64_t part[TPR / 32];
-    const int w = (threadIdx.x & (TPR - 1)) >> 5;
-    if ((threadIdx.x & 31) == 0) part[w] = m;
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < TPR / 32; ++i) m = part[i] > m ? part[i] : m;
-  }
-  return m;
-}
-
 // Digit t of the balanced expansion of N as an exact FP32 value, from
 // M = N + 128 (1 + 256 + ... + 256^6): the top digit is M >> 56, digit t >= 1
 // is byte 7-t of M minus 128.  The FP32 is built as (1.5 2^23 + byte) - (1.5
@@ -94,23 +69,21 @@ template <int TPR, bool kVec2>
 __device__ __forceinline__ void split_row(const double *__restrict__ row, int cols, int lane, int nslices,
                                           int *__restrict__ exp, uint16_t *__restrict__ drow, long long plane_stride,
                                           uint32_t *nz) {
-  uint64_t m = 0;
-  uint32_t bits = 0u;
+  uint32_t mh = 0u, bits = 0u;
 #pragma unroll 4
   for (int c = 4 * lane; c < cols; c += 4 * TPR) {
-    uint64_t v[4], any = 0;
+    uint64_t v[4];
     load4<kVec2>(row, c, cols, v);
+    uint32_t h[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint64_t a = v[i] & 0x7FFFFFFFFFFFFFFFull;
-      m = a > m ? a : m;
-      any |= a;
-    }
-    if (nz && any) bits |= 1u << ((c >> 6) & 31);
+    for (int i = 0; i < 4; ++i) h[i] = (uint32_t)(v[i] >> 32) & 0x7FFFFFFFu;
+    mh = max(max(mh, max(h[0], h[1])), max(h[2], h[3]));
+    if (nz && (h[0] | h[1] | h[2] | h[3] | (uint32_t)v[0] | (uint32_t)v[1] | (uint32_t)v[2] | (uint32_t)v[3]))
+      bits |= 1u << ((c >> 6) & 31);
   }
   if (nz) *nz = bits;
-  m = row_max_u64<TPR>(m);
-  const int e = exponent_from_max_bits_dev(m);
+  const int e = row_exponent<TPR>(
+      mh, lane, cols, [&](int c) { return (uint64_t)__double_as_longlong(__ldg(row + c)); });
   if (lane == 0) *exp = e;
   for (int c = 4 * lane; c < cols; c += 4 * TPR) {
     uint64_t v[4];
@@ -148,7 +121,11 @@ __global__ void __launch_bounds__(256) split_rows_bf16_kernel(const double *__re
 // 64-wide column chunks into mask_mu[mu] (null past 2048 columns).  B comes from
 // DRAM once: the transposed tiles and the second pass of a row are L2 and L1
 // hits.  As three kernels (check, split, masks: one CTA per mu walking all P)
-// the setup of 90 atoms (2.2 GB of B in, 3.3 GB of digits out) took 4.0 ms.
+// the setup of 90 atoms (2.2 GB of B in, 3.3 GB of digits out) took 4.0 ms; this
+// one took 2.0 with dependent tile loads, 1.55 with the next pair in flight
+// (73% of the issue slots, 150 instructions a value) and 1.36 with the row maximum
+// from the high words and a rounding without branches (5.4 TB/s of DRAM traffic:
+// the strips in flight and their digits overflow L2, so part of B is read twice).
 template <bool kVec2>
 __global__ void __launch_bounds__(256) setup_rows_kernel(const double *__restrict__ B, int nao, int nslices,
                                                          int *__restrict__ exps, uint16_t *__restrict__ digits,
@@ -161,16 +138,34 @@ __global__ void __launch_bounds__(256) setup_rows_kernel(const double *__restric
   const double *BP = B + (long long)(perm ? perm[Pq] : Pq) * nao * nao;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   bool bad = false;
+  // tile (bi, bj) and its mirror (bj, bi): B[i][j] of the mirror must equal B[j][i]
+  // = tile[lane][r].  The next pair's loads are in flight while one is compared.
+  double a[4], m[4];
+  const int i0 = bi * 32 + warp, jm = bi * 32 + lane;
+  const double *pa = BP + (long long)i0 * nao + jm, *pm = pa;  // of the diagonal tile; each moves by a tile
+  const long long row8 = 8ll * nao;
+  auto load = [&](int bj) {
+    const int j = bj * 32 + lane, im0 = bj * 32 + warp;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      a[k] = i0 + 8 * k < nao && j < nao ? __ldg(pa + k * row8) : 0.0;
+      m[k] = im0 + 8 * k < nao && jm < nao ? __ldg(pm + k * row8) : 0.0;
+    }
+    pa += 32;
+    pm += 4 * row8;
+  };
+  load(bi);
   for (int bj = bi; bj < nt; ++bj) {
-    for (int r = warp; r < 32; r += 8) {
-      const int i = bi * 32 + r, j = bj * 32 + lane;
-      if (i < nao && j < nao) tile[r][lane] = __ldg(BP + (long long)i * nao + j);
+    double c[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      tile[warp + 8 * k][lane] = a[k];
+      c[k] = m[k];
     }
+    if (bj + 1 < nt) load(bj + 1);
     __syncthreads();
-    for (int r = warp; r < 32; r += 8) {
-      const int i = bj * 32 + r, j = bi * 32 + lane;  // B[i][j] must equal B[j][i] = tile[lane][r]
-      if (i < nao && j < nao && !(__ldg(BP + (long long)i * nao + j) == tile[lane][r])) bad = true;
-    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) bad |= !(c[k] == tile[lane][warp + 8 * k]);
     __syncthreads();
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(flag, 1);
@@ -214,7 +209,7 @@ __global__ void __launch_bounds__(256) split_rows_packed_kernel(const double *__
     const uint64_t a = abs_bits(at(c));
     m = a > m ? a : m;
   }
-  m = warp_max_u64(m);
+  m = warp_max(m);
   const int e = exponent_from_max_bits_dev(m);
   if (lane == 0) exps[r] = e;
   uint16_t *drow = digits + r * dld;
@@ -256,7 +251,7 @@ __global__ void split_rows_int8_kernel(const double *__restrict__ A, int rows, i
     uint64_t a = abs_bits(row[c]);
     m = a > m ? a : m;
   }
-  m = warp_max_u64(m);
+  m = warp_max(m);
   const int e = exponent_from_max_bits_dev(m);
   if (lane == 0) exps[r] = e;
   for (int c = lane; c < cols; c += 32) {

@@ -69,3 +69,31 @@ def test_setup_digits_and_masks(df, naux, nao):
         kt, ch = ctx.sparsity()
         assert ch == pytest.approx(np.mean(upper), abs=1e-12)
         assert kt == pytest.approx(sum(tiles) / (len(tiles) * nk), abs=1e-12)
+
+
+@pytest.mark.parametrize("cols", [150, 2100])
+def test_rounding_at_every_exponent(df, cols):
+    # digits (round to nearest even of v 2^(63-e)) of values from the row's maximum
+    # down to far below its last digit, ties among them, subnormals, signed zeros and
+    # a row that is subnormal throughout; 2100 columns: a whole block per row
+    from oracle import crt_oracle as CO
+    rng = np.random.default_rng(cols)
+    j = np.arange(cols)
+    A = np.zeros((6, cols))
+    A[0] = np.ldexp(rng.integers(2 ** 52, 2 ** 53, cols).astype(float), -52 - j % 75)
+    A[1] = np.ldexp(2.0 * rng.integers(0, 2 ** (1 + j % 51)) + 1.0, -65)   # odd multiples of half a unit (e = 0)
+    A[2] = np.ldexp(2.0 * rng.integers(0, 2 ** (1 + j % 51)) + 1.0, -66 + j % 3)
+    A[1, 0] = A[2, 0] = 0.75
+    A[3] = rng.integers(1, 2 ** 40, cols) * 5e-324
+    A[4] = 5e-324
+    A[4, 1] = -0.0
+    A *= rng.choice([-1.0, 1.0], (6, cols))
+    e_ref, d_ref = O.split_rows(A, 8)
+    e, d = df.split_int8(torch.from_numpy(A).cuda(), 8)
+    assert np.array_equal(e.cpu().numpy(), e_ref.astype(np.int32))
+    assert np.array_equal(d.cpu().numpy(), d_ref)
+    e_ref, Ai = CO.scaled_integers(A, CO.operand_bits(cols, 9))
+    e, R = df.crt_split_rows(torch.from_numpy(A).cuda(), 9)
+    assert np.array_equal(e.cpu().numpy(), e_ref)
+    for i, m in enumerate(CO.moduli(9)):
+        assert np.array_equal(R[i].cpu().numpy(), CO.residues(Ai, m)), m
