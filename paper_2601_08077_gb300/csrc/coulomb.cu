@@ -27,73 +27,29 @@ namespace df {
 
 namespace {
 
-// rho_P for a B with zero 64-wide chunks (a Schwarz-screened B), row by row:
-// warp w takes rows mu = w, w + 8, ...; lanes stride nu > mu.  With masks a
-// warp skips each 32-wide window whose chunks are all zero as a whole (no
-// loads, no FMAs) and keeps the order of the rest; without (DF_OPT_SPARSE
-// off) it runs every window in the same order, so the two are bit-identical
-// (a skipped term is an exact zero).  The row-pair stream would visit every
-// element of the triangle to skip the zero ones.
-template <bool kPacked>
-__device__ __forceinline__ void rho_one_rows(const double *__restrict__ B, const double *__restrict__ D, int nao,
-                                             double *__restrict__ rho, double *__restrict__ rho2,
-                                             const uint32_t *__restrict__ mask_mu, int P, double *red) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double *BP = B + (long long)P * (kPacked ? (long long)nao * (nao + 1) / 2 : (long long)nao * nao);
-  double off = 0.0, dia = 0.0;
-  for (int mu = warp; mu < nao; mu += 8) {
-    // brow[nu] is B_P mu nu for nu >= mu in either layout
-    const double *brow = kPacked ? BP + packed_row(mu, nao) - mu : BP + (long long)mu * nao;
-    const double *drow = D + (long long)mu * nao;
-    if (lane == 0) dia = fma(__ldg(brow + mu), __ldg(drow + mu), dia);
-    if (!mask_mu) {
-      for (int nu = mu + 1 + lane; nu < nao; nu += 32) off = fma(__ldg(brow + nu), __ldg(drow + nu), off);
-    } else {
-      const uint32_t mk = __ldg(mask_mu + mu);
-      for (int base = mu + 1; base < nao; base += 32) {
-        if (!(((mk >> (base >> 6)) | (mk >> ((base + 31) >> 6))) & 1u)) continue;
-        const int nu = base + lane;
-        if (nu < nao && ((mk >> (nu >> 6)) & 1u)) off = fma(__ldg(brow + nu), __ldg(drow + nu), off);
-      }
-    }
-  }
-  double v = 2.0 * off + dia;
-  v = warp_sum(v);
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += red[w];
-    rho[P] = t;
-    if (rho2) rho2[P] = t;
-  }
-}
-
-// rho in the row-by-row order of a B with zero chunks, one CTA per P; rho2
-// (optional): a second copy.
-template <bool kPacked>
-__global__ void __launch_bounds__(256) rho_rows_kernel(const double *__restrict__ B, const double *__restrict__ D,
-                                                       int nao, double *__restrict__ rho, double *__restrict__ rho2,
-                                                       const uint32_t *__restrict__ mask_mu) {
-  __shared__ double red[8];
-  rho_one_rows<kPacked>(B, D, nao, rho, rho2, mask_mu, blockIdx.x, red);
-}
-
-// rho in row-pair order, one CTA per P: its 8 warps are the 8 parts.
-template <bool kPacked>
+// rho of G functions per CTA, whose 8 warps are the 8 parts: in row-pair order
+// (G = 1), or row by row for a B of mostly zero chunks.
+template <bool kPacked, bool kRows, int G>
 __global__ void __launch_bounds__(256, 4) rho_kernel(const double *__restrict__ B, const double *__restrict__ D,
-                                                     int naux, int nao, double *__restrict__ rho,
-                                                     double *__restrict__ rho2) {
-  __shared__ double part[8];
-  double v[1];
-  rho_part<kPacked, 1, 8>(B, D, naux, nao, blockIdx.x, threadIdx.x >> 5, v);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v[0];
+                                                     int naux, int nao, const uint32_t *__restrict__ mask,
+                                                     double *__restrict__ rho, double *__restrict__ rho2) {
+  __shared__ double part[8][G];
+  double v[G];
+  const int P0 = blockIdx.x * G;
+  if constexpr (kRows)
+    rho_part_rows<kPacked, G>(B, D, naux, nao, mask, P0, threadIdx.x >> 5, v);
+  else
+    rho_part<kPacked, G, 8>(B, D, naux, nao, P0, threadIdx.x >> 5, v);
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int g = 0; g < G; ++g) part[threadIdx.x >> 5][g] = v[g];
   __syncthreads();
-  if (threadIdx.x == 0) {
+  const int g = threadIdx.x;
+  if (g < G && P0 + g < naux) {
     double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += part[w];
-    rho[blockIdx.x] = t;
-    if (rho2) rho2[blockIdx.x] = t;
+    for (int w = 0; w < 8; ++w) t += part[w][g];
+    rho[P0 + g] = t;
+    if (rho2) rho2[P0 + g] = t;
   }
 }
 
@@ -304,7 +260,8 @@ cudaError_t launch_density_change(const double *D, double *Dprev, bool have_prev
   return cudaGetLastError();
 }
 
-CoulombWork rho_work(const double *B, const double *D, int naux, int nao, bool packed, double *part, int *work) {
+CoulombWork rho_work(const double *B, const double *D, int naux, int nao, bool packed, bool rows, const uint32_t *mask,
+                     double *part, int *work) {
   CoulombWork w{};
   w.kind = 1;
   w.naux = naux;
@@ -317,11 +274,14 @@ CoulombWork rho_work(const double *B, const double *D, int naux, int nao, bool p
   w.B = B;
   w.D = D;
   w.part = part;
+  w.rows = rows;
+  w.mask = mask;
   w.work = work;
   return w;
 }
 
-CoulombWork coulomb_work_of(const double *B, const double *rho, int naux, int nao, bool packed, double *J, int *work) {
+CoulombWork coulomb_work_of(const double *B, const double *rho, int naux, int nao, bool packed, const uint32_t *mask,
+                            double *J, int *work) {
   CoulombWork w{};
   w.kind = 2;
   w.naux = naux;
@@ -331,22 +291,22 @@ CoulombWork coulomb_work_of(const double *B, const double *rho, int naux, int na
   w.B = B;
   w.rho = rho;
   w.J = J;
+  w.mask = mask;
   w.work = work;
   return w;
 }
 
 cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, double *rho, double *rho2,
                        cudaStream_t st, const uint32_t *mask_mu, bool packed, bool rows) {
-  if (rows || mask_mu) {
-    if (packed)
-      rho_rows_kernel<true><<<(unsigned)naux, 256, 0, st>>>(B, D, nao, rho, rho2, mask_mu);
-    else
-      rho_rows_kernel<false><<<(unsigned)naux, 256, 0, st>>>(B, D, nao, rho, rho2, mask_mu);
-  } else if (packed) {
-    rho_kernel<true><<<(unsigned)naux, 256, 0, st>>>(B, D, naux, nao, rho, rho2);
-  } else {
-    rho_kernel<false><<<(unsigned)naux, 256, 0, st>>>(B, D, naux, nao, rho, rho2);
-  }
+  // row order: the walk over rows and masks costs more instructions than the FMAs,
+  // so functions share it while the SMs keep two CTAs (350 AOs: 700 functions 130
+  // us one by one, 102 by two, 113 by four; 1050 functions 145 by two, 114 by four)
+  const int group = !rows ? 1 : naux >= 1024 ? 4 : naux >= 304 ? 2 : 1;
+  auto kern = packed ? rho_kernel<true, false, 1> : rho_kernel<false, false, 1>;
+  if (rows && group == 4) kern = packed ? rho_kernel<true, true, 4> : rho_kernel<false, true, 4>;
+  if (rows && group == 2) kern = packed ? rho_kernel<true, true, 2> : rho_kernel<false, true, 2>;
+  if (rows && group == 1) kern = packed ? rho_kernel<true, true, 1> : rho_kernel<false, true, 1>;
+  kern<<<(unsigned)((naux + group - 1) / group), 256, 0, st>>>(B, D, naux, nao, mask_mu, rho, rho2);
   return cudaGetLastError();
 }
 

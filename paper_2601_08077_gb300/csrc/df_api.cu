@@ -608,9 +608,8 @@ df_status setup_common(df_ctx *c, const double *B_dev, const int *perm_host, boo
     c->frac_chunks = all ? (double)on / all : 1.0;
     c->frac_ktiles = (double)kon / ((double)ntiles * nk);
     c->sparse = on < all;
-    // rho and J skip chunks only where most are zero: the row order and the mask
-    // tests cost more than a few skipped chunks save (90-atom cube, 2 % zero: rho
-    // 502 us in row order, ~230 in row-pair order)
+    // rho and J skip chunks only where most are zero: the mask tests cost more than
+    // a few skipped chunks save
     c->rows = 2 * on < all;
   }
   c->ready = true;
@@ -658,10 +657,9 @@ df_status df_build_JK(df_ctx *c, const double *D, const double *C, int nocc, int
     s = df::level_count(c, level);
   }
   if (s > c->s_max) return record(c, DF_ERR_ARG);
-  // the native FP64 build, the learned counts, a B of mostly zero chunks (its
-  // masked kernels) and the no-overlap option run the two builds one after the
-  // other
-  if (c->jk_ctas == 0 || s == 0 || (nslices == -2 && c->level > 0) || c->rows) {
+  // the native FP64 build, the learned counts and the no-overlap option run the
+  // two builds one after the other
+  if (c->jk_ctas == 0 || s == 0 || (nslices == -2 && c->level > 0)) {
     df_status r = df_build_J(c, D, J, rho, stream);
     return r == DF_OK ? df_build_K(c, C, nocc, nslices, K, stats, stream) : r;
   }
@@ -673,9 +671,9 @@ df_status df_build_JK(df_ctx *c, const double *D, const double *C, int nocc, int
   // idle: their spare warps run rho beside the first GEMM and J beside the
   // second
   double *rr = rho ? rho : c->rho;
-  const df::CoulombWork w1 = df::rho_work(c->B, D, c->naux, c->nao, c->packed, c->rho_part, c->jk_work);
+  const df::CoulombWork w1 = df::rho_work(c->B, D, c->naux, c->nao, c->packed, c->rows, df::use_mask_mu(c), c->rho_part, c->jk_work);
   const df::RhoParts rp{c->rho_part, rr, rr == c->rho ? nullptr : c->rho, c->naux};
-  const df::CoulombWork w2 = df::coulomb_work_of(c->B, rr, c->naux, c->nao, c->packed, J, c->jk_work + 1);
+  const df::CoulombWork w2 = df::coulomb_work_of(c->B, rr, c->naux, c->nao, c->packed, df::use_mask_mu(c), J, c->jk_work + 1);
   df_status r = df::k_front(c, C, nocc, sb, 0, st, &w1, rp);
   if (r == DF_OK) r = df::k_back(c, nocc, K, st, &w2);
   if (r != DF_OK) return r;

@@ -206,17 +206,18 @@ int fixed_point_shift(int s, long long k);
 // mask_mu (optional, block-sparse B): per mu, bit c set when some B_P mu nu
 // with nu in [64c, 64c + 64) is nonzero; null = dense.
 // packed: B holds per P the upper triangle row by row ([naux][nao (nao + 1) / 2]).
-// rows: rho in the row-by-row order of a B with many zero chunks (taken whenever
-// mask_mu is given), else in row-pair order; the order is the B's, so a
-// screened B gives the same bits with and without its masks.
+// rows: rho in the row-by-row order of a B of mostly zero chunks (nao <= 2048), else
+// in row-pair order; the order is the B's, so a screened B gives the same bits
+// with and without its masks.
 cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, double *rho, double *rho2,
                        cudaStream_t st, const uint32_t *mask_mu, bool packed, bool rows);
 cudaError_t launch_coulomb(const double *B, const double *rho, int naux, int nao, double *J, cudaStream_t st,
                            const uint32_t *mask_mu, bool packed);
-// The same passes as work for a slice GEMM's spare warps (row-pair order, no
-// masks): `work` is zeroed before the launch, part holds 8 naux doubles.
-CoulombWork rho_work(const double *B, const double *D, int naux, int nao, bool packed, double *part, int *work);
-CoulombWork coulomb_work_of(const double *B, const double *rho, int naux, int nao, bool packed, double *J, int *work);
+// The same passes as work for a slice GEMM's spare warps: `work` is zeroed before the launch, part holds 8 naux doubles.
+CoulombWork rho_work(const double *B, const double *D, int naux, int nao, bool packed, bool rows, const uint32_t *mask,
+                     double *part, int *work);
+CoulombWork coulomb_work_of(const double *B, const double *rho, int naux, int nao, bool packed, const uint32_t *mask,
+                            double *J, int *work);
 // The masks of a packed B (pair flags through stream-ordered scratch of nao (nao + 1) / 2 bytes).
 cudaError_t launch_pair_masks_packed(const double *Bp, int naux, int nao, uint32_t *mask_mu, cudaStream_t st);
 // Dense B_P, P = P0 .. P0 + nP - 1, into out [nP][nao][nao] from a packed B.

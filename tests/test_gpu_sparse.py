@@ -136,3 +136,40 @@ def test_screened_chain_in_a_batch(df, chain):
     stream.synchronize()
     for k, k1 in zip(Ks, single):
         assert torch.equal(k, k1)
+
+
+@pytest.mark.parametrize("naux,nao", [(5, 129), (305, 200), (1027, 250), (611, 257)])
+def test_banded_coulomb_alone_and_beside(df, naux, nao):
+    """A banded B (most 64-wide chunks zero), one, two and four functions at a time: rho and J
+    alone, beside the exchange GEMMs, without the masks and from the packed layout, all the same
+    bits; against FP64 within the sums' rounding (each lane adds at most nao products)."""
+    rng = np.random.default_rng(naux + nao)
+    band = np.abs(np.subtract.outer(np.arange(nao), np.arange(nao))) < 12
+    B = np.where(band, rng.standard_normal((naux, nao, nao)), 0.0)
+    B = np.triu(B) + np.triu(B, 1).transpose(0, 2, 1)
+    D = rng.standard_normal((nao, nao))
+    D = D + D.T
+    C = torch.from_numpy(rng.standard_normal((nao, 9))).cuda()
+    Bg, Dg = torch.from_numpy(B).cuda(), torch.from_numpy(D).cuda()
+    iu = np.triu_indices(nao)
+    got = []
+    for packed in (False, True):
+        ctx = df.Context(nao, naux, 9, 3)
+        if packed:
+            ctx.setup_packed(torch.from_numpy(np.ascontiguousarray(B[:, iu[0], iu[1]])).cuda())
+        else:
+            ctx.setup(Bg)
+        assert ctx.sparsity()[1] < 0.5
+        for on in (True, False):
+            ctx.set_sparse(on)
+            J, rho = ctx.build_J(Dg)
+            got.append((J.cpu().numpy(), rho.cpu().numpy()))
+            J, rho, K, _ = ctx.build_JK(Dg, C, 3)
+            got.append((J.cpu().numpy(), rho.cpu().numpy()))
+    for J, rho in got[1:]:
+        assert np.array_equal(J, got[0][0]) and np.array_equal(rho, got[0][1])
+    J, rho = got[0]
+    ref = np.einsum("pij,ij->p", B, D)
+    assert np.all(np.abs(rho - ref) <= 2 * nao * 2.0 ** -52 * np.einsum("pij,ij->p", np.abs(B), np.abs(D)))
+    Jr = np.einsum("pij,p->ij", B, rho)
+    assert np.all(np.abs(J - Jr) <= 2 * naux * 2.0 ** -52 * np.einsum("pij,p->ij", np.abs(B), np.abs(rho)))
