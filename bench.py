@@ -37,6 +37,7 @@ import numpy as np  # noqa: E402
 METRIC = "DF K-build effective FP64 TFLOP/s, INT8-adaptive vs native FP64, max|dK|<=1e-10"
 UNIT = "TFLOP/s"
 LAUNCHES_PER_STEP = 7      # split C, GEMM1 (with rho), split X, GEMM2 (with J), reduce, density change, energy
+FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
 
 
 def parse():
@@ -735,8 +736,8 @@ def main():
     value = FK * world / (ms * 1e-3) / 1e12
     # roofline of the dominant kernel (the slice GEMM launch with the largest share)
     pk, src = peaks()
-    g1_ms = phases["gemm1"][0] / max(1, phases["gemm1"][1])
-    g2_ms = phases["gemm2"][0] / max(1, phases["gemm2"][1])
+    g1_ms = k_phases["gemm1"][0] / max(1, k_phases["gemm1"][1])  # the exchange build alone: no rho and J inside
+    g2_ms = k_phases["gemm2"][0] / max(1, k_phases["gemm2"][1])
     pairs = s * (s + 1) // 2
     g1_flops = pairs * 2.0 * w.nocc * w.naux * w.nao * w.nao
     g2_flops = pairs * 2.0 * (w.nao * (w.nao + 1) / 2) * w.naux * w.nocc
@@ -755,9 +756,7 @@ def main():
                    "slice_count": "fixed for every step (5 = Table 1 level 2's count, the first level meeting "
                                   "max|dK| <= 1e-10 max|K|)" if s == 5 else "fixed for every step", "l2": "inputs larger than L2 (B %.1f GB)" % (B_bytes / 1e9),
                    "cluster_pairs": args.cluster_pairs,
-                   "jk_overlap": ("J, then K, in one stream (df_build_JK; a B of mostly zero chunks runs its "
-                                  "masked kernels in order)" if sparsity[1] < 0.5 else
-                                  "rho and J by spare warps of the exchange GEMMs (df_build_JK)")
+                   "jk_overlap": "rho and J by spare warps of the exchange GEMMs (df_build_JK)"
                                  if args.jk_overlap else "J, then K, in one stream",
                    "parallelism": "replicas" if world > 1 else "single"},
         "e2e": {"value": FK / (ms_e2e * 1e-3) / 1e12 * world, "unit": UNIT, "h2d_bytes_per_step": h2d,

@@ -80,8 +80,8 @@ struct SgParams {
   int *rowE;
 };
 
-// "No nonzero element yet" in a row bound (the byte 0x80 repeated, so a
-// memset resets it); below every real bound.
+// "No nonzero element yet" in a row bound (the C split resets the bounds);
+// below every real bound.
 constexpr int kRowBoundNone = (int)0x80808080;
 
 // Work units of a launch: tiles, and tile pairs in CTA-pair mode (0 = the
@@ -110,7 +110,11 @@ void grid_params(SgParams *p, int mode, int M, int N, int K, int s);
 
 // CRT variant: the planes of a residue product, the upper tiles only (sym: A ==
 // B, whose products are symmetric) and, if the caller can add partial residues,
-// K splits, single tiles or CTA pairs.
+// K splits, single tiles or CTA pairs: the fewest waves over the SMs or pairs of
+// them, weighted with the cycles a K tile takes (515 a tile of its own, 370 a tile
+// of a pair, which takes in 24 KB instead of 32) and 3000 for a unit's store.
+// 600 rows, 240 K tiles, 12 moduli: 15 of 25 tiles, in pairs of two K parts, 105 us
+// for 130.
 constexpr int kModSplitMax = 4;
 void plan_mod_gemm(SgParams *p, int planes, bool sym, bool split);
 
@@ -213,7 +217,8 @@ cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, doub
                        cudaStream_t st, const uint32_t *mask_mu, bool packed, bool rows);
 cudaError_t launch_coulomb(const double *B, const double *rho, int naux, int nao, double *J, cudaStream_t st,
                            const uint32_t *mask_mu, bool packed);
-// The same passes as work for a slice GEMM's spare warps: `work` is zeroed before the launch, part holds 8 naux doubles.
+// The same passes as work for a slice GEMM's spare warps: `work` is zeroed before
+// the launch, part holds 8 naux doubles.
 CoulombWork rho_work(const double *B, const double *D, int naux, int nao, bool packed, bool rows, const uint32_t *mask,
                      double *part, int *work);
 CoulombWork coulomb_work_of(const double *B, const double *rho, int naux, int nao, bool packed, const uint32_t *mask,
