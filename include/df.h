@@ -240,8 +240,9 @@ df_status df_crt_residue_products(const double *A_dev, const double *B_dev, int 
 
 /* out = A B^T (A [M][K], B [N][K], out [M][N], all device, row-major)
  * emulated with nmod moduli; K <= 2^26.  Allocates scratch (2 nmod (M + N)
- * round_up(K, 16) bytes of residue planes, nmod M round_up(N, 16) bytes of
- * residue products); synchronises `stream`.  DF_ERR_ARG for sizes or a
+ * round_up(K, 16) bytes of residue planes, the N term dropping out when A == B
+ * and M == N; nmod M round_up(N, 16) bytes of residue products, up to four
+ * times that while the product has few tiles); synchronises `stream`.  DF_ERR_ARG for sizes or a
  * modulus count that admit no width q >= 2. */
 df_status df_emulated_gemm_crt(const double *A_dev, const double *B_dev, int M, int N, int K, int nmod,
                                double *out_dev, void *stream);
