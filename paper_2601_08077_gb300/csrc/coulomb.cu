@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(256, 5) coulomb_kernel(const double *__restric
   if (!mask_mu || ((__ldg(mask_mu + mu) >> (nu >> 6)) & 1u)) {
     const long long off = kPacked ? packed_row(mu, nao) + (nu - mu) : (long long)mu * nao + nu;
     const long long stride = kPacked ? (long long)nao * (nao + 1) / 2 : (long long)nao * nao;
-    acc = coulomb_sum<8>(B + off, stride, srho, naux);
+    acc = coulomb_sum<8, false>(B + off, stride, srho, naux);
   }
   J[(long long)mu * nao + nu] = acc;
   J[(long long)nu * nao + mu] = acc;

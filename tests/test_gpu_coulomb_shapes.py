@@ -91,3 +91,25 @@ def test_coulomb_odd_molecule(df):
     """27 atoms: nao 135 (odd), naux 405 (a ragged fourth block of 21 functions)."""
     mol, B, C, D = inputs.make_inputs(inputs.Workload("df-27atom-nao135-naux405-nocc27", 27, 27, 7300))
     _check(df, B, C)
+
+
+@pytest.mark.parametrize("naux", [1, 7, 8, 9, 15, 16, 17, 31, 32, 33, 48])
+def test_coulomb_at_the_edges_of_its_load_ring(df, naux):
+    """J's sum over P keeps 8 (alone) or 16 (beside the second exchange GEMM) loads ahead: below one
+    ring, one, two and three of them, and remainders.  Both give the same bits; against FP64 within
+    the rounding of naux additions."""
+    nao = 40
+    rng = np.random.default_rng(naux)
+    B = rng.standard_normal((naux, nao, nao))
+    B = B + B.transpose(0, 2, 1)
+    D = rng.standard_normal((nao, nao))
+    D = D + D.T
+    ctx = df.Context(nao, naux, 4, 3)
+    ctx.setup(torch.from_numpy(B).cuda())
+    Dg = torch.from_numpy(D).cuda()
+    J, rho = ctx.build_J(Dg)
+    J2, rho2, _, _ = ctx.build_JK(Dg, torch.from_numpy(rng.standard_normal((nao, 4))).cuda(), 3)
+    assert torch.equal(J, J2) and torch.equal(rho, rho2)
+    J, rho = J.cpu().numpy(), rho.cpu().numpy()
+    ref = np.einsum("pij,p->ij", B, rho)
+    assert np.all(np.abs(J - ref) <= 2 * naux * 2.0 ** -52 * np.einsum("pij,p->ij", np.abs(B), np.abs(rho)))
