@@ -28,8 +28,8 @@ namespace df {
 namespace {
 
 // rho of G functions per CTA, whose 8 warps are the 8 parts: in row-pair order
-// (G = 1), or row by row for a B of mostly zero chunks.
-template <bool kPacked, bool kRows, int G>
+// (G = 1, with offsets of type Off), or row by row for a B of mostly zero chunks.
+template <bool kPacked, bool kRows, int G, typename Off = int>
 __global__ void __launch_bounds__(256, 4) rho_kernel(const double *__restrict__ B, const double *__restrict__ D,
                                                      int naux, int nao, const uint32_t *__restrict__ mask,
                                                      double *__restrict__ rho, double *__restrict__ rho2) {
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(256, 4) rho_kernel(const double *__restrict__ 
   if constexpr (kRows)
     rho_part_rows<kPacked, G>(B, D, naux, nao, mask, P0, threadIdx.x >> 5, v);
   else
-    rho_part<kPacked, G, 8>(B, D, naux, nao, P0, threadIdx.x >> 5, v);
+    rho_part<kPacked, G, 8, Off>(B, D, naux, nao, P0, threadIdx.x >> 5, v);
   if ((threadIdx.x & 31) == 0)
 #pragma unroll
     for (int g = 0; g < G; ++g) part[threadIdx.x >> 5][g] = v[g];
@@ -303,6 +303,9 @@ cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, doub
   // us one by one, 102 by two, 113 by four; 1050 functions 145 by two, 114 by four)
   const int group = !rows ? 1 : naux >= 1024 ? 4 : naux >= 304 ? 2 : 1;
   auto kern = packed ? rho_kernel<true, false, 1> : rho_kernel<false, false, 1>;
+  // one B_P past 2^31 elements (at 32 bits everywhere else: 64-bit offsets cost a packed B
+  // 8 %, 587 -> 637 us at 600 AOs and 1800 functions)
+  if (nao > kRho32Nao) kern = packed ? rho_kernel<true, false, 1, long long> : rho_kernel<false, false, 1, long long>;
   if (rows && group == 4) kern = packed ? rho_kernel<true, true, 4> : rho_kernel<false, true, 4>;
   if (rows && group == 2) kern = packed ? rho_kernel<true, true, 2> : rho_kernel<false, true, 2>;
   if (rows && group == 1) kern = packed ? rho_kernel<true, true, 1> : rho_kernel<false, true, 1>;

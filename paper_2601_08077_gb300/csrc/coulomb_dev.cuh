@@ -90,20 +90,23 @@ constexpr int kRhoLanes = 256;  // eight parts of a warp each
 // for G functions P = P0 .. P0 + G-1 at once (the last one repeated past naux),
 // in every lane.  The diagonal terms are spread over the lanes; the strictly
 // upper ones stream in row-pair order, kQ steps of loads ahead of their FMAs,
-// one load of D for G functions.  Offsets within G functions fit 32 bits (G
-// nao^2 <= 2^31; G = 1 for a larger nao).
-template <bool kPacked, int G, int kQ>
+// one load of D for G functions.  Offsets within the G functions are Off: 32 bits hold
+// them while G nao^2 < 2^31 (kRho32Nao for one function), 64 for any nao.
+constexpr int kRho32Nao = 46340;
+template <bool kPacked, int G, int kQ, typename Off>
 __device__ __forceinline__ void rho_part(const double *__restrict__ B, const double *__restrict__ D, int naux, int nao,
                                          int P0, int w, double (&v)[G]) {
   const int t = 32 * w + (threadIdx.x & 31);
-  const int stride = kPacked ? nao * (nao + 1) / 2 : nao * nao;
+  const Off n = nao;
+  const Off stride = kPacked ? n * (n + 1) / 2 : n * n;
   const double *BP = B + (long long)P0 * stride;
-  int gs[G];
+  Off gs[G];
 #pragma unroll
   for (int g = 0; g < G; ++g) gs[g] = G == 1 ? 0 : min(g, naux - 1 - P0) * stride;
-  auto load = [&](int idx, int g) -> double { return __ldg(BP + (G == 1 ? idx : idx + gs[g])); };
-  auto index = [&](int mu, int nu) -> int {
-    return kPacked ? mu * nao - mu * (mu - 1) / 2 + (nu - mu) : mu * nao + nu;
+  auto load = [&](Off idx, int g) -> double { return __ldg(BP + (G == 1 ? idx : idx + gs[g])); };
+  auto index = [&](int mu, int nu) -> Off {
+    const Off m = mu;
+    return kPacked ? m * n - m * (m - 1) / 2 + (nu - mu) : m * n + nu;
   };
   double dia[G], off[G];
 #pragma unroll
@@ -113,7 +116,7 @@ __device__ __forceinline__ void rho_part(const double *__restrict__ B, const dou
 #pragma unroll
     for (int g = 0; g < G; ++g) dia[g] = fma(load(index(mu, mu), g), d, dia[g]);
   }
-  const int total = nao * (nao - 1) / 2;
+  const Off total = n * (n - 1) / 2;
   if (total > t) {
     PairStream ps;
     ps.init(t, nao);
@@ -125,16 +128,16 @@ __device__ __forceinline__ void rho_part(const double *__restrict__ B, const dou
       if (ps.valid()) {
         int mu, nu;
         ps.at(mu, nu);
-        const int idx = index(mu, nu);
+        const Off idx = index(mu, nu);
 #pragma unroll
         for (int g = 0; g < G; ++g) bq[k][g] = load(idx, g);
-        dq[k] = __ldg(D + (mu * nao + nu));
+        dq[k] = __ldg(D + (mu * n + nu));
       }
       ps.advance(kRhoLanes);
     };
 #pragma unroll
     for (int k = 0; k < kQ; ++k) fill(k);
-    const int mine = (total - t + kRhoLanes - 1) / kRhoLanes;
+    const int mine = (int)((total - t + kRhoLanes - 1) / kRhoLanes);
     const int rounds = (mine + kQ - 1) / kQ;
     for (int r = 0; r < rounds; ++r) {
 #pragma unroll
@@ -266,7 +269,7 @@ __device__ __forceinline__ int take_item(int *work) {
 }
 __device__ __forceinline__ int item_of_warp(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
-template <bool kPacked, bool kRows, int G, int kQ>
+template <bool kPacked, bool kRows, int G, int kQ, typename Off>
 __device__ __forceinline__ void rho_items(const CoulombWork &w) {
   int it = item_of_warp(take_item(w.work));
   while (it < w.nitems) {
@@ -276,7 +279,7 @@ __device__ __forceinline__ void rho_items(const CoulombWork &w) {
     if constexpr (kRows)
       rho_part_rows<kPacked, G>(w.B, w.D, w.naux, w.nao, w.mask, P0, it & 7, v);
     else
-      rho_part<kPacked, G, kQ>(w.B, w.D, w.naux, w.nao, P0, it & 7, v);
+      rho_part<kPacked, G, kQ, Off>(w.B, w.D, w.naux, w.nao, P0, it & 7, v);
     if ((threadIdx.x & 31) == 0) {
 #pragma unroll
       for (int g = 0; g < G; ++g)
@@ -306,12 +309,13 @@ __device__ __forceinline__ void coulomb_items(const CoulombWork &w) {
   }
 }
 
+// A group of four has nao <= 16384 (rho_work); one function at a time takes any nao.
 template <bool kPacked, bool kRows>
 __device__ __forceinline__ void rho_any_group(const CoulombWork &w) {
   if (w.group == 4)
-    rho_items<kPacked, kRows, 4, 3>(w);
+    rho_items<kPacked, kRows, 4, 3, int>(w);
   else
-    rho_items<kPacked, kRows, 1, 8>(w);
+    rho_items<kPacked, kRows, 1, 8, long long>(w);
 }
 
 template <int kKind>
