@@ -286,8 +286,9 @@ const char *df_strerror(df_status s);
  * units of every molecule, the X splits, ONE persistent launch of the second
  * GEMM, and the reductions (Section 3.3 blocking per molecule, Section 3.2
  * emulation).  With graphs on (the default) the whole sequence is captured
- * once per (nslices, argument pointers) as a CUDA graph and replayed; a NULL
- * stream runs it without a graph.  The per-molecule kernels between the
+ * once per (nslices, argument pointers) as a CUDA graph and replayed, and
+ * captured again after a context was set up on another B or had an option
+ * changed; a NULL stream runs it without a graph.  The per-molecule kernels between the
  * grouped launches (X splits, reductions; in df_batch_build_J each
  * molecule's rho and J) run concurrently on four internal streams that fork
  * from and join back into `stream`, so a call is still ordered with the

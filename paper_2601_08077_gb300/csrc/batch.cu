@@ -44,9 +44,9 @@ struct df_batch {
   cudaStream_t side[kFan] = {};
   cudaEvent_t ev_fork = nullptr;
   cudaEvent_t ev_join[kFan] = {};
-  // graph cache
+  // graph cache; the keys hold what a recorded graph, or the tables it runs on, rest on
   cudaGraphExec_t exec_K = nullptr, exec_J = nullptr;
-  std::vector<const void *> key_K, key_J;
+  std::vector<const void *> key_K, key_J, key_tables;
   int key_s = -1;
 };
 
@@ -74,6 +74,16 @@ cudaError_t join(df_batch *b, cudaStream_t st) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, b->ev_join[k], 0);
   }
   return e;
+}
+
+// What the grouped tables take from the contexts that a later setup or option can change.
+std::vector<const void *> tables_key(const df_batch *b) {
+  std::vector<const void *> key;
+  for (const df_ctx *c : b->ctx) {
+    key.push_back(df::use_mask_tile(c));
+    key.push_back(reinterpret_cast<const void *>((uintptr_t)c->pair_mode));
+  }
+  return key;
 }
 
 // Molecule order for the unit lists.
@@ -121,6 +131,7 @@ df_status build_tables(df_batch *b, const int *nocc) {
   if (e == cudaSuccess) e = cudaMemcpy(b->off1, o1.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(b->off2, o2.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice);
   b->nocc.assign(nocc, nocc + n);
+  b->key_tables = tables_key(b);
   return cerr(e);
 }
 
@@ -178,7 +189,7 @@ df_status prepare(df_batch *b, const int *nocc, int s, cudaStream_t st) {
     df_status r = df::ctx_upload_slices(c, sb.data(), st);
     if (r != DF_OK) return r;
   }
-  bool same = b->tables_for_s == s && (int)b->nocc.size() == n;
+  bool same = b->tables_for_s == s && (int)b->nocc.size() == n && b->key_tables == tables_key(b);
   for (int i = 0; same && i < n; ++i) same = b->nocc[i] == nocc[i];
   if (!same) {
     if (cudaStreamSynchronize(st) != cudaSuccess) return DF_ERR_CUDA;
@@ -313,8 +324,13 @@ df_status df_batch_build_J(df_batch *b, const double *const *D, double *const *J
   if (!b->graphs || st == nullptr) return enqueue();
   std::vector<const void *> key;
   for (int i = 0; i < n; ++i) {
+    const df_ctx *c = b->ctx[i];
     key.push_back(D[i]);
     key.push_back(J[i]);
+    // a context that was set up again: another B, layout or sparsity
+    key.push_back(c->B);
+    key.push_back(df::use_mask_mu(c));
+    key.push_back(reinterpret_cast<const void *>((uintptr_t)(c->packed ? 1 : 0) + (c->rows ? 2 : 0)));
   }
   if (!b->exec_J || key != b->key_J) {
     drop_graph(b->exec_J);

@@ -143,3 +143,46 @@ def test_batch_side_streams_join_the_callers_stream(df, molecules):
             assert torch.equal(k, k1)
         for j, j1 in zip(Jc, Js1):
             assert torch.equal(j, j1)
+
+
+def test_batch_follows_a_context_that_is_set_up_again(df):
+    """A geometry step inside a batch: the contexts get another B (dense, packed, screened to a
+    band, dense again) while D, C, J and K stay the same buffers.  Every recorded graph must run
+    on the new B: J and K equal the single builds bit for bit.  All the tensors stay alive."""
+    s, nao, naux, nocc = 3, 140, 150, 20
+    rng = np.random.default_rng(7)
+    D = rng.standard_normal((nao, nao))
+    Ds = [torch.from_numpy(D + D.T).cuda() for _ in range(2)]
+    Cs = [torch.from_numpy(rng.standard_normal((nao, nocc))).cuda() for _ in range(2)]
+    band = np.abs(np.subtract.outer(np.arange(nao), np.arange(nao))) < 9
+    iu = np.triu_indices(nao)
+    ctxs = [df.Context(nao, naux, nocc, s_max=s) for _ in range(2)]
+    keep, batch = [], None
+    stream = torch.cuda.Stream()
+    Js, Ks = [torch.empty_like(d) for d in Ds], [torch.empty_like(d) for d in Ds]
+    for step in ("dense", "dense", "packed", "band", "dense"):
+        B = rng.standard_normal((naux, nao, nao))
+        B = np.triu(B) + np.triu(B, 1).transpose(0, 2, 1)
+        if step == "band":
+            B = np.where(band, B, 0.0)
+        # the first context changes, the second one keeps its B after the first step
+        for ctx in ctxs[:1] if keep else ctxs:
+            if step == "packed":
+                keep.append(torch.from_numpy(np.ascontiguousarray(B[:, iu[0], iu[1]])).cuda())
+                ctx.setup_packed(keep[-1])
+            else:
+                keep.append(torch.from_numpy(B).cuda())
+                ctx.setup(keep[-1])
+        if batch is None:
+            batch = df.Batch(ctxs)
+        assert (ctxs[0].sparsity()[1] < 0.5) == (step == "band")
+        single_J = [ctx.build_J(d)[0].clone() for ctx, d in zip(ctxs, Ds)]
+        single_K = [ctx.build_K(c, s)[0].clone() for ctx, c in zip(ctxs, Cs)]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            for _ in range(2):
+                batch.build_J(Ds, Js, stream=stream)
+                batch.build_K(Cs, s, Ks, stream=stream)
+        stream.synchronize()
+        for got, want in zip(Js + Ks, single_J + single_K):
+            assert torch.equal(got, want), step
