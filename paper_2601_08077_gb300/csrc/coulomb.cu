@@ -78,16 +78,14 @@ __global__ void __launch_bounds__(256, 5) coulomb_kernel(const double *__restric
 }
 
 // True in every thread of the last CTA of the grid to arrive here (each CTA's
-// global writes before it are visible to that CTA); it also resets the ticket
-// for the next launch.
+// global writes before it are visible to that CTA).  The ticket wraps to zero at
+// the last arrival in one atomic, so it is zero after any number of whole
+// launches, also when two of them shared it at the same time.
 __device__ __forceinline__ bool last_block(unsigned *ticket) {
   __shared__ bool last;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    if (last) *ticket = 0u;
-  }
+  if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
   __syncthreads();
   if (last) __threadfence();
   return last;

@@ -113,3 +113,27 @@ def test_coulomb_at_the_edges_of_its_load_ring(df, naux):
     J, rho = J.cpu().numpy(), rho.cpu().numpy()
     ref = np.einsum("pij,p->ij", B, rho)
     assert np.all(np.abs(J - ref) <= 2 * naux * 2.0 ** -52 * np.einsum("pij,p->ij", np.abs(B), np.abs(rho)))
+
+
+def test_energies_after_overlapping_calls(df):
+    """Energies of one context asked for from four threads on their own streams (their launches
+    share the context's partial sums and its count of finished blocks), then alone: the count must
+    be back at zero, so the later call reduces all of its blocks and returns the usual values."""
+    from concurrent.futures import ThreadPoolExecutor
+
+    B, C = _random(5, 40, 96, 12)
+    ctx = df.Context(96, 40, 12, 3)
+    ctx.setup(torch.from_numpy(B).cuda())
+    D = torch.from_numpy(C @ C.T).cuda()
+    J, rho, K, _ = ctx.build_JK(D, torch.from_numpy(C).cuda(), 3)
+    torch.cuda.synchronize()
+    want = ctx.energy(D, J, K, rho)
+    streams = [torch.cuda.Stream() for _ in range(4)]
+
+    def ask(st):
+        for _ in range(200):
+            ctx.energy(D, J, K, rho, stream=st)
+
+    with ThreadPoolExecutor(4) as ex:
+        list(ex.map(ask, streams))
+    assert all(ctx.energy(D, J, K, rho) == want for _ in range(3))
