@@ -546,14 +546,17 @@ namespace {
 df_status setup_common(df_ctx *c, const double *B_dev, const int *perm_host, bool packed, void *stream) {
   if (!c || !B_dev) return record(c, DF_ERR_ARG);
   cudaStream_t st = as_stream(stream);
-  c->B = B_dev;
-  c->packed = packed;
-  if (perm_host) {
+  if (perm_host) {  // before anything changes: a refused order leaves the context as it is
     std::vector<char> seen(c->naux, 0);
     for (int i = 0; i < c->naux; ++i) {
       if (perm_host[i] < 0 || perm_host[i] >= c->naux || seen[perm_host[i]]) return record(c, DF_ERR_ARG);
       seen[perm_host[i]] = 1;
     }
+  }
+  c->ready = false;
+  c->B = B_dev;
+  c->packed = packed;
+  if (perm_host) {
     if (!c->perm) DF_TRY(c, cudaMalloc(&c->perm, sizeof(int) * c->naux));
     DF_TRY(c, cudaMemcpy(c->perm, perm_host, sizeof(int) * c->naux, cudaMemcpyHostToDevice));
     c->perm_h.assign(perm_host, perm_host + c->naux);
@@ -566,7 +569,6 @@ df_status setup_common(df_ctx *c, const double *B_dev, const int *perm_host, boo
     cudaFree(c->bstats);
     c->bstats = nullptr;
   }
-  c->ready = false;
   const long long rows = (long long)c->naux * c->nao;
   const int ntiles = (int)((rows + df::kTile - 1) / df::kTile);
   // block sparsity of a screened B (Section 2.1): exact zero chunks of the AO pairs

@@ -277,27 +277,27 @@ class Context:
     def setup(self, B: torch.Tensor, perm=None, stream=None):
         """Attach B; `perm` (new position -> original P) orders the exchange path's auxiliary functions."""
         assert B.shape == (self.naux, self.nao, self.nao)
-        self._B = B  # the library keeps the pointer: keep the tensor alive
         if perm is None:
             _check(lib().df_setup(self._h, _f64(B), _stream(stream)), "df_setup")
         else:
             arr = (ctypes.c_int * self.naux)(*[int(x) for x in perm])
             _check(lib().df_setup_ordered(self._h, _f64(B), arr, _stream(stream)), "df_setup_ordered")
+        self._B = B  # the library keeps the pointer: keep the tensor alive (a refused one is not attached)
 
     def setup_packed(self, Bp: torch.Tensor, perm=None, stream=None):
         """Attach B given as packed upper triangles [naux, nao (nao + 1) / 2] (see inputs.pack_upper)."""
         assert Bp.shape == (self.naux, self.nao * (self.nao + 1) // 2)
-        self._B = Bp
         arr = None if perm is None else (ctypes.c_int * self.naux)(*[int(x) for x in perm])
         _check(lib().df_setup_packed(self._h, _f64(Bp), arr, _stream(stream)), "df_setup_packed")
+        self._B = Bp
 
     def setup_integrals(self, T: torch.Tensor, V: torch.Tensor, perm=None, stream=None):
         """Form B = L^{-1} T in place on the device (L L^T = V) and attach it; returns T (now B)."""
         assert T.shape == (self.naux, self.nao, self.nao) and V.shape == (self.naux, self.naux)
         assert T.dtype == torch.float64 and V.dtype == torch.float64 and T.is_contiguous() and V.is_contiguous()
-        self._B = T
         arr = None if perm is None else (ctypes.c_int * self.naux)(*[int(x) for x in perm])
         _check(lib().df_setup_integrals(self._h, _f64(T), _f64(V), arr, _stream(stream)), "df_setup_integrals")
+        self._B = T
         return T
 
     def build_J(self, D, J=None, rho=None, stream=None):

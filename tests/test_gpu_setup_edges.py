@@ -97,3 +97,28 @@ def test_rounding_at_every_exponent(df, cols):
     assert np.array_equal(e.cpu().numpy(), e_ref)
     for i, m in enumerate(CO.moduli(9)):
         assert np.array_equal(R[i].cpu().numpy(), CO.residues(Ai, m)), m
+
+
+def test_refused_order_leaves_the_context_as_it_was(df):
+    # a set-up context that is offered another B (packed) with an order that is no
+    # permutation: DF_ERR_ARG, and the builds go on with the B that it holds
+    nao, naux = 65, 20
+    B = torch.from_numpy(_tensor(1, naux, nao)).cuda()
+    iu = torch.triu_indices(nao, nao, device="cuda")
+    other = torch.from_numpy(_tensor(2, naux, nao)).cuda()[:, iu[0], iu[1]].contiguous()
+    rng = np.random.default_rng(3)
+    D = torch.from_numpy(rng.standard_normal((nao, nao))).cuda()
+    D = D + D.T
+    C = torch.from_numpy(rng.standard_normal((nao, 7))).cuda()
+    ctx = df.Context(nao, naux, 7, 3)
+    ctx.setup(B)
+    J, rho, K, _ = ctx.build_JK(D, C, 3)
+    del B  # the context keeps it
+    for perm in (np.zeros(naux, dtype=np.int32), np.arange(1, naux + 1, dtype=np.int32)):
+        with pytest.raises(df.DFError) as e:
+            ctx.setup_packed(other, perm)
+        assert e.value.status == -1
+        junk = torch.full((naux, nao, nao), float("nan"), dtype=torch.float64, device="cuda")  # takes freed memory
+        J1, rho1 = ctx.build_J(D)
+        K1, _ = ctx.build_K(C, 3)
+        assert torch.equal(J1, J) and torch.equal(rho1, rho) and torch.equal(K1, K)
