@@ -404,9 +404,9 @@ int64_t df_workspace_bytes(const df_ctx *ctx);
  * counts the surviving pairs as N_scr).  At setup the library records, per mu,
  * which 64-wide chunks of nu hold a nonzero B_P mu nu for some P; when some
  * chunk is zero (and nao <= 2048) the first exchange GEMM runs only the
- * nonzero 64-wide K tiles of each 128-row tile of B's (P, mu) rows, and, when
- * most chunks are zero, rho and J skip them.  Skipped terms are exact zeros: every result is
- * the one of the dense build.  frac_ktiles: nonzero K tiles / all of the first
+ * nonzero 64-wide K tiles of each 128-row tile of B's (P, mu) rows, J skips the
+ * zero chunks and so does rho when most chunks are zero.  Skipped terms are exact
+ * zeros: every result is the one of the dense build.  frac_ktiles: nonzero K tiles / all of the first
  * GEMM's row tiles; frac_chunks: nonzero (mu, chunk) pairs of the upper
  * triangle / all.  Both 1 for a B without zero chunks.  DF_ERR_STATE before
  * setup. */

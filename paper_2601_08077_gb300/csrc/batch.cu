@@ -313,10 +313,10 @@ df_status df_batch_build_J(df_batch *b, const double *const *D, double *const *J
     for (int i = 0; i < n; ++i) {
       df_ctx *c = b->ctx[i];
       cudaStream_t si = b->side[i % df_batch::kFan];
-      const uint32_t *mk = df::use_mask_mu(c);
-      if (df::launch_rho(c->B, D[i], c->naux, c->nao, c->rho, nullptr, si, mk, c->packed, c->rows) != cudaSuccess)
+      if (df::launch_rho(c->B, D[i], c->naux, c->nao, c->rho, nullptr, si, df::use_mask_rho(c), c->packed, c->rows) !=
+          cudaSuccess)
         return DF_ERR_CUDA;
-      if (df::launch_coulomb(c->B, c->rho, c->naux, c->nao, J[i], si, mk, c->packed) != cudaSuccess)
+      if (df::launch_coulomb(c->B, c->rho, c->naux, c->nao, J[i], si, df::use_mask_j(c), c->packed) != cudaSuccess)
         return DF_ERR_CUDA;
     }
     return join(b, st) == cudaSuccess ? DF_OK : DF_ERR_CUDA;
@@ -329,7 +329,8 @@ df_status df_batch_build_J(df_batch *b, const double *const *D, double *const *J
     key.push_back(J[i]);
     // a context that was set up again: another B, layout or sparsity
     key.push_back(c->B);
-    key.push_back(df::use_mask_mu(c));
+    key.push_back(df::use_mask_rho(c));
+    key.push_back(df::use_mask_j(c));
     key.push_back(reinterpret_cast<const void *>((uintptr_t)(c->packed ? 1 : 0) + (c->rows ? 2 : 0)));
   }
   if (!b->exec_J || key != b->key_J) {

@@ -610,8 +610,8 @@ df_status setup_common(df_ctx *c, const double *B_dev, const int *perm_host, boo
     c->frac_chunks = all ? (double)on / all : 1.0;
     c->frac_ktiles = (double)kon / ((double)ntiles * nk);
     c->sparse = on < all;
-    // rho and J skip chunks only where most are zero: the mask tests cost more than
-    // a few skipped chunks save
+    // rho skips chunks only where most are zero: its walk over rows and masks costs more
+    // than a few skipped chunks save
     c->rows = 2 * on < all;
   }
   c->ready = true;
@@ -635,12 +635,12 @@ df_status df_build_J(df_ctx *c, const double *D, double *J, double *rho, void *s
   double *r = rho ? rho : c->rho;
   {
     PhaseTimer t(c, DF_PHASE_RHO, st);
-    DF_TRY(c, df::launch_rho(c->B, D, c->naux, c->nao, r, r == c->rho ? nullptr : c->rho, st, df::use_mask_mu(c),
+    DF_TRY(c, df::launch_rho(c->B, D, c->naux, c->nao, r, r == c->rho ? nullptr : c->rho, st, df::use_mask_rho(c),
                              c->packed, c->rows));
   }
   {
     PhaseTimer t(c, DF_PHASE_COULOMB, st);
-    DF_TRY(c, df::launch_coulomb(c->B, r, c->naux, c->nao, J, st, df::use_mask_mu(c), c->packed));
+    DF_TRY(c, df::launch_coulomb(c->B, r, c->naux, c->nao, J, st, df::use_mask_j(c), c->packed));
   }
   // the density change since the last Coulomb build (an input of the learned slice counts)
   DF_TRY(c, df::launch_density_change(D, c->Dprev, c->have_Dprev, (long long)c->nao * c->nao, c->dD_part, c->tickets, c->dD, st));
@@ -673,9 +673,9 @@ df_status df_build_JK(df_ctx *c, const double *D, const double *C, int nocc, int
   // idle: their spare warps run rho beside the first GEMM and J beside the
   // second
   double *rr = rho ? rho : c->rho;
-  const df::CoulombWork w1 = df::rho_work(c->B, D, c->naux, c->nao, c->packed, c->rows, df::use_mask_mu(c), c->rho_part, c->jk_work);
+  const df::CoulombWork w1 = df::rho_work(c->B, D, c->naux, c->nao, c->packed, c->rows, df::use_mask_rho(c), c->rho_part, c->jk_work);
   const df::RhoParts rp{c->rho_part, rr, rr == c->rho ? nullptr : c->rho, c->naux};
-  const df::CoulombWork w2 = df::coulomb_work_of(c->B, rr, c->naux, c->nao, c->packed, df::use_mask_mu(c), J, c->jk_work + 1);
+  const df::CoulombWork w2 = df::coulomb_work_of(c->B, rr, c->naux, c->nao, c->packed, df::use_mask_j(c), J, c->jk_work + 1);
   df_status r = df::k_front(c, C, nocc, sb, 0, st, &w1, rp);
   if (r == DF_OK) r = df::k_back(c, nocc, K, st, &w2);
   if (r != DF_OK) return r;

@@ -173,3 +173,56 @@ def test_banded_coulomb_alone_and_beside(df, naux, nao):
     assert np.all(np.abs(rho - ref) <= 2 * nao * 2.0 ** -52 * np.einsum("pij,ij->p", np.abs(B), np.abs(D)))
     Jr = np.einsum("pij,p->ij", B, rho)
     assert np.all(np.abs(J - Jr) <= 2 * naux * 2.0 ** -52 * np.einsum("pij,p->ij", np.abs(B), np.abs(rho)))
+
+
+@pytest.mark.parametrize("nao,half", [(130, 70), (200, 130), (300, 170)])
+def test_partly_screened_coulomb_skips_zero_chunks(df, nao, half):
+    """A B with some zero 64-wide chunks, but not most of them: J skips the zero ones alone, beside
+    the second exchange GEMM and in a batch, dense and packed.  With finite rho every result equals
+    the unmasked one; where a rho is infinite a skipped pair stays exactly zero."""
+    rng = np.random.default_rng(nao)
+    naux = 37
+    keep = np.abs(np.subtract.outer(np.arange(nao), np.arange(nao))) < half
+    B = np.where(keep, rng.standard_normal((naux, nao, nao)), 0.0)
+    B = np.triu(B) + np.triu(B, 1).transpose(0, 2, 1)
+    D = rng.standard_normal((nao, nao))
+    D = D + D.T
+    huge = np.where(D > 0, 1e308, -1e308)
+    huge = np.triu(huge) + np.triu(huge, 1).T
+    C = torch.from_numpy(rng.standard_normal((nao, 9))).cuda()
+    iu = np.triu_indices(nao)
+    # pairs (mu, nu >= mu) in a chunk of mu's row without a nonzero
+    nz = np.zeros((nao, (nao + 63) // 64), bool)
+    for c in range(nz.shape[1]):
+        nz[:, c] = keep[:, 64 * c:64 * c + 64].any(1)
+    skipped = ~nz[:, np.arange(nao) // 64] & (np.arange(nao)[:, None] <= np.arange(nao)[None, :])
+    assert skipped.any()
+    for packed in (False, True):
+        ctx = df.Context(nao, naux, 9, 3)
+        if packed:
+            Bg = torch.from_numpy(np.ascontiguousarray(B[:, iu[0], iu[1]])).cuda()
+            ctx.setup_packed(Bg)
+        else:
+            Bg = torch.from_numpy(B).cuda()
+            ctx.setup(Bg)
+        assert 0.5 <= ctx.sparsity()[1] < 1.0
+        batch = df.Batch([ctx])
+        stream = torch.cuda.Stream()
+        for d in (D, huge):
+            Dg = torch.from_numpy(d).cuda()
+            J, rho = (t.clone() for t in ctx.build_J(Dg))
+            J2, rho2 = (t.clone() for t in ctx.build_JK(Dg, C, 3)[:2])
+            Jb = torch.empty_like(J)
+            torch.cuda.synchronize()
+            with torch.cuda.stream(stream):
+                batch.build_J([Dg], [Jb], stream=stream)
+            stream.synchronize()
+            for x, y in ((J2, J), (rho2, rho), (Jb, J)):
+                assert np.array_equal(x.cpu().numpy(), y.cpu().numpy(), equal_nan=True)
+            assert np.all(J.cpu().numpy()[skipped] == 0.0)
+            if d is D:
+                ctx.set_sparse(False)
+                assert torch.equal(ctx.build_J(Dg)[0], J)
+                ctx.set_sparse(True)
+            else:
+                assert not np.isfinite(rho.cpu().numpy()).all()
