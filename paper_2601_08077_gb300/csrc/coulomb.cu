@@ -29,8 +29,8 @@ namespace {
 
 // rho of G functions per CTA, whose 8 warps are the 8 parts: in row-pair order
 // (G = 1, with offsets of type Off), or row by row for a B of mostly zero chunks.
-template <bool kPacked, bool kRows, int G, typename Off = int>
-__global__ void __launch_bounds__(256, 4) rho_kernel(const double *__restrict__ B, const double *__restrict__ D,
+template <bool kPacked, bool kRows, int G, int kCtas = 4, typename Off = int>
+__global__ void __launch_bounds__(256, kCtas) rho_kernel(const double *__restrict__ B, const double *__restrict__ D,
                                                      int naux, int nao, const uint32_t *__restrict__ mask,
                                                      double *__restrict__ rho, double *__restrict__ rho2) {
   __shared__ double part[8][G];
@@ -300,10 +300,16 @@ cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, doub
   // so functions share it while the SMs keep two CTAs (350 AOs: 700 functions 130
   // us one by one, 102 by two, 113 by four; 1050 functions 145 by two, 114 by four)
   const int group = !rows ? 1 : naux >= 1024 ? 4 : naux >= 304 ? 2 : 1;
+  // dense: a CTA a function, four or five of them an SM, whichever takes less: a wave of five
+  // is a quarter longer (152 SMs, 235 AOs and 705 functions: 60 us in two waves of four, 51 in
+  // one of five; packed, 435 and 1305: 275 and 245; 600 and 1800, three waves of either: 583 and
+  // 619).  At 48 registers 64-bit offsets suit the dense layout (435 and 1305: 252 us for 300) and
+  // 32-bit ones the packed (254 for 270); past 2^31 elements of a B_P they have to be 64-bit.
+  const long long sms = slice_gemm_grid(1 << 30);
+  const bool five = (naux + 5 * sms - 1) / (5 * sms) * 5 < (naux + 4 * sms - 1) / (4 * sms) * 4;
   auto kern = packed ? rho_kernel<true, false, 1> : rho_kernel<false, false, 1>;
-  // one B_P past 2^31 elements (at 32 bits everywhere else: 64-bit offsets cost a packed B
-  // 8 %, 587 -> 637 us at 600 AOs and 1800 functions)
-  if (nao > kRho32Nao) kern = packed ? rho_kernel<true, false, 1, long long> : rho_kernel<false, false, 1, long long>;
+  if (five) kern = packed ? rho_kernel<true, false, 1, 5> : rho_kernel<false, false, 1, 5, long long>;
+  if (nao > kRho32Nao) kern = packed ? rho_kernel<true, false, 1, 5, long long> : rho_kernel<false, false, 1, 5, long long>;
   if (rows && group == 4) kern = packed ? rho_kernel<true, true, 4> : rho_kernel<false, true, 4>;
   if (rows && group == 2) kern = packed ? rho_kernel<true, true, 2> : rho_kernel<false, true, 2>;
   if (rows && group == 1) kern = packed ? rho_kernel<true, true, 1> : rho_kernel<false, true, 1>;

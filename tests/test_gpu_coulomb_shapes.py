@@ -137,3 +137,27 @@ def test_energies_after_overlapping_calls(df):
     with ThreadPoolExecutor(4) as ex:
         list(ex.map(ask, streams))
     assert all(ctx.energy(D, J, K, rho) == want for _ in range(3))
+
+
+@pytest.mark.parametrize("naux", [608, 609, 760, 761, 1216, 1217, 1520])
+def test_rho_at_the_edges_of_whole_waves(df, naux):
+    """rho alone runs four or five CTAs an SM by the waves that naux takes (152 SMs: 608 and 760
+    CTAs a wave): the same bits on either side of each edge as beside the exchange GEMM, dense and
+    packed, and the FP64 sums within their rounding."""
+    nao = 35
+    B, C = _random(naux, naux, nao, 4)
+    D = torch.from_numpy(C @ C.T).cuda()
+    Bg = torch.from_numpy(B).cuda()
+    iu = torch.triu_indices(nao, nao, device="cuda")
+    Bp = Bg[:, iu[0], iu[1]].contiguous()
+    got = []
+    for packed in (False, True):
+        ctx = df.Context(nao, naux, 4, 2)
+        ctx.setup_packed(Bp) if packed else ctx.setup(Bg)
+        got.append(ctx.build_J(D)[1].cpu().numpy())
+        got.append(ctx.build_JK(D, torch.from_numpy(C).cuda(), 2)[1].cpu().numpy())
+    for r in got[1:]:
+        assert np.array_equal(r, got[0])
+    Dn = D.cpu().numpy()
+    ref, mag = np.einsum("pij,ij->p", B, Dn), np.einsum("pij,ij->p", np.abs(B), np.abs(Dn))
+    assert np.all(np.abs(got[0] - ref) <= 2 * nao * 2.0 ** -52 * mag)
