@@ -136,3 +136,16 @@ def test_slice_gram_product_shares_one_split(df, s):
     assert np.array_equal(out, O.emulated_matmul(A, A.T, s))      # T = 0 here: bit-exact
     Bt = At.clone()                                                 # a different pointer: two splits
     assert np.array_equal(df.emulated_gemm(At, Bt, s).cpu().numpy(), out)
+
+
+@pytest.mark.parametrize("M,N,K,nmod", [(100, 0, 2112, 6), (100, 0, 3110, 6), (257, 0, 4100, 14), (100, 0, 4161, 2),
+                                        (129, 100, 2112, 3), (129, 100, 3301, 8), (129, 100, 4200, 16)])
+def test_reconstruction_by_part_count(df, M, N, K, nmod):
+    # two, three and four K parts (a kernel each), of a Gram matrix (N = 0) and of two
+    # operands; fewer than 64 K tiles never take four
+    rng = np.random.default_rng(M + N + K + nmod)
+    A = _mat(rng, M, K, zero_row=1)
+    B = _mat(rng, N, K, spread=2.0) if N else A
+    Ag = torch.from_numpy(A).cuda()
+    out = df.emulated_gemm_crt(Ag, torch.from_numpy(B).cuda() if N else Ag, nmod).cpu().numpy()
+    assert np.array_equal(out, CO.emulated_gemm_crt(A, B, nmod))
