@@ -211,15 +211,16 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
       for (int h = 0; h < 4; ++h) res[h] = i == 0 ? residue_256(lo[h]) : residue_odd(lo[h], hi[h], t, i);
       uint16_t *dst = drow + (long long)i * pstride + c;
-      if (kInspect) {
-        for (int h = 0; h < nv; ++h) dst[h] = (uint16_t)(int16_t)(int)res[h];
-      } else if (nv == 4 && ((reinterpret_cast<uintptr_t>(dst) & 7) == 0)) {
-        // BF16 of an exact small integer: its FP32's upper half
-        *reinterpret_cast<uint2 *>(dst) = make_uint2(__byte_perm(__float_as_uint(res[0]), __float_as_uint(res[1]), 0x7632u),
-                                                     __byte_perm(__float_as_uint(res[2]), __float_as_uint(res[3]), 0x7632u));
-      } else {
-        for (int h = 0; h < nv; ++h) dst[h] = (uint16_t)(__float_as_uint(res[h]) >> 16);
-      }
+      // int16, or the BF16 of an exact small integer: its FP32's upper half
+      uint32_t v[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h)
+        v[h] = kInspect ? (uint32_t)(int)res[h] & 0xFFFFu : __float_as_uint(res[h]) >> 16;
+      if (nv == 4 && ((reinterpret_cast<uintptr_t>(dst) & 7) == 0))
+        *reinterpret_cast<uint2 *>(dst) =
+            make_uint2(__byte_perm(v[0], v[1], 0x5410u), __byte_perm(v[2], v[3], 0x5410u));
+      else
+        for (int h = 0; h < nv; ++h) dst[h] = (uint16_t)v[h];
     }
   }
 }
