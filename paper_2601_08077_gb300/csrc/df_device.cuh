@@ -11,6 +11,18 @@ namespace df {
 constexpr int kSMax = 8;            // digits per value
 constexpr int kBlock = 128;         // auxiliary functions per block
 
+// Truncation T of the int64 fixed-point sum of s slices and k products: |R| <= sum_g
+// (g+1) k 2^14 2^(8(s-1-g)) must stay below 2^61 after dropping T low bits.  T = 0
+// (exact) whenever that bound allows it.  In integers: a launch asks for nine of these,
+// and on a host whose long double is emulated (Arm) they took 7 us of a call that way.
+inline int fixed_point_shift(int s, long long k) {
+  unsigned __int128 bound = 0;
+  for (int g = 0; g < s; ++g) bound += ((unsigned __int128)(g + 1) * (unsigned __int128)k) << (14 + 8 * (s - 1 - g));
+  int bits = 0;
+  while (bits < 127 && ((unsigned __int128)1 << bits) < bound) ++bits;
+  return bits > 61 ? bits - 61 : 0;
+}
+
 #ifdef __CUDACC__
 // Row exponent from the bit pattern of max|row| (a non-negative double):
 // the smallest e with vmax < 127/128 * 2^e; 0 for a zero row.

@@ -204,7 +204,6 @@ int slice_gemm_grid(int nunits);
 // after limit_ns and sets bit 0 of *status (bit 1: it returned without the
 // abort path, which would be a defect).
 cudaError_t launch_wait_selftest(int *status, unsigned long long limit_ns, cudaStream_t st);
-int fixed_point_shift(int s, long long k);
 
 // rho_P for every P into rho (and rho2 if given), J from rho.
 // mask_mu (optional, block-sparse B): per mu, bit c set when some B_P mu nu

@@ -1355,18 +1355,6 @@ bool make_operand_maps(SgMaps *m, const SgOperand &a, const SgOperand &b, int nw
          make_tmap_bf16(&m->h, b.base, b.k, b.rows, b.planes, b.ld, b.plane_stride, nw / 2);
 }
 
-// Truncation T of the int64 fixed-point sum: |R| <= sum_g (g+1) K 2^14
-// 2^(8(s-1-g)) must stay below 2^61 after dropping T low bits.  T = 0 (exact)
-// whenever that bound allows it.
-int fixed_point_shift(int s, long long k) {
-  if (s <= 0) return 0;
-  long double bound = 0.0L;
-  for (int g = 0; g < s; ++g) bound += (long double)(g + 1) * (long double)k * 16384.0L * ldexpl(1.0L, 8 * (s - 1 - g));
-  int bits = 0;
-  while (ldexpl(1.0L, bits) < bound) ++bits;
-  return bits > 61 ? bits - 61 : 0;
-}
-
 void grid_params(SgParams *p, int mode, int M, int N, int K, int s) {
   std::memset(p, 0, sizeof(*p));
   p->mode = mode;
