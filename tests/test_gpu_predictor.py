@@ -54,6 +54,23 @@ def test_mlp_gradients_at_tile_edges(df, n):
     assert np.array_equal(g, g2) and loss == loss2
 
 
+@pytest.mark.parametrize("n", [2, 3, 4, 5, 28, 29, 61, 257])
+def test_mlp_gradients_at_warp_edges(df, n):
+    """A warp takes four rows of a tile: counts that leave its last rows, whole warps or a tile but
+    one row empty, with X at a four-byte boundary.  FP32 sums against FP64 as above."""
+    rng = np.random.default_rng(100 + n)
+    theta = (M.init_params(6) + 0.05 * rng.standard_normal(M.N_PARAMS)).astype(np.float32)
+    flat = rng.standard_normal(16 * n + 1).astype(np.float32)
+    y = rng.integers(0, 8, size=n)
+    net = df.MLP(theta)
+    Xg = torch.from_numpy(flat).cuda()[1:].view(n, 16)
+    g, loss = net.gradients(Xg, torch.from_numpy(y.astype(np.int32)).cuda())
+    X = flat[1:].reshape(n, 16).astype(np.float64)
+    ref = M.gradients(theta.astype(np.float64), X, y)
+    assert abs(loss - M.loss(theta.astype(np.float64), X, y)) < 1e-5
+    assert np.max(np.abs(g - ref)) <= 1e-5 + 1e-4 * np.max(np.abs(ref))
+
+
 def test_adam_steps_match_oracle(df):
     """Three df_mlp_train_step calls against the oracle's Adam (beta 0.9 / 0.999, bias
     correction) on the oracle's FP64 gradients, element by element.  The first update is
