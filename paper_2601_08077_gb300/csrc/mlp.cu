@@ -96,6 +96,10 @@ __global__ void __launch_bounds__(256) mlp_forward_kernel(const float *__restric
 constexpr int kTileRows = 32;
 constexpr int kMaxParts = 256;    // CTAs, each with one partial gradient
 constexpr int kPart = kNParams + 1;  // and its part of the loss
+// Partial gradients that a network brings along: with its parameters below 1 MB, up to which
+// cudaMalloc takes 1.5 us and past which 55 (a network with all 256 took 110 us to create,
+// 40 before it held any).
+constexpr int kOwnParts = 40;
 constexpr int kHP = kH + 4;       // activation pitch: rows of a tile on different banks, 16-byte aligned
 
 struct alignas(16) MlpTile {
@@ -525,7 +529,8 @@ __global__ void __launch_bounds__(256) check_exponents_kernel(const int *__restr
 
 struct df_mlp {
   float *P = nullptr, *G = nullptr, *m1 = nullptr, *m2 = nullptr, *loss = nullptr;
-  float *part = nullptr;  // [kMaxParts][kPart] partial gradients
+  float *part = nullptr;  // [kOwnParts][kPart] partial gradients
+  float *more = nullptr;  // [kMaxParts][kPart], allocated for the first larger training set
   int t = 0;
 };
 
@@ -535,9 +540,10 @@ df_status df_mlp_create(df_mlp **out) {
   if (!out) return DF_ERR_ARG;
   df_mlp *m = new (std::nothrow) df_mlp();
   if (!m) return DF_ERR_OOM;
-  // one allocation: P, the two moments, G, the loss, the partial gradients
+  // one allocation: P, the two moments, G, the loss, the first partial gradients
   const size_t np = (kNParams + 63) / 64 * 64;
-  cudaError_t e = cudaMalloc(&m->P, sizeof(float) * (4 * np + 64 + (size_t)kMaxParts * kPart));
+  static_assert(sizeof(float) * (4 * (kNParams + 63) / 64 * 64 + 64 + kOwnParts * kPart) <= 1 << 20, "a cheap allocation");
+  cudaError_t e = cudaMalloc(&m->P, sizeof(float) * (4 * np + 64 + (size_t)kOwnParts * kPart));
   if (e == cudaSuccess) {
     m->m1 = m->P + np;
     m->m2 = m->P + 2 * np;
@@ -557,6 +563,7 @@ df_status df_mlp_create(df_mlp **out) {
 void df_mlp_destroy(df_mlp *m) {
   if (!m) return;
   cudaFree(m->P);
+  cudaFree(m->more);
   delete m;
 }
 
@@ -594,9 +601,27 @@ df_status df_mlp_gradients(df_mlp *m, const float *X, const int *y, int n, float
   if (e != cudaSuccess) return DF_ERR_CUDA;
   const int ntiles = (n + kTileRows - 1) / kTileRows;
   const int parts = ntiles < kMaxParts ? ntiles : kMaxParts;
-  mlp_backward_kernel<<<parts, 256, sizeof(MlpTile), st>>>(m->P, X, y, n, m->part);
-  mlp_sum_kernel<<<(kPart + 31) / 32, 256, 0, st>>>(m->part, parts, m->G, m->loss);
+  float *part = parts <= kOwnParts ? m->part : m->more, *recorded = nullptr;
+  if (!part) {
+    const size_t bytes = sizeof(float) * (size_t)kMaxParts * kPart;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing(st, &cs);
+    if (e == cudaSuccess && cs != cudaStreamCaptureStatusNone) {
+      e = cudaMallocAsync(&recorded, bytes, st);  // no cudaMalloc while recording: the graph's own
+      part = recorded;
+    } else if (e == cudaSuccess) {
+      e = cudaMalloc(&m->more, bytes);
+      part = m->more;
+    }
+    if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? DF_ERR_OOM : DF_ERR_CUDA;
+  }
+  mlp_backward_kernel<<<parts, 256, sizeof(MlpTile), st>>>(m->P, X, y, n, part);
+  mlp_sum_kernel<<<(kPart + 31) / 32, 256, 0, st>>>(part, parts, m->G, m->loss);
   e = cudaGetLastError();
+  if (recorded) {
+    const cudaError_t ef = cudaFreeAsync(recorded, st);
+    if (e == cudaSuccess) e = ef;
+  }
   if (e != cudaSuccess) return DF_ERR_CUDA;
   if (grad_host) e = cudaMemcpyAsync(grad_host, m->G, sizeof(float) * kNParams, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && loss_host) e = cudaMemcpyAsync(loss_host, m->loss, sizeof(float), cudaMemcpyDeviceToHost, st);

@@ -71,6 +71,31 @@ def test_mlp_gradients_at_warp_edges(df, n):
     assert np.max(np.abs(g - ref)) <= 1e-5 + 1e-4 * np.max(np.abs(ref))
 
 
+@pytest.mark.parametrize("n", [1280, 1281])
+def test_mlp_steps_recorded_in_a_graph(df, n):
+    """Forty partial gradients come with the network, a larger set's are allocated with its first
+    gradients, also when that first call is being recorded: a replayed first step leaves the bits
+    of a direct one."""
+    rng = np.random.default_rng(n)
+    theta = M.init_params(8).astype(np.float32)
+    Xg = torch.from_numpy(rng.standard_normal((n, 16)).astype(np.float32)).cuda()
+    yg = torch.from_numpy(rng.integers(0, 8, size=n).astype(np.int32)).cuda()
+    direct, net = df.MLP(theta), df.MLP(theta)
+    direct.train_step(Xg, yg, 1e-3)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        net.train_step(Xg, yg, 1e-3)
+    torch.cuda.synchronize()
+    assert np.array_equal(net.get_params(), theta)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(net.get_params(), direct.get_params())
+    assert not np.array_equal(net.get_params(), theta)
+    g0, g1 = direct.gradients(Xg, yg), net.gradients(Xg, yg)
+    assert np.array_equal(g0[0], g1[0]) and g0[1] == g1[1]
+
+
 def test_adam_steps_match_oracle(df):
     """Three df_mlp_train_step calls against the oracle's Adam (beta 0.9 / 0.999, bias
     correction) on the oracle's FP64 gradients, element by element.  The first update is
