@@ -187,7 +187,11 @@ __global__ void __launch_bounds__(256) setup_rows_kernel(const double *__restric
 // Rows of B from its packed layout (per P the upper triangle row by row,
 // nao (nao + 1) / 2 values): output row r = (P', mu), P = perm[P'] (or P'),
 // holds B_P mu nu for every nu (nu < mu read at the transposed position).
-// One warp per row; the same two passes and digits as split_rows_bf16_kernel.
+// One warp per row; the same two passes and digits as split_rows_bf16_kernel, two columns a
+// lane (the transposed reads are a value each).  120 atoms, 600 AOs, six planes: the setup took
+// 5.05 ms with the digits in arrays and a conversion each, 4.27 with their bytes placed in
+// FP32; a screened chain of 60 atoms, whose zeros cost as much as any value since the rounding
+// has no branches, 1.19 and 1.09.
 __global__ void __launch_bounds__(256) split_rows_packed_kernel(const double *__restrict__ Bp, long long rows,
                                                                 int nao, int nslices, int *__restrict__ exps,
                                                                 uint16_t *__restrict__ digits, long long dld,
@@ -213,29 +217,16 @@ __global__ void __launch_bounds__(256) split_rows_packed_kernel(const double *__
   const int e = exponent_from_max_bits_dev(m);
   if (lane == 0) exps[r] = e;
   uint16_t *drow = digits + r * dld;
+  // a pair past an odd row's end gets zero digits (rows of a multiple of 8 digits)
   for (int c = 2 * lane; c < nao; c += 64) {
-    int d0[kSMax], d1[kSMax];
-    balanced_digits(scaled_rne((uint64_t)__double_as_longlong(at(c)), e), d0);
-    const bool two = c + 1 < nao;
-    if (two) {
-      balanced_digits(scaled_rne((uint64_t)__double_as_longlong(at(c + 1)), e), d1);
-    } else {
+    const uint64_t b1 = c + 1 < nao ? (uint64_t)__double_as_longlong(at(c + 1)) : 0ull;
+    const long long M0 = scaled_rne((uint64_t)__double_as_longlong(at(c)), e) + kDigitBias;
+    const long long M1 = scaled_rne(b1, e) + kDigitBias;
 #pragma unroll
-      for (int t = 0; t < kSMax; ++t) d1[t] = 0;
-    }
-#pragma unroll
-    for (int t = 0; t < kSMax; ++t) {
-      if (t < nslices) {
-        const uint32_t pk = (uint32_t)int_to_bf16_bits(d0[t]) | ((uint32_t)int_to_bf16_bits(d1[t]) << 16);
-        uint16_t *dst = drow + (long long)t * plane_stride + c;
-        if (two && ((reinterpret_cast<uintptr_t>(dst) & 3) == 0)) {
-          *reinterpret_cast<uint32_t *>(dst) = pk;
-        } else {
-          dst[0] = (uint16_t)(pk & 0xFFFF);
-          if (two) dst[1] = (uint16_t)(pk >> 16);
-        }
-      }
-    }
+    for (int t = 0; t < kSMax; ++t)
+      if (t < nslices)
+        *reinterpret_cast<uint32_t *>(drow + (long long)t * plane_stride + c) =
+            bf16x2_of(digit_f32(M0, t), digit_f32(M1, t));
   }
 }
 

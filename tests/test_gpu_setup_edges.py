@@ -122,3 +122,22 @@ def test_refused_order_leaves_the_context_as_it_was(df):
         J1, rho1 = ctx.build_J(D)
         K1, _ = ctx.build_K(C, 3)
         assert torch.equal(J1, J) and torch.equal(rho1, rho) and torch.equal(K1, K)
+
+
+@pytest.mark.parametrize("nao", [1, 2, 15, 16, 17, 33, 129])
+def test_packed_digits_at_row_ends(df, nao):
+    # rows that end inside a lane's pair, inside a digit row's padding or fill it: K and the
+    # masks of a packed B are the dense ones, bit for bit
+    B = _tensor(50 + nao, 5, nao)
+    B[:, nao // 2, :] = 0.0
+    B[:, :, nao // 2] = 0.0
+    Bg = torch.from_numpy(B).cuda()
+    iu = torch.triu_indices(nao, nao, device="cuda")
+    C = torch.from_numpy(np.random.default_rng(nao).standard_normal((nao, 3))).cuda()
+    perm = [3, 0, 4, 1, 2]
+    for s in (3, 6):
+        dense, packed = df.Context(nao, 5, 3, s), df.Context(nao, 5, 3, s)
+        dense.setup(Bg, perm)
+        packed.setup_packed(Bg[:, iu[0], iu[1]].contiguous(), perm)
+        assert dense.sparsity() == packed.sparsity()
+        assert torch.equal(dense.build_K(C, s)[0], packed.build_K(C, s)[0])
