@@ -62,3 +62,55 @@ def test_exchange_at_tile_edges(df, naux, nao, nocc, s):
         assert np.array_equal(got[1], ref)
     else:
         assert np.max(np.abs(got[1] - ref)) <= 1e-14 * np.max(np.abs(ref))
+
+
+def _both_builds(df, naux, nao, nocc, s, modes):
+    """J, rho and K of build_JK (512 threads, the Coulomb passes in the GEMMs' spare warps) under
+    each pair mode, and of the separate builds."""
+    rng = np.random.default_rng(naux * 1000 + nao + 1)
+    B = rng.standard_normal((naux, nao, nao)) * np.exp2(rng.integers(-8, 1, (naux, nao, nao)))
+    B = np.triu(B) + np.triu(B, 1).transpose(0, 2, 1)
+    D = rng.standard_normal((nao, nao))
+    Bg, Dg = torch.from_numpy(B).cuda(), torch.from_numpy(D + D.T).cuda()
+    Cg = torch.from_numpy(rng.standard_normal((nao, nocc)) * np.exp2(rng.integers(-4, 1, (1, nocc)))).cuda()
+    got = []
+    for mode in modes:
+        ctx = df.Context(nao, naux, nocc, s)
+        if mode is not None:
+            ctx.set_cluster_pairs(mode)
+        ctx.setup(Bg)
+        J, rho = ctx.build_J(Dg)
+        K, _ = ctx.build_K(Cg, s)
+        got.append([t.clone() for t in (J, rho, K)])
+        J, rho, K, _ = ctx.build_JK(Dg, Cg, s)
+        ctx.sync_status()
+        got.append([J, rho, K])
+    return got
+
+
+@pytest.mark.parametrize("naux,nao,nocc,s", SHAPES)
+def test_coulomb_beside_the_gemms_at_tile_edges(df, naux, nao, nocc, s):
+    # both GEMMs on single CTAs, the first on pairs, both on pairs
+    got = _both_builds(df, naux, nao, nocc, s, (0, 1, 2))
+    for other in got[1:]:
+        for x, y in zip(got[0], other):
+            assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("nao", [769, 800, 897])
+def test_second_gemm_on_pairs_by_default(df, nao):
+    # from 7 AO tile rows on (nao > 768) the default pairs the second GEMM too; an odd row
+    # count leaves a pair whose second tile lies past the last row
+    got = _both_builds(df, 20, nao, 9, 3, (None, 0))
+    for other in got[1:]:
+        for x, y in zip(got[0], other):
+            assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("M", [1930, 2060])
+def test_product_of_many_row_tiles_on_pairs(df, M):
+    # 16 tile rows, and 17, whose last CTA lies wholly past M; odd N, a ragged K
+    rng = np.random.default_rng(M)
+    A, B = rng.standard_normal((M, 70)), rng.standard_normal((67, 70))
+    got = df.emulated_gemm(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), 3).cpu().numpy()
+    assert np.array_equal(got, O.emulated_matmul(A, B.T, 3))
