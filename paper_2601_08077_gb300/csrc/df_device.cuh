@@ -117,6 +117,53 @@ __device__ __forceinline__ int row_exponent(uint32_t mh, int lane, int cols, Bit
   return exponent_from_max_bits_dev(m);
 }
 
+// R to 53 bits, ties to even, for |R| < 2^61.
+__device__ __forceinline__ long long round53(long long R) {
+  const int hi = (int)(R >> 32);
+  const uint32_t a = (uint32_t)(hi ^ (hi >> 31));  // |R|'s (or |R| - 1's) high word
+  if (a >= (1u << 21)) {
+    const int sh = 11 - __clz((int)a);  // bits to drop; exact powers of two have none set
+    const long long lsb = (R >> sh) & 1;
+    R += ((1ll << sh) >> 1) - 1 + lsb;
+    R &= ~((1ll << sh) - 1);
+  }
+  return R;
+}
+
+// RNE(R 2^-r) for r >= 1, |R| < 2^61.
+__device__ __forceinline__ long long rne_down(long long R, int r) {
+  if (r >= 63) return 0;
+  return (R + ((1ll << (r - 1)) - 1) + ((R >> r) & 1)) >> r;
+}
+
+// The X split's fast path for one element: N = RNE(fl64(r 2^k) 2^(63-g)), sh = k + 63 - g, for
+// a row whose exponent bound is g.  kRound: |r| may have more than 53 bits.  top: the largest
+// |N| so far (|N| - 1 of a negative one), its top 31 bits; lost: not zero once a shift pushed
+// bits out of 64.
+template <bool kRound>
+__device__ __forceinline__ long long x_fixed(long long r, int sh, int &top, int &lost) {
+  if (kRound) r = round53(r);
+  const int hi = (int)(r >> 32);
+  if ((unsigned)sh < 32u) {
+    lost |= (hi >> (31 - sh)) ^ (hi >> 31);  // bits that the shift pushes out
+    r <<= sh;
+  } else if (sh < 0) {
+    r = rne_down(r, -sh);
+  } else {
+    lost |= sh > 62 ? (int)(r != 0) : (int)((r >> (63 - sh)) != (r >> 63));
+    r = sh > 62 ? 0 : r << sh;
+  }
+  const int h = (int)(r >> 32);
+  top = max(top, h ^ (h >> 31));
+  return r;
+}
+
+// Whether the bound g is the row's exponent and its N are right: attained (some |N| >= 2^62),
+// no bits lost, and not within one unit of the 31 bits of 127/128 2^g.
+__device__ __forceinline__ bool x_bound_is_exponent(int top, int lost) {
+  return lost == 0 && top >= (1 << 30) && top < (127 << 24) - 1;
+}
+
 // Balanced digits of N: d[7..1] in [-128,127] from the bottom, d[0] the rest.
 // Taking them from the bottom, digit k is ((N_k + 128) mod 256) - 128 and
 // N_{k+1} = floor((N_k + 128) / 256), so with M = N + 128 (1 + 256 + ... +

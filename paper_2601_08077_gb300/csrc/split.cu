@@ -358,25 +358,6 @@ struct XRow {
   int nP, nocc, kpad;
 };
 
-// R to 53 bits, ties to even, for |R| < 2^61.
-__device__ __forceinline__ long long round53(long long R) {
-  const int hi = (int)(R >> 32);
-  const uint32_t a = (uint32_t)(hi ^ (hi >> 31));  // |R|'s (or |R| - 1's) high word
-  if (a >= (1u << 21)) {
-    const int sh = 11 - __clz((int)a);  // bits to drop; exact powers of two have none set
-    const long long lsb = (R >> sh) & 1;
-    R += ((1ll << sh) >> 1) - 1 + lsb;
-    R &= ~((1ll << sh) - 1);
-  }
-  return R;
-}
-
-// RNE(R 2^-r) for r >= 1, |R| < 2^61.
-__device__ __forceinline__ long long rne_down(long long R, int r) {
-  if (r >= 63) return 0;
-  return (R + ((1ll << (r - 1)) - 1) + ((R >> r) & 1)) >> r;
-}
-
 // Exact path of a row: the exact magnitude keys of its elements (bit length +
 // scale, then the normalised mantissa; rounding is monotone, so only the
 // winning element is rounded), the exponent they give, then the digits.
@@ -502,27 +483,12 @@ __global__ void __launch_bounds__(kSplitXThreads, 5)
           ++pl;
         }
       }
-      auto fixed = [&](long long r, int sh) -> long long {
-        if (kRound) r = round53(r);
-        const int hi = (int)(r >> 32);
-        if ((unsigned)sh < 32u) {
-          lost |= (hi >> (31 - sh)) ^ (hi >> 31);  // bits that the shift pushes out
-          r <<= sh;
-        } else if (sh < 0) {
-          r = rne_down(r, -sh);
-        } else {
-          lost |= sh > 62 ? (int)(r != 0) : (int)((r >> (63 - sh)) != (r >> 63));
-          r = sh > 62 ? 0 : r << sh;
-        }
-        const int h = (int)(r >> 32);
-        top = max(top, h ^ (h >> 31));
-        return r + kDigitBias;
-      };
 #pragma unroll
       for (int r = 0; r < kU; ++r) {
         const int q = q0 + r * kSplitXThreads;
         if (q >= pairs) break;
-        const long long M0 = fixed(v[r].x, sx[r]), M1 = fixed(v[r].y, sy[r]);
+        const long long M0 = x_fixed<kRound>(v[r].x, sx[r], top, lost) + kDigitBias;
+        const long long M1 = x_fixed<kRound>(v[r].y, sy[r], top, lost) + kDigitBias;
 #pragma unroll
         for (int t = 0; t < S; ++t) out[q + t * pl2] = bf16x2_of(digit_f32(M0, t), digit_f32(M1, t));
       }
@@ -534,8 +500,7 @@ __global__ void __launch_bounds__(kSplitXThreads, 5)
       if (lost) atomicOr(&sh_lost, lost);
     }
     __syncthreads();
-    // attained, and not within one unit of the 31 bits of 127/128 2^g
-    if (sh_lost == 0 && sh_top >= (1 << 30) && sh_top < (127 << 24) - 1) {
+    if (x_bound_is_exponent(sh_top, sh_lost)) {
       if (threadIdx.x == 0) eX[b * nao + mu] = g;
       return;
     }
