@@ -309,13 +309,18 @@ __device__ __forceinline__ void coulomb_items(const CoulombWork &w) {
   }
 }
 
-// A group of four has nao <= 16384 (rho_work); one function at a time takes any nao.
+// A group of four has nao <= 16384 (rho_work), a B in row order nao <= 2048; one function at
+// a time takes any nao (64-bit offsets throughout cost it 2 to 3 %: 60 functions of 2600 AOs
+// beside the first exchange GEMM, the whole step 3.19 -> 3.30 ms).
 template <bool kPacked, bool kRows>
 __device__ __forceinline__ void rho_any_group(const CoulombWork &w) {
-  if (w.group == 4)
+  if (w.group == 4) {
     rho_items<kPacked, kRows, 4, 3, int>(w);
-  else
-    rho_items<kPacked, kRows, 1, 8, long long>(w);
+  } else if (kRows || w.nao <= kRho32Nao) {
+    rho_items<kPacked, kRows, 1, 8, int>(w);
+  } else {
+    rho_items<kPacked, false, 1, 8, long long>(w);
+  }
 }
 
 template <int kKind>
