@@ -36,8 +36,13 @@ import numpy as np  # noqa: E402
 
 METRIC = "DF K-build effective FP64 TFLOP/s, INT8-adaptive vs native FP64, max|dK|<=1e-10"
 UNIT = "TFLOP/s"
-LAUNCHES_PER_STEP = 7      # split C, GEMM1 (with rho), split X, GEMM2 (with J), reduce, density change, energy
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
+
+
+def launches_per_step(jk_overlap):
+    """Kernels of one step: C split, first GEMM, X split, second GEMM, reduction, density change and
+    energies; rho and J run inside the GEMMs, or (jk_overlap 0) as two kernels of their own."""
+    return 7 if jk_overlap else 9
 
 
 def parse():
@@ -64,7 +69,8 @@ def parse():
                     help="1..4 (alike) run rho and J beside the exchange GEMMs in the J + K build (df_build_JK); "
                          "0 runs J, then K, in one stream")
     ap.add_argument("--cluster-pairs", type=int, choices=[0, 1, 2], default=1,
-                    help="slice GEMMs on CTA pairs (cta_group::2): 0 never, 1 the first GEMM, 2 both GEMMs")
+                    help="slice GEMMs on CTA pairs (cta_group::2): 0 never, 1 the first GEMM and, from 7 AO tile "
+                         "rows (nao > 768) on, the second, 2 both GEMMs")
     return ap.parse_args()
 
 
@@ -736,15 +742,16 @@ def main():
     value = FK * world / (ms * 1e-3) / 1e12
     # roofline of the dominant kernel (the slice GEMM launch with the largest share)
     pk, src = peaks()
-    g1_ms = k_phases["gemm1"][0] / max(1, k_phases["gemm1"][1])  # the exchange build alone: no rho and J inside
-    g2_ms = k_phases["gemm2"][0] / max(1, k_phases["gemm2"][1])
+    # from the exchange build alone (no rho and J inside); the timed step's own beside it
+    g1_ms, g2_ms = (k_phases[g][0] / max(1, k_phases[g][1]) for g in ("gemm1", "gemm2"))
     pairs = s * (s + 1) // 2
     g1_flops = pairs * 2.0 * w.nocc * w.naux * w.nao * w.nao
     g2_flops = pairs * 2.0 * (w.nao * (w.nao + 1) / 2) * w.naux * w.nocc
     if g1_ms >= g2_ms:
-        kname, kms, kfl = "slice_gemm (X = B C)", g1_ms, g1_flops
+        kname, kms, kfl, phase = "slice_gemm (X = B C)", g1_ms, g1_flops, "gemm1"
     else:
-        kname, kms, kfl = "slice_gemm (K_b = X_b X_b^T)", g2_ms, g2_flops
+        kname, kms, kfl, phase = "slice_gemm (K_b = X_b X_b^T)", g2_ms, g2_flops, "gemm2"
+    step_ms = phases[phase][0] / max(1, phases[phase][1])
     peak = float(pk.get("bf16_tflops_sustained", FALLBACK_PEAKS["bf16_tflops_sustained"]))
     achieved = kfl / (kms * 1e-3) / 1e12
     out = {
@@ -761,9 +768,15 @@ def main():
                    "parallelism": "replicas" if world > 1 else "single"},
         "e2e": {"value": FK / (ms_e2e * 1e-3) / 1e12 * world, "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "ms_per_step": ms_e2e},
-        "gpu_launches": LAUNCHES_PER_STEP * args.steps,
+        "gpu_launches": launches_per_step(args.jk_overlap) * args.steps,
         "roofline": {"bound": "tensor", "kernel": kname, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                     "frac": achieved / peak,
+                     "frac": achieved / peak, "ms": kms,
+                     "region": "the exchange build alone (df_build_K), timed after the steps",
+                     "in_step": {"ms": step_ms, "achieved": kfl / (step_ms * 1e-3) / 1e12,
+                                 "frac": kfl / (step_ms * 1e-3) / 1e12 / peak,
+                                 "region": "the timed steps (df_build_JK): %s" % (
+                                     "the launch carries %s too" % ("rho" if phase == "gemm1" else "J")
+                                     if args.jk_overlap else "the same kernel, rho and J before it")},
                      "traffic": recorded_traffic(kname, w.name, s, args.cluster_pairs),
                      "peak_source": "bf16_tflops_sustained (%s)" % src,
                      "algorithmic": "s(s+1)/2 slice-pair products x 2 flops per multiply-add, no padding"},

@@ -74,3 +74,8 @@ def test_oracle_gate_on_the_small_molecule():
     Kbad = K_full.copy()
     Kbad[3, 5] += 2e-10 * np.max(np.abs(K_full))
     assert not b.oracle_gate(Kbad, J_full, (EJ, 0.0, EK), K, J, D)["gate_vs_oracle"]
+
+
+def test_launches_per_step_follow_the_overlap():
+    b = _bench()
+    assert [b.launches_per_step(o) for o in range(5)] == [9, 7, 7, 7, 7]
