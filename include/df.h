@@ -306,9 +306,8 @@ df_status df_batch_build_K(df_batch *b, const double *const *C_dev, const int *n
  * rho goes to each context's internal buffer. */
 df_status df_batch_build_J(df_batch *b, const double *const *D_dev, double *const *J_dev, void *stream);
 /* Autotuner: times, on this batch, every combination of the first GEMM's
- * tile (CTA-pair 256 x 128 tiles with the (P, mu) rows on the MMA's M side,
- * possible when every molecule's orbitals fit one 128-row tile, or
- * single-CTA 128 x 128 tiles with the orbitals on M), the K-split cap of the
+ * tile (256 (P, mu) rows on CTA pairs, offered when every molecule has at
+ * most 128 orbitals, or 128 rows on single CTAs), the K-split cap of the
  * second GEMM (1, 2, 4 or 8, at most the context's own split) and the
  * molecule order of the unit lists (as given, or most expensive first), and
  * keeps the fastest.  choice (host, 3 ints, may be NULL): [0] K-split cap,

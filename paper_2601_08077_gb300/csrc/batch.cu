@@ -108,7 +108,8 @@ df_status build_tables(df_batch *b, const int *nocc) {
   std::vector<int> o1(n + 1, 0), o2(n + 1, 0);
   const std::vector<int> ord = unit_order(b, nocc);
   b->nsplit.assign(n, 1);
-  // the first GEMM runs on CTA pairs when every molecule's orbitals fit one tile
+  // the first GEMM runs on CTA pairs when every molecule's orbitals fit one tile of 128 (the rule,
+  // not the kernel, needs that: its pairs are row tiles of one block whatever the orbitals)
   b->pairs1 = b->tile1 == 1;
   for (int i = 0; i < n; ++i) b->pairs1 = b->pairs1 && b->ctx[i]->pair_mode >= 1 && nocc[i] <= df::kTile;
   for (int k = 0; k < n; ++k) {
@@ -367,7 +368,7 @@ df_status df_batch_autotune(df_batch *b, const double *const *C, const int *nocc
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  // the first GEMM's CTA-pair tiles exist only when every molecule's orbitals fit one tile
+  // the first GEMM's CTA-pair tiles are offered when every molecule's orbitals fit one tile
   bool pairs_possible = true;
   for (size_t i = 0; i < b->ctx.size(); ++i)
     pairs_possible = pairs_possible && b->ctx[i]->pair_mode >= 1 && nocc[i] <= df::kTile;

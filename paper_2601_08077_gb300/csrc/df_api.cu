@@ -404,7 +404,6 @@ df_status df_create(df_ctx **out, int nao, int naux, int nocc_max, int s_max) {
       }
     }
     c->nsplit = best;
-    c->nsm = nsm;
   }
   if (e == cudaSuccess) e = alloc(c, &c->Rp, (size_t)c->nblk * c->nsplit * nao * nao);
   if (e == cudaSuccess) e = alloc(c, &c->rho, (size_t)naux);

@@ -27,7 +27,6 @@ struct df_ctx {
   int *jk_work = nullptr;
   double *rho_part = nullptr;  // [8][naux]
   int jk_ctas = 4;
-  int nsm = 0;
   double *epart = nullptr;
   double *E = nullptr;
   int *sblk = nullptr;      // device per-block slice counts

@@ -40,7 +40,8 @@
 //   warp 0      TMA producer: 64-wide BF16 boxes of A_t and the stacked B
 //               digits, 128B swizzle, into a ring guarded by mbarriers;
 //   warp 1      TMEM allocation and the single-thread tcgen05.mma issuer;
-//   warps 2, 3  idle (they give their registers to the epilogue: setmaxnreg);
+//   warps 2, 3  idle (they give their registers to the epilogue: setmaxnreg), or, in the
+//               512-thread form with warps 12 to 15, a Coulomb pass (kHelp, below);
 //   warps 4..11 epilogue; warp w reads TMEM lanes 32*(w%4)..+31 (tile rows)
 //               and half (w-4)/4 of each digit's columns.
 // The producer's and the issuer's loops bound the kernel when they are written
@@ -394,7 +395,7 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&a)[32]) {
                  : "memory");
 }
 
-// 16-wide K steps of K tile kt of `ktot` when the K range has kvalid values.
+// 16-wide K steps of the last K tile of a range of kvalid values.
 __device__ __forceinline__ int tail_steps(int kvalid) {
   const int rem = (kvalid - 1) % kKTile + 1;
   return (rem + 15) >> 4;
@@ -425,7 +426,7 @@ __device__ __forceinline__ Unit kpart_unit(const SgParams &p, int i, int j, int 
   return w;
 }
 
-// Tile (mt, nt) of the grid layouts (kLayoutGrid, kLayoutCrt).
+// Tile (mt, nt) of a stand-alone product (kModeRaw, kModeGemm, kModeMod).
 __device__ __forceinline__ Unit grid_unit(const SgParams &p, int mt, int nt) {
   Unit w;
   w.m0 = mt * kTile;
@@ -1188,7 +1189,7 @@ __global__ void __launch_bounds__(kHelp ? kThreadsHelp : kThreads, 1)
           };
           auto add = [&](int g, auto h_c, const uint32_t (&a)[32]) {
             constexpr int h = decltype(h_c)::value;
-            const int sh = kMode == kModeRaw ? 0 : 8 * (s - 1 - g) - T;
+            [[maybe_unused]] const int sh = kMode == kModeRaw ? 0 : 8 * (s - 1 - g) - T;
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
               if (32 * h + 16 * i >= hw) break;
