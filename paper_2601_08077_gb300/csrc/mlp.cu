@@ -7,6 +7,8 @@
 //   W1 [64][16], b1 [64], W2 [64][64], b2 [64], W3 [8][64], b3 [8].
 #include "df_ctx.h"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -15,6 +17,8 @@
 #include <vector>
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int kIn = 16, kH = 64, kOut = 8;
 constexpr int oW1 = 0, oB1 = oW1 + kH * kIn, oW2 = oB1 + kH, oB2 = oW2 + kH * kH, oW3 = oB2 + kH,
@@ -78,7 +82,7 @@ __global__ void __launch_bounds__(256) mlp_forward_kernel(const float *__restric
   }
 }
 
-// Gradients of the mean cross-entropy (labels y in 0..7).  A CTA takes tiles of
+// Gradients of the summed cross-entropy (labels y in 0..7; the sum kernel divides by n).  A CTA takes tiles of
 // 32 rows with the weights and the tile's activations in shared memory; every
 // thread owns a fixed part of the gradient (16 entries of W2, 4 of W1, 2 of W3)
 // and keeps it in registers over all its tiles, so a CTA writes one partial
@@ -94,12 +98,15 @@ __global__ void __launch_bounds__(256) mlp_forward_kernel(const float *__restric
 // a tile took 21.5 us, which made a step on one row slower, 32 us, than the kernel with
 // the atomics, 20; now 8.7 and 18.5.)
 constexpr int kTileRows = 32;
-constexpr int kMaxParts = 256;    // CTAs, each with one partial gradient
-constexpr int kPart = kNParams + 1;  // and its part of the loss
-// Partial gradients that a network brings along: with its parameters below 1 MB, up to which
-// cudaMalloc takes 1.5 us and past which 55 (a network with all 256 took 110 us to create,
-// 40 before it held any).
+constexpr int kPart = kNParams + 1;  // a partial gradient and its part of the loss
+// Partial gradients a network holds: with its parameters below 1 MB, up to which cudaMalloc
+// takes 1.5 us and past which 55 (with 256 of them a network took 110 us to create, 40 before
+// it held any).  More tiles than that run in clusters of 8 CTAs, each of which adds its
+// CTAs' gradients through distributed shared memory and writes one partial.
 constexpr int kOwnParts = 40;
+constexpr int kCluster = 8;
+constexpr int kMaxClusters = 32;  // 256 CTAs
+static_assert(kMaxClusters <= kOwnParts, "a partial gradient per cluster");
 constexpr int kHP = kH + 4;       // activation pitch: rows of a tile on different banks, 16-byte aligned
 
 struct alignas(16) MlpTile {
@@ -107,6 +114,7 @@ struct alignas(16) MlpTile {
   float x[kTileRows][kIn], h1[kTileRows][kHP], h2[kTileRows][kHP], d1[kTileRows][kHP], d2[kTileRows][kHP];
   float z[kTileRows][kOut], dz[kTileRows][kOut], loss[kTileRows];
 };
+static_assert(kPart <= kTileRows * (kIn + 4 * kHP), "a CTA's gradient takes the place of its activations");
 
 __device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 
@@ -142,6 +150,8 @@ __device__ __forceinline__ void put4(float *out, const float (&a)[4][2], const f
   }
 }
 
+// kGroups: clusters of kCluster CTAs, one partial gradient each; else one a CTA.
+template <bool kGroups>
 __global__ void __launch_bounds__(256) mlp_backward_kernel(const float *__restrict__ P, const float *__restrict__ X,
                                                            const int *__restrict__ y, int n,
                                                            float *__restrict__ part) {
@@ -180,7 +190,6 @@ __global__ void __launch_bounds__(256) mlp_backward_kernel(const float *__restri
   const int w1j = tid >> 2, w1k = (tid & 3) * 4;
   const int w3c = tid >> 5, w3k = (tid & 31) * 2;
   float g2[4][4] = {}, g1[4] = {}, g3[2] = {}, gb = 0.f, loss = 0.f;
-  const float inv_n = 1.f / (float)n;
   const int ntiles = (n + kTileRows - 1) / kTileRows;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int row0 = tile * kTileRows, rows = min(kTileRows, n - row0);
@@ -228,9 +237,9 @@ __global__ void __launch_bounds__(256) mlp_backward_kernel(const float *__restri
 #pragma unroll
       for (int c = 0; c < kOut; ++c) {
         if (c == yc) py = p[c];
-        s.dz[r0 + lane][c] = valid ? (p[c] - (c == yc ? 1.f : 0.f)) * inv_n : 0.f;
+        s.dz[r0 + lane][c] = valid ? p[c] - (c == yc ? 1.f : 0.f) : 0.f;
       }
-      if (valid) loss += -logf(fmaxf(py, 1e-30f)) * inv_n;
+      if (valid) loss -= logf(fmaxf(py, 1e-30f));
     }
     __syncwarp();
     start(nullptr);
@@ -270,6 +279,10 @@ __global__ void __launch_bounds__(256) mlp_backward_kernel(const float *__restri
     }
   }
   float *G = part + (long long)blockIdx.x * kPart;
+  if constexpr (kGroups) {
+    __syncthreads();  // the last tile is used up
+    G = &s.x[0][0];
+  }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
 #pragma unroll
@@ -291,28 +304,42 @@ __global__ void __launch_bounds__(256) mlp_backward_kernel(const float *__restri
     for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
     if (tid == 0) G[kNParams] = loss;
   }
+  if constexpr (kGroups) {
+    const cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    float *out = part + (long long)(blockIdx.x / kCluster) * kPart;
+    for (int i = (int)cluster.block_rank() * 256 + tid; i < kPart; i += 256 * kCluster) {
+      double v = 0.0;
+#pragma unroll
+      for (int c = 0; c < kCluster; ++c) v += (double)*cluster.map_shared_rank(G + i, c);
+      out[i] = (float)v;
+    }
+    cluster.sync();  // no CTA leaves while its gradient is being read
+  }
 }
 
-// G and the loss from the CTAs' partials: 8 threads per entry add strided
-// partials, then each other's sums (a fixed order).
-__global__ void __launch_bounds__(256) mlp_sum_kernel(const float *__restrict__ part, int nparts,
+// G and the loss from the partials: 8 threads per entry add strided
+// partials, then each other's sums (a fixed order), in FP64, and divide by the rows:
+// neither up to 40 additions nor a rounded 1 / n are in the result.
+__global__ void __launch_bounds__(256) mlp_sum_kernel(const float *__restrict__ part, int nparts, int n,
                                                       float *__restrict__ G, float *__restrict__ loss) {
-  __shared__ float red[8][33];
+  __shared__ double red[8][33];
   const int e = threadIdx.x & 31, q = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + e;
-  float v = 0.f;
+  double v = 0.0;
   if (i < kPart) {
 #pragma unroll 4
-    for (int b = q; b < nparts; b += 8) v += part[(long long)b * kPart + i];
+    for (int b = q; b < nparts; b += 8) v += (double)part[(long long)b * kPart + i];
   }
   red[q][e] = v;
   __syncthreads();
   if (q == 0 && i < kPart) {
     for (int k = 1; k < 8; ++k) v += red[k][e];
+    v /= (double)n;
     if (i < kNParams)
-      G[i] = v;
+      G[i] = (float)v;
     else
-      *loss = v;
+      *loss = (float)v;
   }
 }
 
@@ -530,7 +557,6 @@ __global__ void __launch_bounds__(256) check_exponents_kernel(const int *__restr
 struct df_mlp {
   float *P = nullptr, *G = nullptr, *m1 = nullptr, *m2 = nullptr, *loss = nullptr;
   float *part = nullptr;  // [kOwnParts][kPart] partial gradients
-  float *more = nullptr;  // [kMaxParts][kPart], allocated for the first larger training set
   int t = 0;
 };
 
@@ -540,7 +566,7 @@ df_status df_mlp_create(df_mlp **out) {
   if (!out) return DF_ERR_ARG;
   df_mlp *m = new (std::nothrow) df_mlp();
   if (!m) return DF_ERR_OOM;
-  // one allocation: P, the two moments, G, the loss, the first partial gradients
+  // one allocation: P, the two moments, G, the loss, the partial gradients
   const size_t np = (kNParams + 63) / 64 * 64;
   static_assert(sizeof(float) * (4 * (kNParams + 63) / 64 * 64 + 64 + kOwnParts * kPart) <= 1 << 20, "a cheap allocation");
   cudaError_t e = cudaMalloc(&m->P, sizeof(float) * (4 * np + 64 + (size_t)kOwnParts * kPart));
@@ -563,7 +589,6 @@ df_status df_mlp_create(df_mlp **out) {
 void df_mlp_destroy(df_mlp *m) {
   if (!m) return;
   cudaFree(m->P);
-  cudaFree(m->more);
   delete m;
 }
 
@@ -595,33 +620,28 @@ df_status df_mlp_gradients(df_mlp *m, const float *X, const int *y, int n, float
                            void *stream) {
   if (!m || !X || !y || n <= 0) return DF_ERR_ARG;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  // the attribute is per device and cheap to set; no process-wide flag to keep
-  cudaError_t e = cudaFuncSetAttribute(mlp_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(MlpTile));
-  if (e != cudaSuccess) return DF_ERR_CUDA;
   const int ntiles = (n + kTileRows - 1) / kTileRows;
-  const int parts = ntiles < kMaxParts ? ntiles : kMaxParts;
-  float *part = parts <= kOwnParts ? m->part : m->more, *recorded = nullptr;
-  if (!part) {
-    const size_t bytes = sizeof(float) * (size_t)kMaxParts * kPart;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    e = cudaStreamIsCapturing(st, &cs);
-    if (e == cudaSuccess && cs != cudaStreamCaptureStatusNone) {
-      e = cudaMallocAsync(&recorded, bytes, st);  // no cudaMalloc while recording: the graph's own
-      part = recorded;
-    } else if (e == cudaSuccess) {
-      e = cudaMalloc(&m->more, bytes);
-      part = m->more;
-    }
-    if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? DF_ERR_OOM : DF_ERR_CUDA;
-  }
-  mlp_backward_kernel<<<parts, 256, sizeof(MlpTile), st>>>(m->P, X, y, n, part);
-  mlp_sum_kernel<<<(kPart + 31) / 32, 256, 0, st>>>(part, parts, m->G, m->loss);
+  const bool groups = ntiles > kOwnParts;
+  const int parts = groups ? std::min((ntiles + kCluster - 1) / kCluster, kMaxClusters) : ntiles;
+  auto kern = groups ? mlp_backward_kernel<true> : mlp_backward_kernel<false>;
+  // the attribute is per device and cheap to set; no process-wide flag to keep
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpTile));
+  if (e != cudaSuccess) return DF_ERR_CUDA;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(groups ? parts * kCluster : parts));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = sizeof(MlpTile);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kCluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = groups ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, kern, (const float *)m->P, X, y, n, m->part);
+  if (e != cudaSuccess) return DF_ERR_CUDA;
+  mlp_sum_kernel<<<(kPart + 31) / 32, 256, 0, st>>>(m->part, parts, n, m->G, m->loss);
   e = cudaGetLastError();
-  if (recorded) {
-    const cudaError_t ef = cudaFreeAsync(recorded, st);
-    if (e == cudaSuccess) e = ef;
-  }
   if (e != cudaSuccess) return DF_ERR_CUDA;
   if (grad_host) e = cudaMemcpyAsync(grad_host, m->G, sizeof(float) * kNParams, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && loss_host) e = cudaMemcpyAsync(loss_host, m->loss, sizeof(float), cudaMemcpyDeviceToHost, st);

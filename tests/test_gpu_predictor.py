@@ -73,9 +73,8 @@ def test_mlp_gradients_at_warp_edges(df, n):
 
 @pytest.mark.parametrize("n", [1280, 1281])
 def test_mlp_steps_recorded_in_a_graph(df, n):
-    """Forty partial gradients come with the network, a larger set's are allocated with its first
-    gradients, also when that first call is being recorded: a replayed first step leaves the bits
-    of a direct one."""
+    """One CTA a partial gradient up to forty tiles, clusters of CTAs beyond: a first call that is
+    recorded and replayed leaves the bits of a direct one."""
     rng = np.random.default_rng(n)
     theta = M.init_params(8).astype(np.float32)
     Xg = torch.from_numpy(rng.standard_normal((n, 16)).astype(np.float32)).cuda()
@@ -94,6 +93,25 @@ def test_mlp_steps_recorded_in_a_graph(df, n):
     assert not np.array_equal(net.get_params(), theta)
     g0, g1 = direct.gradients(Xg, yg), net.gradients(Xg, yg)
     assert np.array_equal(g0[0], g1[0]) and g0[1] == g1[1]
+
+
+@pytest.mark.parametrize("n", [1281, 1311, 1312, 1537, 8192, 8195])
+def test_mlp_gradients_in_clusters(df, n):
+    """More than forty tiles: clusters of eight CTAs, the last one with idle CTAs or a ragged tile,
+    and more tiles than CTAs.  FP32 sums against FP64 as above, the same bits on every run."""
+    rng = np.random.default_rng(n)
+    theta = (M.init_params(3) + 0.05 * rng.standard_normal(M.N_PARAMS)).astype(np.float32)
+    X = rng.standard_normal((n, 16)).astype(np.float32)
+    y = rng.integers(0, 8, size=n)
+    net = df.MLP(theta)
+    Xg, yg = torch.from_numpy(X).cuda(), torch.from_numpy(y.astype(np.int32)).cuda()
+    g, loss = net.gradients(Xg, yg)
+    ref = M.gradients(theta.astype(np.float64), X.astype(np.float64), y)
+    assert abs(loss - M.loss(theta.astype(np.float64), X.astype(np.float64), y)) < 1e-5
+    assert np.max(np.abs(g - ref)) <= 1e-5 + 1e-4 * np.max(np.abs(ref))
+    for _ in range(3):
+        g2, loss2 = net.gradients(Xg, yg)
+        assert np.array_equal(g, g2) and loss == loss2
 
 
 def test_adam_steps_match_oracle(df):
