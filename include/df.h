@@ -146,8 +146,8 @@ df_status df_build_K(df_ctx *ctx, const double *C_dev, int nocc, int nslices, do
  * level that runs slices) spare warps of the two exchange GEMMs run the FP64
  * passes, rho beside the first and J beside the second: rho and J stream B
  * through the FP64 pipe, which the GEMMs leave idle.  Native FP64 (0), the
- * learned counts (-2 at a level above 0) and DF_OPT_JK_OVERLAP = 0 run the two
- * builds one after the other.  All of it is in `stream`.  Calls on one context
+ * learned counts (-2 at a level above 0), nao > 46340 and DF_OPT_JK_OVERLAP = 0
+ * run the two builds one after the other.  All of it is in `stream`.  Calls on one context
  * must not overlap (they share its work counters). */
 df_status df_build_JK(df_ctx *ctx, const double *D_dev, const double *C_dev, int nocc, int nslices,
                       double *J_dev, double *rho_dev, double *K_dev, df_kstats *stats, void *stream);

@@ -269,7 +269,10 @@ __device__ __forceinline__ int take_item(int *work) {
 }
 __device__ __forceinline__ int item_of_warp(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
-template <bool kPacked, bool kRows, int G, int kQ, typename Off>
+// 32-bit offsets: rho_work makes groups of four up to nao = 16384, and df_build_JK runs a nao
+// past kRho32Nao in order (64-bit ones beside them cost the GEMM's kernel 0.4 % of a step of
+// 87 atoms without being taken).
+template <bool kPacked, bool kRows, int G, int kQ>
 __device__ __forceinline__ void rho_items(const CoulombWork &w) {
   int it = item_of_warp(take_item(w.work));
   while (it < w.nitems) {
@@ -279,7 +282,7 @@ __device__ __forceinline__ void rho_items(const CoulombWork &w) {
     if constexpr (kRows)
       rho_part_rows<kPacked, G>(w.B, w.D, w.naux, w.nao, w.mask, P0, it & 7, v);
     else
-      rho_part<kPacked, G, kQ, Off>(w.B, w.D, w.naux, w.nao, P0, it & 7, v);
+      rho_part<kPacked, G, kQ, int>(w.B, w.D, w.naux, w.nao, P0, it & 7, v);
     if ((threadIdx.x & 31) == 0) {
 #pragma unroll
       for (int g = 0; g < G; ++g)
@@ -309,18 +312,12 @@ __device__ __forceinline__ void coulomb_items(const CoulombWork &w) {
   }
 }
 
-// A group of four has nao <= 16384 (rho_work), a B in row order nao <= 2048; one function at
-// a time takes any nao (64-bit offsets throughout cost it 2 to 3 %: 60 functions of 2600 AOs
-// beside the first exchange GEMM, the whole step 3.19 -> 3.30 ms).
 template <bool kPacked, bool kRows>
 __device__ __forceinline__ void rho_any_group(const CoulombWork &w) {
-  if (w.group == 4) {
-    rho_items<kPacked, kRows, 4, 3, int>(w);
-  } else if (kRows || w.nao <= kRho32Nao) {
-    rho_items<kPacked, kRows, 1, 8, int>(w);
-  } else {
-    rho_items<kPacked, false, 1, 8, long long>(w);
-  }
+  if (w.group == 4)
+    rho_items<kPacked, kRows, 4, 3>(w);
+  else
+    rho_items<kPacked, kRows, 1, 8>(w);
 }
 
 template <int kKind>

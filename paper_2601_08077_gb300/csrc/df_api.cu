@@ -658,9 +658,9 @@ df_status df_build_JK(df_ctx *c, const double *D, const double *C, int nocc, int
     s = df::level_count(c, level);
   }
   if (s > c->s_max) return record(c, DF_ERR_ARG);
-  // the native FP64 build, the learned counts and the no-overlap option run the
-  // two builds one after the other
-  if (c->jk_ctas == 0 || s == 0 || (nslices == -2 && c->level > 0)) {
+  // the native FP64 build, the learned counts, the no-overlap option and a B_P past 2^31
+  // elements (rho beside a GEMM has 32-bit offsets) run the two builds one after the other
+  if (c->jk_ctas == 0 || s == 0 || (nslices == -2 && c->level > 0) || c->nao > df::kRho32Nao) {
     df_status r = df_build_J(c, D, J, rho, stream);
     return r == DF_OK ? df_build_K(c, C, nocc, nslices, K, stats, stream) : r;
   }
