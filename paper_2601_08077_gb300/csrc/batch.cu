@@ -314,7 +314,8 @@ df_status df_batch_build_J(df_batch *b, const double *const *D, double *const *J
     for (int i = 0; i < n; ++i) {
       df_ctx *c = b->ctx[i];
       cudaStream_t si = b->side[i % df_batch::kFan];
-      if (df::launch_rho(c->B, D[i], c->naux, c->nao, c->rho, nullptr, si, df::use_mask_rho(c), c->packed, c->rows) !=
+      if (df::launch_rho(c->B, D[i], c->naux, c->nao, c->rho, nullptr, si, df::use_mask_rho(c), c->packed, c->rows,
+                         b->ctx.size() == 1) !=
           cudaSuccess)
         return DF_ERR_CUDA;
       if (df::launch_coulomb(c->B, c->rho, c->naux, c->nao, J[i], si, df::use_mask_j(c), c->packed) != cudaSuccess)

@@ -295,18 +295,20 @@ CoulombWork coulomb_work_of(const double *B, const double *rho, int naux, int na
 }
 
 cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, double *rho, double *rho2,
-                       cudaStream_t st, const uint32_t *mask_mu, bool packed, bool rows) {
+                       cudaStream_t st, const uint32_t *mask_mu, bool packed, bool rows, bool alone) {
   // row order: the walk over rows and masks costs more instructions than the FMAs,
   // so functions share it while the SMs keep two CTAs (350 AOs: 700 functions 130
   // us one by one, 102 by two, 113 by four; 1050 functions 145 by two, 114 by four)
   const int group = !rows ? 1 : naux >= 1024 ? 4 : naux >= 304 ? 2 : 1;
-  // dense: a CTA a function, four or five of them an SM, whichever takes less: a wave of five
-  // is a quarter longer (152 SMs, 235 AOs and 705 functions: 60 us in two waves of four, 51 in
-  // one of five; packed, 435 and 1305: 275 and 245; 600 and 1800, three waves of either: 583 and
-  // 619).  At 48 registers 64-bit offsets suit the dense layout (435 and 1305: 252 us for 300) and
-  // 32-bit ones the packed (254 for 270); past 2^31 elements of a B_P they have to be 64-bit.
+  // dense: a CTA a function, four of them an SM or, alone on the GPU, five if that takes less: a
+  // wave of five is a quarter longer (152 SMs, 235 AOs and 705 functions: 60 us in two waves of
+  // four, 51 in one of five; packed, 435 and 1305: 275 and 245; 600 and 1800, three waves of
+  // either: 583 and 619).  A batch's rho and J run beside each other, where waves do not count (16
+  // molecules' J and K 15.3 ms with fours, 15.6 with this rule).  At 48 registers 64-bit offsets
+  // suit the dense layout (435 and 1305: 252 us for 300) and 32-bit ones the packed (254 for 270);
+  // past 2^31 elements of a B_P they have to be 64-bit.
   const long long sms = slice_gemm_grid(1 << 30);
-  const bool five = (naux + 5 * sms - 1) / (5 * sms) * 5 < (naux + 4 * sms - 1) / (4 * sms) * 4;
+  const bool five = alone && (naux + 5 * sms - 1) / (5 * sms) * 5 < (naux + 4 * sms - 1) / (4 * sms) * 4;
   auto kern = packed ? rho_kernel<true, false, 1> : rho_kernel<false, false, 1>;
   if (five) kern = packed ? rho_kernel<true, false, 1, 5> : rho_kernel<false, false, 1, 5, long long>;
   if (nao > kRho32Nao) kern = packed ? rho_kernel<true, false, 1, 5, long long> : rho_kernel<false, false, 1, 5, long long>;

@@ -635,7 +635,7 @@ df_status df_build_J(df_ctx *c, const double *D, double *J, double *rho, void *s
   {
     PhaseTimer t(c, DF_PHASE_RHO, st);
     DF_TRY(c, df::launch_rho(c->B, D, c->naux, c->nao, r, r == c->rho ? nullptr : c->rho, st, df::use_mask_rho(c),
-                             c->packed, c->rows));
+                             c->packed, c->rows, true));
   }
   {
     PhaseTimer t(c, DF_PHASE_COULOMB, st);

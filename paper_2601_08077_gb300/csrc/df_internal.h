@@ -212,8 +212,9 @@ cudaError_t launch_wait_selftest(int *status, unsigned long long limit_ns, cudaS
 // rows: rho in the row-by-row order of a B of mostly zero chunks (nao <= 2048), else
 // in row-pair order; the order is the B's, so a screened B gives the same bits
 // with and without its masks.
+// alone: no other launch is meant to run beside it.
 cudaError_t launch_rho(const double *B, const double *D, int naux, int nao, double *rho, double *rho2,
-                       cudaStream_t st, const uint32_t *mask_mu, bool packed, bool rows);
+                       cudaStream_t st, const uint32_t *mask_mu, bool packed, bool rows, bool alone);
 cudaError_t launch_coulomb(const double *B, const double *rho, int naux, int nao, double *J, cudaStream_t st,
                            const uint32_t *mask_mu, bool packed);
 // The same passes as work for a slice GEMM's spare warps: `work` is zeroed before
