@@ -105,7 +105,12 @@ constexpr int kPart = kNParams + 1;  // a partial gradient and its part of the l
 // CTAs' gradients through distributed shared memory and writes one partial.
 constexpr int kOwnParts = 40;
 constexpr int kCluster = 8;
-constexpr int kMaxClusters = 32;  // 256 CTAs
+// Clusters that get an SM to each CTA (the GPCs hold 15 of eight), and at most: a tile takes 14.4
+// us in a cluster, another one of the same CTA 6.6 more, two CTAs on an SM 22.5 together and
+// 3 a further one.  So two tiles to a CTA of 15 clusters (4600 rows: 20.9 us, in 18
+// clusters 22.1), from 241 tiles on 32 clusters (8192 rows: 22.7 us, 27.6 in 15).
+constexpr int kClustersAlone = 15;
+constexpr int kMaxClusters = 32;
 static_assert(kMaxClusters <= kOwnParts, "a partial gradient per cluster");
 constexpr int kHP = kH + 4;       // activation pitch: rows of a tile on different banks, 16-byte aligned
 
@@ -622,7 +627,8 @@ df_status df_mlp_gradients(df_mlp *m, const float *X, const int *y, int n, float
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int ntiles = (n + kTileRows - 1) / kTileRows;
   const bool groups = ntiles > kOwnParts;
-  const int parts = groups ? std::min((ntiles + kCluster - 1) / kCluster, kMaxClusters) : ntiles;
+  const int most = ntiles <= 2 * kCluster * kClustersAlone ? kClustersAlone : kMaxClusters;
+  const int parts = groups ? std::min((ntiles + kCluster - 1) / kCluster, most) : ntiles;
   auto kern = groups ? mlp_backward_kernel<true> : mlp_backward_kernel<false>;
   // the attribute is per device and cheap to set; no process-wide flag to keep
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpTile));

@@ -95,10 +95,10 @@ def test_mlp_steps_recorded_in_a_graph(df, n):
     assert np.array_equal(g0[0], g1[0]) and g0[1] == g1[1]
 
 
-@pytest.mark.parametrize("n", [1281, 1311, 1312, 1537, 8192, 8195])
+@pytest.mark.parametrize("n", [1281, 1311, 1312, 1537, 3840, 3841, 7680, 7681, 8192, 8195])
 def test_mlp_gradients_in_clusters(df, n):
     """More than forty tiles: clusters of eight CTAs, the last one with idle CTAs or a ragged tile,
-    and more tiles than CTAs.  FP32 sums against FP64 as above, the same bits on every run."""
+    one and two tiles to a CTA of fifteen clusters, and more tiles than the CTAs of 32.  FP32 sums against FP64 as above, the same bits on every run."""
     rng = np.random.default_rng(n)
     theta = (M.init_params(3) + 0.05 * rng.standard_normal(M.N_PARAMS)).astype(np.float32)
     X = rng.standard_normal((n, 16)).astype(np.float32)
